@@ -203,16 +203,12 @@ DecodeArgs make_args(const mkv_ctx *c, const void *q, const void *k, const void 
     return a;
 }
 
-// Free slots and empty ring rows are read by the kernels as whole tiles (their results are
-// masked afterwards), so they must hold finite numbers: zero K, V and the query ring.
+// Stored-profile mode: what no kernel writes before it is read.  (The free slots of the K/V rows and the empty rows of
+// the ring, which the kernels read as whole tiles, are cleared by the prompt phase's gather and ring copy.)
 bool clear_arena(mkv_ctx *c, cudaStream_t stream)
 {
-    const size_t kv = (size_t)c->s.U * c->s.cap * c->s.D * c->s.es, rq = (size_t)c->s.U * c->s.R * c->s.G * c->s.D * c->s.es;
-    if (c->s.stored &&
-        cudaMemsetAsync(c->base + c->L.prof, 0, (size_t)c->s.U * c->s.R * c->s.cap * 4, stream) != cudaSuccess) return false;
-    return cudaMemsetAsync(c->base + c->L.K, 0, kv, stream) == cudaSuccess &&
-           cudaMemsetAsync(c->base + c->L.V, 0, kv, stream) == cudaSuccess &&
-           cudaMemsetAsync(c->base + c->L.ring_q, 0, rq, stream) == cudaSuccess;
+    return !c->s.stored ||
+           cudaMemsetAsync(c->base + c->L.prof, 0, (size_t)c->s.U * c->s.R * c->s.cap * 4, stream) == cudaSuccess;
 }
 
 // Arguments of a launch that covers one layer of the context's own: every arena pointer is moved to the layer's

@@ -282,32 +282,42 @@ __global__ void prefill_identity_pos_kernel(int *pos, int U, int n, int cap)
     pos[(i / n) * cap + (i % n)] = (int)(i % n);
 }
 
-// K/V rows of the kept prompt positions into the arena, 16 bytes per thread.
+// K/V rows of the kept prompt positions into the arena, 16 bytes per thread.  The free slots n .. cap-1 are cleared: the
+// decode kernels read whole tiles and mask afterwards, so a row must hold finite numbers.  (Bound by HBM: 266 MB read
+// and written in 80 us for 256 units of 2032 slots.  Clearing the whole arena first, as two memsets, wrote every kept
+// row twice.)
 template <typename T, int D>
 __global__ void prefill_gather_kernel(const T *__restrict__ k, const T *__restrict__ v, DecodeArgs a, int Ps, int n)
 {
     constexpr int CH = D * sizeof(T) / 16;
     const int u = blockIdx.x;
     const int idx = blockIdx.y * blockDim.x + threadIdx.x;
-    if (idx >= n * CH) return;
+    if (idx >= a.cap * CH) return;
     const int slot = idx / CH, c = idx % CH;
+    uint4 *Kd = reinterpret_cast<uint4 *>(static_cast<T *>(a.K) + ((size_t)u * a.cap + slot) * D) + c;
+    uint4 *Vd = reinterpret_cast<uint4 *>(static_cast<T *>(a.V) + ((size_t)u * a.cap + slot) * D) + c;
+    if (slot >= n) {
+        *Kd = make_uint4(0, 0, 0, 0);
+        *Vd = make_uint4(0, 0, 0, 0);
+        return;
+    }
     const int p = a.pos[(size_t)u * a.cap + slot];
     const uint4 *ks = reinterpret_cast<const uint4 *>(k + ((size_t)u * Ps + p) * D) + c;
     const uint4 *vs = reinterpret_cast<const uint4 *>(v + ((size_t)u * Ps + p) * D) + c;
-    reinterpret_cast<uint4 *>(static_cast<T *>(a.K) + ((size_t)u * a.cap + slot) * D)[c] = *ks;
-    reinterpret_cast<uint4 *>(static_cast<T *>(a.V) + ((size_t)u * a.cap + slot) * D)[c] = *vs;
+    *Kd = *ks;
+    *Vd = *vs;
 }
 
-// window queries into their ring rows (row p % R)
+// window queries into their ring rows (row p % R); the rows that a prompt shorter than the window leaves empty are zero
 template <typename T, int D>
 __global__ void prefill_ring_kernel(const T *__restrict__ qwin, DecodeArgs a, int P, int Rw, int Rws, int shift)
 {
     const int u = blockIdx.x, G = a.G, Gq = a.Gq;       // heads Gq .. G-1 of a ring slot are padding (zero query)
     T *rq = static_cast<T *>(a.ring_q) + (size_t)u * a.R * G * D;
-    for (int idx = threadIdx.x; idx < Rw * G * D; idx += blockDim.x) {
+    for (int idx = threadIdx.x; idx < a.R * G * D; idx += blockDim.x) {
         const int dd = idx % D, g = (idx / D) % G, i = idx / (D * G);
         const int rslot = (P - Rw + i + shift) % a.R;
-        if (g < Gq) rq[((size_t)rslot * G + g) * D + dd] = qwin[(((size_t)u * Gq + g) * Rws + i) * D + dd];
+        if (g < Gq && i < Rw) rq[((size_t)rslot * G + g) * D + dd] = qwin[(((size_t)u * Gq + g) * Rws + i) * D + dd];
         else stf(rq + ((size_t)rslot * G + g) * D + dd, 0.f);
     }
 }
@@ -319,11 +329,11 @@ __global__ void prefill_ring_vec_kernel(const T *__restrict__ qwin, DecodeArgs a
     constexpr int CH = D * sizeof(T) / 16;
     const int u = blockIdx.x, G = a.G, Gq = a.Gq;
     const int idx = blockIdx.y * blockDim.x + threadIdx.x;
-    if (idx >= Rw * G * CH) return;
+    if (idx >= a.R * G * CH) return;
     const int c = idx % CH, g = (idx / CH) % G, i = idx / (CH * G);
     const int rslot = (P - Rw + i + shift) % a.R;
     uint4 v = make_uint4(0, 0, 0, 0);
-    if (g < Gq) v = reinterpret_cast<const uint4 *>(qwin + (((size_t)u * Gq + g) * Rws + i) * D)[c];
+    if (g < Gq && i < Rw) v = reinterpret_cast<const uint4 *>(qwin + (((size_t)u * Gq + g) * Rws + i) * D)[c];
     reinterpret_cast<uint4 *>(static_cast<T *>(a.ring_q) + (((size_t)u * a.R + rslot) * G + g) * D)[c] = v;
 }
 
@@ -452,9 +462,9 @@ cudaError_t run_prefill_t(const DecodeArgs &a, const T *k, const T *v, const T *
         ++*launches;
     }
     constexpr int CH = D * sizeof(T) / 16;
-    prefill_gather_kernel<T, D><<<dim3(U, (n * CH + 255) / 256), 256, 0, stream>>>(k, v, a, Ps, n);
+    prefill_gather_kernel<T, D><<<dim3(U, (a.cap * CH + 255) / 256), 256, 0, stream>>>(k, v, a, Ps, n);
     if (((uintptr_t)qwin & 15) == 0)
-        prefill_ring_vec_kernel<T, D><<<dim3(U, (Rw * G * CH + 255) / 256), 256, 0, stream>>>(qwin, a, P, Rw, Rws, shift);
+        prefill_ring_vec_kernel<T, D><<<dim3(U, (R * G * CH + 255) / 256), 256, 0, stream>>>(qwin, a, P, Rw, Rws, shift);
     else
         prefill_ring_kernel<T, D><<<U, 256, 0, stream>>>(qwin, a, P, Rw, Rws, shift);
     if (a.norm_current && select) {
