@@ -54,12 +54,12 @@ typedef enum mkv_dtype { MKV_DTYPE_BF16 = 0, MKV_DTYPE_F32 = 1 } mkv_dtype;
  * row's token was generated.  CURRENT: renormalised over the tokens that are
  * still cached when the scores are taken (a row never saw tokens newer than itself); not with evict_interval > 1. */
 typedef enum mkv_norm { MKV_NORM_FROZEN = 0, MKV_NORM_CURRENT = 1 } mkv_norm;
-/* where the window tokens' attention profiles come from when the fused scores are taken (Eq. 4-6):
- * RECOMPUTE (default): from the stored window queries and their frozen soft-max normalisers, inside the decode
- *   kernel (same numbers, no table);
- * STORED: from a table of the weights themselves, kept beside the KV cache as the paper's implementation keeps
- *   them (Implementation paragraph): R * (C + R) more floats per unit, read once per policy step.  Trades bytes
- *   for arithmetic; it pays for wide windows.  bf16 / head_dim 128 on the tensor-core kernel only, with per-step
+/* how the window tokens' attention profiles are kept (Eq. 4-6).  With MKV_NORM_FROZEN a weight never changes once its
+ * row has been generated, so the tensor-core kernel scores each row of the window once and keeps the sums of finished
+ * blocks of rows beside the cache ((number of blocks + 2) * (C + R) * 4 bytes per unit), in either mode:
+ * RECOMPUTE (default): any kernel, normalisation and eviction interval;
+ * STORED: the paper's implementation keeps the weights themselves (Implementation paragraph).  Same numbers; lifts the
+ *   tensor-core kernel's limit on the window.  bf16 / head_dim 128 on the tensor-core kernel only, with per-step
  *   eviction and MKV_NORM_FROZEN; not with mkv_prefill_ragged. */
 typedef enum mkv_profile { MKV_PROFILE_RECOMPUTE = 0, MKV_PROFILE_STORED = 1 } mkv_profile;
 /* which decode kernel to use: AUTO picks the tensor-core kernel when the shape allows it (bf16, head_dim 128, a
@@ -232,7 +232,9 @@ mkv_status mkv_decode_step_host(mkv_ctx *ctx, const void *q_host, const void *k_
                                 const void *v_new_host, void *out_host, void *stream);
 
 /* Device pointers into one layer of the cache.  Valid until the context is destroyed;
- * contents change with every decode step.  Reading them needs a stream synchronisation. */
+ * contents change with every decode step.  Reading them needs a stream synchronisation.
+ * The view is for reading, with one exception: slot order is free, so rows of K, V and pos may be
+ * moved together between two steps, by whoever has called this function since the earlier one. */
 mkv_status mkv_cache_view(mkv_ctx *ctx, int layer, mkv_view *view);
 
 /* Waits for `stream` and reports device-side errors (MKV_DEVICE_TIMEOUT) recorded so far. */

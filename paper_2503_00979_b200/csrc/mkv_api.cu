@@ -16,7 +16,7 @@ using namespace mkv;
 namespace {
 
 struct Layout {
-    size_t K, V, pos, ring_q, ring_c, s_new, F, Fc, prof, part_ml, part_o, ticket, evicted, state, rows, row_shift, stage_q, stage_k, stage_v,
+    size_t K, V, pos, ring_q, ring_c, s_new, F, Fc, slab, pre, sum_pos, part_ml, part_o, ticket, evicted, state, rows, row_shift, stage_q, stage_k, stage_v,
         stage_o, total;
 };
 
@@ -28,8 +28,8 @@ struct Shape {
     int B, Hkv;             // batch rows and KV heads (upl = B * Hkv)
     int U, G, D, R, C, cap, splits, T, tc_grid_size, tc_grid_layer;
     int Gq;                 // the model's GQA ratio; G is it rounded up to a power of two on the tensor-core path
-    int nc;                 // ring chunks of the tensor-core kernel (1 unless the window has more than 256 rows)
-    int stored;             // 1: the window tokens' attention profiles are kept as a table (profile_mode STORED)
+    int nc;                 // ring chunks of the tensor-core kernel (1 unless CURRENT and the window has more than 256 rows)
+    int bs, nblk;           // slots per block of the ring and blocks (DecodeArgs::slab)
     size_t es;
 };
 
@@ -46,8 +46,10 @@ Layout make_layout(const Shape &s)
     L.ring_c = take(U * R * G * 4);
     L.s_new = take(U * G * cap * 4);
     L.F = take(U * cap * 4);
-    L.Fc = take(s.nc > 1 && !s.stored ? U * (size_t)s.nc * cap * 4 : 0);
-    L.prof = take(s.stored ? U * R * cap * 4 : 0);
+    L.Fc = take(s.nc > 1 ? U * (size_t)s.nc * cap * 4 : 0);
+    L.slab = take(s.nblk > 1 ? U * (size_t)s.nblk * cap * 4 : 0);
+    L.pre = take(s.nblk > 1 ? U * cap * 4 : 0);
+    L.sum_pos = take(s.nblk > 1 ? U * cap * 4 : 0);
     L.part_ml = take(U * sp * G * 2 * 4);
     L.part_o = take(U * sp * G * D * 4);
     L.ticket = take(U * 4);
@@ -103,19 +105,23 @@ bool resolve(const mkv_params *p, Shape *s, KernelKind *kind)
     s->cap = p->C + p->R + (s->T > 1 ? s->T : 0);
     s->es = p->dtype == MKV_DTYPE_F32 ? 4 : 2;
     s->nc = 1;
-    s->stored = p->profile_mode == MKV_PROFILE_STORED ? 1 : 0;
-    if (s->stored && (s->T > 1 || p->norm_mode != MKV_NORM_FROZEN || p->kernel == MKV_KERNEL_SIMT)) return false;
+    const bool current = p->norm_mode == MKV_NORM_CURRENT;
+    // (STORED asks for weights that are kept instead of recomputed: with FROZEN normalisation every tensor-core context
+    // keeps their sums.  What is left of the mode is its own range: the tensor-core kernel, windows of any width.)
+    const bool stored = p->profile_mode == MKV_PROFILE_STORED;
+    if (stored && (s->T > 1 || p->norm_mode != MKV_NORM_FROZEN || p->kernel == MKV_KERNEL_SIMT)) return false;
     if (s->T > 64) return false;
     if (p->norm_mode == MKV_NORM_CURRENT && s->T > 1) return false;     // the compaction drops several tokens at once
-    // stored-profile mode: the decode kernel only ever needs the ring rows of the new query, whatever the window's size
-    const int nc = s->stored ? 1 : tc_ring_chunks(s->G, s->R);
-    const bool tc_ok = tc_shape_supported(p->dtype == MKV_DTYPE_F32, s->D, s->G, s->stored ? 1 : s->R) &&
+    const int nc = current ? tc_ring_chunks(s->G, s->R) : 1;
+    const bool tc_ok = tc_shape_supported(p->dtype == MKV_DTYPE_F32, s->D, s->G, stored ? 1 : s->R) &&
                        (long long)s->U * nc * ((s->cap + 127) / 128) <= (1ll << 30);     // tile indices stay 32-bit
     if (p->kernel == MKV_KERNEL_TC && !tc_ok) return false;
     if (tc_ok && p->kernel != MKV_KERNEL_SIMT) {
         *kind = kKindTc;
         s->G = tc_padded_group(s->Gq);
         s->nc = nc;       // a unit appears in the schedule once per ring chunk
+        s->bs = tc_block_slots(s->Gq, s->R, current);
+        s->nblk = current ? 1 : (s->R + s->bs - 1) / s->bs;
         // the persistent grid (148 SMs on B200; correctness does not depend on the count)
         s->tc_grid_size = tc_grid(s->U * nc, s->cap, p->splits, 148);
         // a per-layer call sees only a layer's units: ranges of about an eighth of a unit's tiles, so that a layer
@@ -129,8 +135,10 @@ bool resolve(const mkv_params *p, Shape *s, KernelKind *kind)
         s->splits = sp_all > sp_layer ? sp_all : sp_layer;
         return true;
     }
-    if (s->stored) return false;        // the profile table is kept by the tensor-core kernel's epilogue only
+    if (stored) return false;
     *kind = kKindSimt;
+    s->bs = s->R;
+    s->nblk = 1;
     const int max_splits = (s->cap + 31) / 32;
     int sp = p->splits > 0 ? p->splits : simt_default_splits(s->U, s->cap);
     if (sp > max_splits) sp = max_splits;
@@ -162,6 +170,7 @@ struct mkv_ctx {
     int next_layer;   // per-layer calls: the layer (of this context's own) expected next; 0 at a step boundary
     int cursor;       // per-layer calls: the layer of the whole model expected next (kept by the outer context)
     int state_ahead;  // 0: whole-stack and per-layer device states level, 1: whole-stack ahead, 2: per-layer ahead
+    unsigned char *viewed;       // [layers] (contexts that keep window sums): a view has been handed out since the last step
     unsigned long long launches;
     PrefillScratch prefill_scratch;
     char err[256];
@@ -185,8 +194,10 @@ DecodeArgs make_args(const mkv_ctx *c, const void *q, const void *k, const void 
     a.ring_q = b + c->L.ring_q; a.ring_c = (float *)(b + c->L.ring_c);
     a.q = q; a.k_new = k; a.v_new = v; a.out = out;
     a.s_new = (float *)(b + c->L.s_new); a.F = (float *)(b + c->L.F);
-    a.Fc = c->s.nc > 1 && !c->s.stored ? (float *)(b + c->L.Fc) : nullptr; a.nc = c->s.nc;
-    a.prof = c->s.stored ? (float *)(b + c->L.prof) : nullptr;
+    a.Fc = c->s.nc > 1 ? (float *)(b + c->L.Fc) : nullptr; a.nc = c->s.nc;
+    a.bs = c->s.bs; a.nblk = c->s.nblk;
+    a.slab = a.nblk > 1 ? (float *)(b + c->L.slab) : nullptr; a.pre = a.nblk > 1 ? (float *)(b + c->L.pre) : nullptr;
+    a.sum_pos = a.nblk > 1 ? (int *)(b + c->L.sum_pos) : nullptr;
     a.part_ml = (float *)(b + c->L.part_ml); a.part_o = (float *)(b + c->L.part_o);
     a.ticket = (int *)(b + c->L.ticket); a.evicted_pos = (int *)(b + c->L.evicted);
     a.st = (DevState *)(b + c->L.state);
@@ -203,14 +214,6 @@ DecodeArgs make_args(const mkv_ctx *c, const void *q, const void *k, const void 
     return a;
 }
 
-// Stored-profile mode: what no kernel writes before it is read.  (The free slots of the K/V rows and the empty rows of
-// the ring, which the kernels read as whole tiles, are cleared by the prompt phase's gather and ring copy.)
-bool clear_arena(mkv_ctx *c, cudaStream_t stream)
-{
-    return !c->s.stored ||
-           cudaMemsetAsync(c->base + c->L.prof, 0, (size_t)c->s.U * c->s.R * c->s.cap * 4, stream) == cudaSuccess;
-}
-
 // Arguments of a launch that covers one layer of the context's own: every arena pointer is moved to the layer's
 // first unit, the inputs and `out` are that layer's tensors, and the layer's own step state is used.
 // `row` >= 0 narrows the launch further, to that batch row's units of the layer (prompt phase of a ragged batch).
@@ -224,7 +227,7 @@ DecodeArgs make_args_layer(const mkv_ctx *c, int layer, const void *q, const voi
     a.ring_q = (char *)a.ring_q + u0 * s.R * s.G * s.D * s.es; a.ring_c += u0 * s.R * s.G;
     a.s_new += u0 * s.G * s.cap; a.F += u0 * s.cap;
     if (a.Fc) a.Fc += u0 * s.nc * s.cap;
-    if (a.prof) a.prof += u0 * s.R * s.cap;
+    if (a.slab) { a.slab += u0 * s.nblk * s.cap; a.pre += u0 * s.cap; a.sum_pos += u0 * s.cap; }
     a.part_ml += u0 * s.splits * s.G * 2; a.part_o += u0 * s.splits * s.G * s.D;
     a.ticket += u0; a.evicted_pos += u0;
     a.st = a.st + 1 + layer;
@@ -257,13 +260,19 @@ mkv_status launch_step(mkv_ctx *ctx, int layer, const void *q, const void *k, co
     const mkv_status ls = level_states(ctx, layer < 0 ? 1 : 2, stream);
     if (ls != MKV_OK) return ls;
     const DecodeArgs a = layer < 0 ? make_args(ctx, q, k, v, out) : make_args_layer(ctx, layer, q, k, v, out);
-    // stored-profile mode: a policy step reads its fused scores from the table first.  Launched on every step: the
-    // kernel decides by the device's step state and returns at once when no policy runs, so that a recorded
-    // sequence of steps stays valid when it is replayed into another phase of the sequence.
-    if (ctx->s.stored) {
-        const cudaError_t ef = launch_profile_fuse(a, stream);
-        if (ef != cudaSuccess) return fail(ctx, MKV_CUDA, "profile launch failed: %s", cudaGetErrorString(ef));
-        ctx->launches += 1;
+    // A view of the cache has been handed out since the last step, and its holder may have rearranged the slots (their
+    // order is free): the window sums of slots whose token has changed are taken again.  At the start of a step that
+    // is looked after for all layers at once, within a step for the layer concerned.
+    if (ctx->viewed) {
+        const bool start = layer <= 0;
+        bool any = false;
+        for (int l = start ? 0 : layer; l < (start ? ctx->s.layers : layer + 1); ++l) { any |= ctx->viewed[l] != 0; ctx->viewed[l] = 0; }
+        if (any) {
+            DecodeArgs w = a;
+            if (layer == 0) { w = make_args(ctx, q, k, v, out); w.st = a.st; }
+            const cudaError_t ef = launch_window_sums(w, ctx->p.dtype == MKV_DTYPE_F32, ctx->s.D, &ctx->launches, stream);
+            if (ef != cudaSuccess) return fail(ctx, MKV_CUDA, "window sums launch failed: %s", cudaGetErrorString(ef));
+        }
     }
     const cudaError_t e = ctx->kind == kKindTc ? launch_decode_tc(layer < 0 ? ctx->plan : ctx->plan_layer, a, stream)
                                                : launch_decode_simt(a, ctx->p.dtype == MKV_DTYPE_F32, ctx->s.D, stream);
@@ -325,7 +334,11 @@ mkv_status core_create(mkv_ctx **out, const mkv_params *p, void *workspace, size
     c->row_n = new (std::nothrow) int[2 * (size_t)s.B];
     if (!c->row_n) { delete c; return MKV_OOM; }
     c->row_shift = c->row_n + s.B;
-    if (cudaGetDevice(&c->device) != cudaSuccess) { cudaGetLastError(); delete[] c->row_n; delete c; return MKV_CUDA; }
+    if (s.nblk > 1) {
+        c->viewed = new (std::nothrow) unsigned char[s.layers]();
+        if (!c->viewed) { delete[] c->row_n; delete c; return MKV_OOM; }
+    }
+    if (cudaGetDevice(&c->device) != cudaSuccess) { cudaGetLastError(); delete[] c->row_n; delete[] c->viewed; delete c; return MKV_CUDA; }
     if (workspace) {
         c->base = (char *)workspace;
     } else {
@@ -333,6 +346,7 @@ mkv_status core_create(mkv_ctx **out, const mkv_params *p, void *workspace, size
         if (cudaMalloc(&mem, L.total) != cudaSuccess) {
             cudaGetLastError();
             delete[] c->row_n;
+            delete[] c->viewed;
             delete c;
             return MKV_OOM;
         }
@@ -349,6 +363,7 @@ mkv_status core_create(mkv_ctx **out, const mkv_params *p, void *workspace, size
             if (c->plan) tc_plan_destroy(c->plan);
             if (c->owns_workspace) cudaFree(c->base);
             delete[] c->row_n;
+            delete[] c->viewed;
             delete c;
             return e == cudaErrorMemoryAllocation ? MKV_OOM : MKV_CUDA;
         }
@@ -365,6 +380,7 @@ void core_destroy(mkv_ctx *ctx)
     if (ctx->prefill_scratch.ptr) cudaFree(ctx->prefill_scratch.ptr);
     if (ctx->owns_workspace && ctx->base) cudaFree(ctx->base);
     delete[] ctx->row_n;
+    delete[] ctx->viewed;
     delete ctx;
 }
 
@@ -390,7 +406,6 @@ mkv_status core_prefill(mkv_ctx *ctx, const void *k, const void *v, const void *
     }
     ctx->ragged = false;
     const DecodeArgs a = make_args(ctx, nullptr, nullptr, nullptr, nullptr);
-    if (!clear_arena(ctx, stream)) return fail(ctx, MKV_CUDA, "%s: clearing the arena failed", where);
     const bool f32 = ctx->p.dtype == MKV_DTYPE_F32;
     const int n_states = 1 + ctx->s.layers;
     const cudaError_t e = use_static
@@ -400,12 +415,6 @@ mkv_status core_prefill(mkv_ctx *ctx, const void *k, const void *v, const void *
     if (e == cudaErrorLaunchTimeout) { cudaGetLastError(); return fail(ctx, MKV_DEVICE_TIMEOUT, "%s: a device-side wait of the prompt phase ran out", where); }
     if (e != cudaSuccess) return fail(ctx, MKV_CUDA, "prompt phase: %s", cudaGetErrorString(e));
     ctx->n = (prompt_len - Rw > ctx->s.C) ? ctx->s.C + Rw : prompt_len;
-    if (ctx->s.stored) {        // the window rows' profiles over the kept tokens
-        cudaError_t ep = launch_prefill_profile(a, ctx->n, prompt_len, stream);
-        if (ep == cudaSuccess) ep = cudaStreamSynchronize(stream);
-        if (ep != cudaSuccess) return fail(ctx, MKV_CUDA, "prompt phase (profile table): %s", cudaGetErrorString(ep));
-        ctx->launches += 1;
-    }
     ctx->t = prompt_len;
     ctx->steps = 0;
     ctx->next_layer = 0;
@@ -422,12 +431,11 @@ mkv_status core_prefill_ragged(mkv_ctx *ctx, const void *k, const void *v, const
     const Shape &s = ctx->s;
     if (ctx->prefilled) return fail(ctx, MKV_BAD_STATE, "mkv_prefill_ragged: context already holds a sequence%s");
     if (s.T > 1) return fail(ctx, MKV_UNSUPPORTED, "mkv_prefill_ragged: not available with coarse-grained eviction%s");
-    if (s.stored) return fail(ctx, MKV_UNSUPPORTED, "mkv_prefill_ragged: not available with the stored attention profile%s");
-    if (s.nc > 1) return fail(ctx, MKV_UNSUPPORTED, "mkv_prefill_ragged: not available with a window of more than 256 ring rows on the tensor-core kernel; create the context with the CUDA-core kernel%s");
+    if (ctx->p.profile_mode == MKV_PROFILE_STORED) return fail(ctx, MKV_UNSUPPORTED, "mkv_prefill_ragged: not available with the stored attention profile%s");
+    if (ctx->kind == kKindTc && tc_ring_chunks(s.Gq, s.R) > 1) return fail(ctx, MKV_UNSUPPORTED, "mkv_prefill_ragged: not available with a window of more than 256 ring rows on the tensor-core kernel; create the context with the CUDA-core kernel%s");
     int longest = 0;
     for (int b = 0; b < s.B; ++b) longest = std::max(longest, (int)prompt_len[b]);
     ctx->ragged = true;          // make_args hands the row arrays to the kernels from here on
-    if (!clear_arena(ctx, stream)) return fail(ctx, MKV_CUDA, "mkv_prefill_ragged: clearing the arena failed%s");
     const bool f32 = ctx->p.dtype == MKV_DTYPE_F32;
     const int qw_stride = padded_len < s.R ? padded_len : s.R;
     int nmax = 0;
@@ -456,11 +464,11 @@ mkv_status core_prefill_ragged(mkv_ctx *ctx, const void *k, const void *v, const
     for (int i = 0; i < ns * 2; ++i) memcpy(rows_h + (size_t)i * s.B, ctx->row_n, sizeof(int) * s.B);
     cudaError_t e = cudaMemcpyAsync(ctx->base + ctx->L.rows, rows_h, sizeof(int) * ns * 2 * s.B, cudaMemcpyHostToDevice, stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->base + ctx->L.row_shift, ctx->row_shift, sizeof(int) * s.B, cudaMemcpyHostToDevice, stream);
-    if (e == cudaSuccess) e = launch_set_state((DevState *)(ctx->base + ctx->L.state), ns, (long long)longest, nmax, stream);
+    const DecodeArgs all = make_args(ctx, nullptr, nullptr, nullptr, nullptr);
+    if (e == cudaSuccess) e = launch_finish_prompt(all, longest, nmax, ns, &all.st->err, &ctx->launches, stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
     delete[] rows_h;
     if (e != cudaSuccess) return fail(ctx, MKV_CUDA, "prompt phase: %s", cudaGetErrorString(e));
-    ctx->launches += 1;
     ctx->n = nmax;
     ctx->t = longest;
     ctx->steps = 0;
@@ -521,6 +529,7 @@ void core_view(mkv_ctx *ctx, int layer, mkv_view *view)
     const size_t u0 = (size_t)ctx->s.upl * layer;
     const Shape &s = ctx->s;
     char *b = ctx->base;
+    if (ctx->viewed) ctx->viewed[layer] = 1;
     view->K = b + ctx->L.K + u0 * s.cap * s.D * s.es;
     view->V = b + ctx->L.V + u0 * s.cap * s.D * s.es;
     view->pos = (int32_t *)(b + ctx->L.pos) + u0 * s.cap;

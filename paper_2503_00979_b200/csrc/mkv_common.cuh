@@ -62,10 +62,22 @@ struct DecodeArgs {
     int *row_n;                // [2][B]
     const int *row_shift;      // [B]
     int B, Hkv;                // unit u (of this launch) belongs to batch row (u / Hkv) % B
-    float *prof;               // [U][R][cap]  stored-profile mode (nullptr otherwise): prof[r][k] is the weight, summed
-                               // over the group, that the window token of ring slot r gave to the token in cache slot
-                               // k when it was generated (the attention profile the paper's implementation stores
-                               // beside the KV cache); the fused scores are then read from this table, not recomputed
+    // Window sums kept across steps (FROZEN normalisation on the tensor-core kernel; nullptr / 1 block otherwise).
+    // The weight a window row gave a key when the row was generated never changes, so nothing has to be scored twice.
+    // The ring is cut into nblk blocks of bs slots, and a lap is one run of t % R over it.  Only the block that is
+    // being filled, a mixture of this lap's rows and the last lap's, is scored on every step; the step that opens the
+    // next block scores the finished one for good.  With j the open block and + the fusion (sum or max; nothing is
+    // ever subtracted):
+    //   slab[i], i < j   fused score of block i, filled in this lap;   pre = slab[0] + .. + slab[j - 1]
+    //   slab[i], i > j   fused score of the last lap's blocks i .. nblk - 1 (made from the single ones at the lap's end)
+    //   window           pre + block j + slab[j + 1]
+    // An entry counts for a key only once the key has left the window (Eq. 7 has no other candidates): every row of
+    // the window is then newer than the key, so whatever the entries held before the key took its slot is gone.
+    float *slab;               // [U][nblk][cap]
+    float *pre;                // [U][cap]
+    int *sum_pos;              // [U][cap]  position of the token a slot's entries belong to (= pos, unless a holder of a
+                               // cache view has rearranged the slots)
+    int bs, nblk;
     int n_hint;                // the host's view of st->n when the launch was enqueued (0: none).  Only used to
                                // prefetch: a stale value (steps replayed from a CUDA graph) costs time, not results
 };
@@ -183,6 +195,14 @@ __device__ __forceinline__ void group_sync(int bar_id, int nthr)
     asm volatile("barrier.sync %0, %1;" ::"r"(bar_id), "r"(nthr) : "memory");
 }
 
+// The block of the ring that is open before the step at position t, and whether that step opens the next one (it then
+// scores block `open` for good: see DecodeArgs::slab).
+__host__ __device__ inline int open_block(long long t, int R, int bs) { return (int)((t - 1) % R) / bs; }
+__host__ __device__ inline bool step_opens_block(long long t, int R, int bs, int nblk)
+{
+    return nblk > 1 && (int)(t % R) % bs == 0;
+}
+
 // CURRENT normalisation (the reading of Eq. 4 in which a window row's weights are taken over the tokens that are
 // still cached): the token in `e_slot` is about to be evicted, so every window row loses the weight w it had on it
 // and its log2-domain normaliser becomes c + log2(1 - w); the surviving weights of the row grow by 1 / (1 - w).
@@ -233,8 +253,7 @@ __device__ void renormalise_after_eviction(const DecodeArgs &a, int u, int e_slo
 // group size when known at compile time (0: use a.G); it lets the loads of a round be
 // issued together.  Loads are batched so that the whole epilogue costs a handful of L2
 // round trips.
-// PROF: the caller may be serving the stored-profile mode (a.prof); compiled out otherwise.
-template <typename T, int D, int GT, bool PROF = false>
+template <typename T, int D, int GT>
 __device__ void finalize_unit(const DecodeArgs &a, int u, long long t, int n, int active, bool evict, float *sm,
                               int tid, int nthr, int bar_id, int shift = 0)
 {
@@ -311,17 +330,6 @@ __device__ void finalize_unit(const DecodeArgs &a, int u, long long t, int n, in
     int *pos = a.pos + (size_t)u * a.cap;
     float *F = a.F + (size_t)u * a.cap;
     int e_slot = n, e_pos = -1;
-    // stored-profile mode: the new token's row of the table is written on every step, policy or not
-    float *prof_row = nullptr;
-    if constexpr (PROF) prof_row = a.prof ? a.prof + ((size_t)u * a.R + (int)(t % a.R)) * a.cap : nullptr;
-    if (PROF && prof_row != nullptr && !evict) {
-        const float *sn = a.s_new + (size_t)u * G * a.cap;
-        for (int k = tid; k < n; k += nthr) {
-            float s = 0.f;
-            for (int g = 0; g < G; ++g) s += exp2f(__ldcg(sn + (size_t)g * a.cap + k) - cnew[g]);
-            prof_row[k] = s;
-        }
-    }
     if (evict) {
         const float *sn = a.s_new + (size_t)u * G * a.cap;
         const long long thr = t - shift - a.R;        // positions are the row's own; ring slots follow t
@@ -356,7 +364,6 @@ __device__ void finalize_unit(const DecodeArgs &a, int u, long long t, int n, in
             for (int b = 0; b < 4; ++b) {
                 const int k = kb + b * nthr;
                 if (k >= n) continue;
-                if (PROF && prof_row != nullptr) prof_row[k] = s[b];
                 if ((long long)p[b] <= thr) {
                     const float f = fuse(a.fusion, f0[b], s[b]);
                     F[k] = f;
@@ -412,15 +419,9 @@ __device__ void finalize_unit(const DecodeArgs &a, int u, long long t, int n, in
     T *rq = static_cast<T *>(a.ring_q) + ((size_t)u * a.R + rs) * G * D;
     for (int i = tid; i < G * D; i += nthr) stf(rq + i, i < Gq * D ? ldf(q + i) : 0.f);
     if (tid < G) a.ring_c[((size_t)u * a.R + rs) * G + tid] = cnew[tid];
-    if (PROF && a.prof != nullptr) {
-        // the slot the new token takes: no older window token ever attended to it; the new token's weight on itself
-        float self_w = 0.f;
-        for (int g = 0; g < G; ++g) self_w += exp2f(s_self[g] - cnew[g]);
-        float *col = a.prof + (size_t)u * a.R * a.cap + e_slot;
-        for (int r = tid; r < a.R; r += nthr) col[(size_t)r * a.cap] = r == rs ? self_w : 0.f;
-    }
     if (tid == 0) {
         pos[e_slot] = (int)(t - shift);
+        if (a.nblk > 1) a.sum_pos[(size_t)u * a.cap + e_slot] = (int)(t - shift);
         a.evicted_pos[u] = e_pos;
         a.ticket[u] = 0;
     }

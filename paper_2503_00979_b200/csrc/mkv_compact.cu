@@ -17,7 +17,7 @@ constexpr int kCT = 1024;         // threads per CTA
 
 // KPT slots per thread, held in registers (indices are compile-time constants after unrolling)
 template <typename T, int D, int KPT>
-__global__ void __launch_bounds__(kCT) compact_kernel(DecodeArgs a)
+__global__ void __launch_bounds__(kCT, KPT <= 4 ? 2 : 1) compact_kernel(DecodeArgs a)
 {
     __shared__ unsigned long long red_key[kCT / 32];
     __shared__ int red_slot[kCT / 32];
@@ -108,8 +108,21 @@ __global__ void __launch_bounds__(kCT) compact_kernel(DecodeArgs a)
         }
         __syncthreads();
         if (tid < nh) { pos[holes[tid]] = pos[movers[tid]]; F[holes[tid]] = F[movers[tid]]; }
+        if (a.nblk > 1) {           // the window sums move with their slot
+            float *slab = a.slab + (size_t)u * a.nblk * a.cap, *pre = a.pre + (size_t)u * a.cap;
+            for (int idx = tid; idx < nh * (a.nblk + 1); idx += kCT) {
+                const int i = idx % nh, j = idx / nh;
+                float *row = j < a.nblk ? slab + (size_t)j * a.cap : pre;
+                row[holes[i]] = row[movers[i]];
+            }
+            if (tid < nh) a.sum_pos[(size_t)u * a.cap + holes[tid]] = pos[movers[tid]];
+        }
         __syncthreads();
-        for (int k = keep + tid; k < n; k += kCT) { pos[k] = -1; F[k] = 0.f; }
+        for (int k = keep + tid; k < n; k += kCT) {
+            pos[k] = -1;
+            F[k] = 0.f;
+            if (a.nblk > 1) a.sum_pos[(size_t)u * a.cap + k] = -1;
+        }
         if (tid == 0) a.evicted_pos[u] = -1;
     }
     // the last CTA publishes the new fill (all CTAs have read the state by then)

@@ -22,6 +22,7 @@ cudaError_t launch_compact(const DecodeArgs &a, bool f32, int D, cudaStream_t st
 bool tc_shape_supported(bool f32, int D, int G, int R);
 int tc_padded_group(int G);
 int tc_ring_chunks(int G, int R);
+int tc_block_slots(int G, int R, bool current);   // slots per block of the ring (DecodeArgs::bs)
 int tc_grid(int U, int cap, int splits_hint, int n_sm);
 int tc_partials_per_unit(int U, int cap, int grid);
 struct TcPlan;
@@ -50,7 +51,6 @@ struct PrefillRow {
 cudaError_t run_prefill(const DecodeArgs &a, bool f32, int D, const void *k, const void *v, const void *q_window,
                         int P, cudaStream_t stream, unsigned long long *launches, PrefillScratch *scratch, int n_states,
                         const PrefillRow *row = nullptr);
-cudaError_t launch_set_state(DevState *st, int n_states, long long t, int n, cudaStream_t stream);
 
 // Tensor-core scoring of the prompt phase (mkv_prefill_tc.cu): two passes over the prompt keys, window-row
 // normalisers into ring_c and fused scores of the older tokens into Fp [nb][P].
@@ -67,11 +67,14 @@ size_t prefill_static_max_floats();
 cudaError_t run_prefill_static(const DecodeArgs &a, bool f32, int D, const void *k, const void *v, const void *q_window,
                                int P, cudaStream_t stream, unsigned long long *launches, int device, int n_states);
 
-// Stored-profile mode (bf16, head_dim 128, tensor-core kernel): the fused scores of a policy step from the profile
-// table into a.F (a no-op on other steps; launched in front of the decode kernel), and the table after the prompt
-// phase (the arena's ring, K rows and positions must be in place; the table must have been cleared).
-cudaError_t launch_profile_fuse(const DecodeArgs &a, cudaStream_t stream);
-cudaError_t launch_prefill_profile(const DecodeArgs &a, int n, long long P, cudaStream_t stream);
+// The window sums (DecodeArgs::slab) of the slots whose token is no longer the one in sum_pos, for the step that a.st
+// holds.  *launches counts the launches.
+cudaError_t launch_window_sums(const DecodeArgs &a, bool f32, int D, unsigned long long *launches, cudaStream_t stream);
+// Last launch(es) of the prompt phase: the window sums of every slot, where the context keeps them, for the step at
+// position t of n cached tokens, and the n_states step states at a.st.  `err`: word in which a wait that runs out is
+// reported.
+cudaError_t launch_finish_prompt(const DecodeArgs &a, long long t, int n, int n_states, int *err, unsigned long long *launches,
+                                 cudaStream_t stream);
 
 // Copies one step state over n_dst others (the whole-stack state and the per-layer states are brought level when
 // a context switches between whole-stack and per-layer calls).

@@ -36,16 +36,9 @@ __global__ void init_arena_kernel(DecodeArgs a)
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const size_t ncap = (size_t)a.U * a.cap;
     if (i < ncap) { a.pos[i] = -1; a.F[i] = 0.f; }
+    if (i < ncap && a.nblk > 1) a.sum_pos[i] = -1;
     if (i < (size_t)a.U * a.R * a.G) a.ring_c[i] = INFINITY;   // empty ring row: weight 0
     if (i < (size_t)a.U) { a.ticket[i] = 0; a.evicted_pos[i] = -1; }
-}
-
-// the whole-stack state and one state per layer (per-layer calls advance their own)
-__global__ void set_state_kernel(DevState *st, int n_states, long long t, int n)
-{
-    for (int i = threadIdx.x; i < n_states; i += blockDim.x) {
-        st[i].t = t; st[i].n = n; st[i].steps = 0; st[i].err = 0; st[i].done = 0; st[i].compact = 0;
-    }
 }
 
 // S[ub][row = i*G + g][j] = log2-domain logit of window row (i, g) against prompt key j,
@@ -432,7 +425,8 @@ cudaError_t run_prefill_t(const DecodeArgs &a, const T *k, const T *v, const T *
     const size_t init_n = max((size_t)U * a.cap, (size_t)U * R * G);
     init_arena_kernel<<<(unsigned)((init_n + 255) / 256), 256, 0, stream>>>(a);
     ++*launches;
-    if (tc) {
+    const bool waits = tc || a.nblk > 1;            // kernels with bounded waits are launched
+    if (waits) {
         e = cudaMemsetAsync(err_word, 0, sizeof(int), stream);
         if (e != cudaSuccess) return e;
     }
@@ -473,12 +467,11 @@ cudaError_t run_prefill_t(const DecodeArgs &a, const T *k, const T *v, const T *
     }
     *launches += 2;
     if (row) return cudaGetLastError();
-    set_state_kernel<<<1, 32, 0, stream>>>(a.st, n_states, (long long)P, n);
-    *launches += 1;
     e = cudaGetLastError();
+    if (e == cudaSuccess) e = launch_finish_prompt(a, P, n, n_states, err_word, launches, stream);
     const cudaError_t e2 = cudaStreamSynchronize(stream);
     if (e != cudaSuccess || e2 != cudaSuccess) return e != cudaSuccess ? e : e2;
-    if (tc) {       // a bounded wait of the scoring kernels that ran out
+    if (waits) {    // a bounded wait that ran out
         int werr = 0;
         e = cudaMemcpy(&werr, err_word, sizeof(int), cudaMemcpyDeviceToHost);
         if (e != cudaSuccess) return e;
@@ -560,12 +553,6 @@ cudaError_t run_prefill(const DecodeArgs &a, bool f32, int D, const void *k, con
     }
     return dispatch_prefill(a, f32, D, k, v, q_window, P, stream, launches, static_cast<float *>(scratch->ptr),
                             scratch->bytes / sizeof(float), n_states, row);
-}
-
-cudaError_t launch_set_state(DevState *st, int n_states, long long t, int n, cudaStream_t stream)
-{
-    set_state_kernel<<<1, 32, 0, stream>>>(st, n_states, t, n);
-    return cudaGetLastError();
 }
 
 namespace {

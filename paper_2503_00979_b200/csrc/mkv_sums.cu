@@ -1,0 +1,349 @@
+// The window sums of the cached slots (DecodeArgs::slab, pre) from the arena as it stands.
+//
+// window_sums_tc_kernel ends the prompt phase of the tensor-core contexts: every key is scored against all ring rows,
+// block by block from the last block of the ring to the first, so that the sums of the last lap's blocks accumulate in
+// a register on the way.  It has the decode kernel's orientation (keys in the TMEM lanes, ring rows as the N operand,
+// up to 256 at a time) and the CTA layout of the prompt phase's scoring passes: warps 0-3 and 6-9 are two consumer
+// groups on alternate key tiles and accumulator buffers, warp 4 feeds K tiles with TMA, warp 5 issues the MMAs.
+// Bound by the kept keys' bytes and R*G exponentials per key (256 units of 2048 slots, 128 rows: 38 us).
+//
+// window_sums_kernel does the same on the CUDA cores for the slots whose token is no longer the one their sums belong
+// to: a holder of a cache view may rearrange the slots, so the first step after a view has been handed out runs it (as cheap as reading 8 bytes per slot).
+// Nothing has moved as a rule, and it ends after comparing two positions per slot.
+#include <string.h>
+
+#include "mkv_common.cuh"
+#include "mkv_kernels.h"
+#include "mkv_sm100.cuh"
+
+namespace mkv {
+
+namespace {
+
+constexpr int kSumThreads = 320;
+constexpr int kSumGroups = 2;
+constexpr int kSumMaxRows = 2048;            // ring rows of one launch: their normalisers sit in shared memory
+enum SumWait { kSumKEmpty = 31, kSumKFull, kSumTEmpty, kSumTFull, kSumDrain };
+
+struct SumArgs {
+    DecodeArgs d;
+    long long t;              // the sums are those the step at position t finds
+    int n;
+    int set_states;           // step states at d.st to set to (t, n)
+    int *err;
+    int row0, rows;           // ring rows of this launch (whole blocks; the launches of a wide window go from the last
+    int last;                 // rows to the first, and the last one leaves sum_pos)
+    int piece;                // rows of one MMA operand
+    int splits;               // CTAs per unit along the keys
+    int tmem_cols, stages;
+    long long wait_cycles;
+};
+
+__device__ __forceinline__ void set_states(const SumArgs &a)
+{
+    for (int i = threadIdx.x; i < a.set_states; i += blockDim.x) {
+        DevState *s = a.d.st + i;
+        s->t = a.t; s->n = a.n; s->steps = 0; s->err = 0; s->done = 0; s->compact = 0;
+    }
+}
+
+// The fused score S of ring block j joins the sums of one key; blocks come in descending order, acc and pre run along.
+__device__ __forceinline__ void take_block(float S, int j, int open, int fusion, float *slab, size_t cap, bool valid,
+                                           float &acc, float &pre)
+{
+    if (j > open) {
+        acc = fuse(fusion, acc, S);
+        if (valid) slab[(size_t)j * cap] = acc;
+    } else if (j < open) {
+        pre = fuse(fusion, pre, S);
+        if (valid) slab[(size_t)j * cap] = S;
+    }
+}
+
+template <int G, int FUSION>
+__global__ void __launch_bounds__(kSumThreads, 2)
+window_sums_tc_kernel(const __grid_constant__ SumArgs a, const __grid_constant__ CUtensorMap tmK)
+{
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+    const DecodeArgs &d = a.d;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int sp = blockIdx.x, u = blockIdx.y;
+    const int PR = a.piece, ST = a.stages;
+    const uint32_t sbase = smem_u32(smem);
+    const uint32_t q_addr = sbase, kst_addr = sbase + PR * 256;
+    float *negc = reinterpret_cast<float *>(smem + PR * 256 + ST * kStageBytes);        // [kSumMaxRows]
+    uint64_t *bars = reinterpret_cast<uint64_t *>(negc + kSumMaxRows);
+    const uint32_t bar_kfull = smem_u32(bars), bar_kempty = smem_u32(bars + 4);
+    const uint32_t bar_tfull = smem_u32(bars + 8), bar_tempty = smem_u32(bars + 10);
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 12);
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(bars + 13);
+    const long long WL = a.wait_cycles;
+
+    const int n = a.n, nt = (n + kTile - 1) / kTile, per = (nt + a.splits - 1) / a.splits;
+    const int t0 = sp * per, t1 = min(nt, t0 + per), ntile = max(0, t1 - t0);
+    if (sp == 0 && u == 0) set_states(a);
+    const int blk_rows = d.bs * G, RG = d.R * G, open = open_block(a.t, d.R, d.bs);
+    const int npiece = (a.rows + PR - 1) / PR;
+
+    if (tid == 0) {
+        prefetch_tensormap(&tmK);
+        for (int s = 0; s < ST; ++s) { mbar_init(bar_kfull + 8 * s, 1); mbar_init(bar_kempty + 8 * s, 1); }
+        for (int b = 0; b < 2; ++b) { mbar_init(bar_tfull + 8 * b, 1); mbar_init(bar_tempty + 8 * b, 4); }
+        *abort_flag = 0;
+        fence_barrier_init();
+    }
+    if (warp == 5) tmem_alloc(smem_u32(tmem_slot), (uint32_t)a.tmem_cols);
+    for (int i = tid; i < kSumMaxRows; i += kSumThreads) {
+        const int row = a.row0 + i;
+        negc[i] = i < a.rows && row < RG ? -d.ring_c[(size_t)u * RG + row] : -INFINITY;     // empty and padding rows: weight 0
+    }
+
+    int done = 0;               // tiles of the pieces before this one
+    for (int pc = npiece - 1; pc >= 0; --pc, done += ntile) {
+        // the piece's ring rows, K-major with the 128-byte swizzle (two 64-column panels of PR rows)
+        const int r0 = a.row0 + pc * PR, rn = min(PR, a.rows - pc * PR);
+        for (int c = tid; c < PR * 16; c += kSumThreads) {
+            const int row = c >> 4, ch = c & 15;
+            uint4 v = make_uint4(0, 0, 0, 0);
+            if (row < rn && r0 + row < RG)
+                v = reinterpret_cast<const uint4 *>(static_cast<const __nv_bfloat16 *>(d.ring_q) + ((size_t)u * RG + r0 + row) * kD)[ch];
+            *reinterpret_cast<uint4 *>(smem + (uint32_t)((ch >> 3) * (PR * 128) + row * 128 + (((ch & 7) ^ (row & 7)) << 4))) = v;
+        }
+        fence_proxy_async();
+        tc_fence_before();
+        __syncthreads();
+        tc_fence_after();
+        const uint32_t tmem_base = *tmem_slot;
+        bool ok = true;
+        if (warp == 4) {
+            // ------------------------------------------------ TMA producer of K tiles (one lane)
+            if (lane == 0) {
+                const uint64_t pol = l2_policy_evict_first();
+                int issued = done;
+                for (int j = done; j < done + ntile && ok; ++j) {
+                    const int s = j % ST;
+                    ok = mbar_wait(bar_kempty + 8 * s, (uint32_t)(((j / ST) & 1) ^ 1), abort_flag, kSumKEmpty, WL);
+                    if (!ok) break;
+                    const int row = (t0 + j - done) * kTile;
+                    mbar_expect_tx(bar_kfull + 8 * s, kStageBytes);
+                    tma_load_3d(kst_addr + s * kStageBytes, &tmK, 0, row, u, bar_kfull + 8 * s, pol);
+                    tma_load_3d(kst_addr + s * kStageBytes + kStageBytes / 2, &tmK, 64, row, u, bar_kfull + 8 * s, pol);
+                    issued = j + 1;
+                }
+                if (!ok) {      // let the copies in flight land before the CTA exits
+                    int dummy = 0;
+                    for (int j = max(done, issued - ST); j < issued; ++j)
+                        mbar_wait(bar_kfull + 8 * (j % ST), (uint32_t)((j / ST) & 1), &dummy, kSumDrain, kWaitCycles);
+                }
+            }
+            __syncwarp();
+        } else if (warp == 5) {
+            // ------------------------------------------------ MMA issue: D[128 keys x rows] = K_tile . Q^T
+            const int np = (rn + 31) & ~31;
+            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kTile >> 4) << 24) | ((uint32_t)(np >> 3) << 17);
+            int j = done;
+            for (; j < done + ntile; ++j) {
+                const int s = j % ST, b = j & 1;
+                bool k = mbar_wait(bar_kfull + 8 * s, (uint32_t)((j / ST) & 1), abort_flag, kSumKFull, WL);
+                k = k && mbar_wait(bar_tempty + 8 * b, (uint32_t)(((j >> 1) & 1) ^ 1), abort_flag, kSumTEmpty, WL);
+                ok = __all_sync(0xffffffffu, k);
+                if (!ok) break;
+                tc_fence_after();
+                if (lane == 0) {
+                    const uint32_t d_tmem = tmem_base + (uint32_t)(b * PR);
+#pragma unroll
+                    for (int ks = 0; ks < kD / 16; ++ks) {
+                        const uint64_t ad = smem_desc_sw128(kst_addr + s * kStageBytes + (ks >> 2) * (kStageBytes / 2) + (ks & 3) * 32);
+                        const uint64_t bd = smem_desc_sw128(q_addr + (ks >> 2) * (PR * 128) + (ks & 3) * 32);
+                        umma_bf16(d_tmem, ad, bd, idesc, ks > 0 ? 1u : 0u);
+                    }
+                    umma_commit(bar_kempty + 8 * s);
+                    umma_commit(bar_tfull + 8 * b);
+                }
+                __syncwarp();
+            }
+            {   // every commit is observed before the operand is overwritten, TMEM is freed or the CTA exits
+                int dummy = 0;
+                for (int i = max(done, j - ST); i < j; ++i)
+                    mbar_wait(bar_kempty + 8 * (i % ST), (uint32_t)((i / ST) & 1), &dummy, kSumDrain, kWaitCycles);
+                if (!ok)
+                    for (int i = max(done, j - 2); i < j; ++i)
+                        mbar_wait(bar_tfull + 8 * (i & 1), (uint32_t)((i >> 1) & 1), &dummy, kSumDrain, kWaitCycles);
+                __syncwarp();
+            }
+        } else {
+            // ------------------------------------------------ consumers: one key per thread; group g takes the tiles
+            // whose running number has its parity (= accumulator buffer g)
+            const int grp = warp < 4 ? 0 : 1, lq = (warp & 3) * 32 + lane;
+            const uint32_t tlane = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(grp * PR);
+            const int jtop = (r0 + rn) / blk_rows;                       // block behind this piece's last one
+            const bool top = jtop >= d.nblk;
+            for (int j = done + (((done & 1) != grp) ? 1 : 0); j < done + ntile && ok; j += kSumGroups) {
+                ok = __all_sync(0xffffffffu, mbar_wait(bar_tfull + 8 * grp, (uint32_t)((j >> 1) & 1), abort_flag, kSumTFull, WL));
+                if (!ok) break;
+                tc_fence_after();
+                const int key = (t0 + j - done) * kTile + lq;
+                const bool valid = key < n;
+                float *slab = d.slab + (size_t)u * d.nblk * d.cap + key, *prep = d.pre + (size_t)u * d.cap + key;
+                float acc = !top && valid && jtop > open ? slab[(size_t)jtop * d.cap] : 0.f;
+                float pre = !top && valid ? *prep : 0.f;
+                float S = 0.f;
+                for (int c = ((rn + 31) & ~31) - 32; c >= 0; c -= 32) {
+                    uint32_t v[32];
+                    tmem_ld32(tlane + (uint32_t)c, v);
+                    score_chunk<G, FUSION>(v, negc + pc * PR + c, d.scale2, S);
+                    if (c % blk_rows == 0) {
+                        take_block(S, (r0 + c) / blk_rows, open, FUSION, slab, d.cap, valid, acc, pre);
+                        S = 0.f;
+                        __syncwarp();                        // converged again in front of the aligned TMEM load
+                    }
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar_tempty + 8 * grp);
+                if (valid) {
+                    *prep = pre;
+                    if (a.last && pc == 0) d.sum_pos[(size_t)u * d.cap + key] = d.pos[(size_t)u * d.cap + key];
+                }
+                __syncwarp();
+            }
+        }
+        tc_fence_before();
+        __syncthreads();        // the operand's and the accumulators' readers are done
+        tc_fence_after();
+        if (*abort_flag) break;
+    }
+    if (warp == 5) tmem_dealloc(*tmem_slot, (uint32_t)a.tmem_cols);
+    if (tid == 0 && *abort_flag) atomicCAS(a.err, 0, *abort_flag);
+}
+
+// What is timed is the comparison, 8 bytes per slot in 16-byte loads; a slot that was moved is redone by one thread.
+constexpr int kSumKeys = 256;
+template <typename T, int D>
+__global__ void __launch_bounds__(kSumKeys) window_sums_kernel(const __grid_constant__ DecodeArgs d)
+{
+    const size_t total = (size_t)d.U * d.cap, i4 = ((size_t)blockIdx.x * kSumKeys + threadIdx.x) * 4;
+    if (i4 >= total) return;
+    // (a layer's arrays need not start on a 16-byte boundary)
+    if (i4 + 4 <= total && (((uintptr_t)d.pos | (uintptr_t)d.sum_pos) & 15) == 0) {
+        const int4 x = *reinterpret_cast<const int4 *>(d.pos + i4), y = *reinterpret_cast<const int4 *>(d.sum_pos + i4);
+        if (x.x == y.x && x.y == y.y && x.z == y.z && x.w == y.w) return;
+    }
+    for (size_t at = i4; at < total && at < i4 + 4; ++at) {
+        if (d.pos[at] == d.sum_pos[at] || d.pos[at] < 0) continue;
+        const size_t u = at / d.cap;
+        const int key = (int)(at % d.cap), G = d.G, open = open_block(d.st->t, d.R, d.bs);
+        const T *kr = static_cast<const T *>(d.K) + at * D;
+        float acc = 0.f, pre = 0.f;
+        for (int j = d.nblk - 1; j >= 0; --j) {
+            float S = 0.f;
+            for (int s = j * d.bs; s < min(d.R, (j + 1) * d.bs); ++s) {
+                float Sr = 0.f;
+                for (int g = 0; g < G; ++g) {
+                    const size_t row = (u * d.R + s) * G + g;
+                    const T *qr = static_cast<const T *>(d.ring_q) + row * D;
+                    float x = 0.f;
+                    for (int i = 0; i < D; ++i) x += ldf(qr + i) * ldf(kr + i);
+                    Sr += exp2f(x * d.scale2 - d.ring_c[row]);
+                }
+                S = fuse(d.fusion, S, Sr);
+            }
+            take_block(S, j, open, d.fusion, d.slab + u * d.nblk * d.cap + key, d.cap, true, acc, pre);
+        }
+        d.pre[at] = pre;
+        d.sum_pos[at] = d.pos[at];
+    }
+}
+
+__global__ void set_states_kernel(const __grid_constant__ SumArgs a) { set_states(a); }
+
+template <int G>
+cudaError_t launch_sums_g(const SumArgs &a, const CUtensorMap &tm, cudaStream_t stream)
+{
+    auto kern = a.d.fusion == kFusionSum ? window_sums_tc_kernel<G, kFusionSum> : window_sums_tc_kernel<G, kFusionMax>;
+    const int smem = a.piece * 256 + a.stages * kStageBytes + kSumMaxRows * 4 + 256 + 1024;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    kern<<<dim3(a.splits, a.d.U), kSumThreads, smem, stream>>>(a, tm);
+    return cudaGetLastError();
+}
+
+// `d` for a launch over its units u0 .. u0 + count - 1 (grid.y takes 65535 units at most)
+DecodeArgs unit_range(const DecodeArgs &d, int D, size_t es, int u0, int count)
+{
+    DecodeArgs p = d;
+    const size_t u = u0;
+    p.U = count;
+    p.K = static_cast<char *>(d.K) + u * d.cap * D * es;
+    p.ring_q = static_cast<char *>(d.ring_q) + u * d.R * d.G * D * es;
+    p.ring_c += u * d.R * d.G;
+    p.pos += u * d.cap; p.sum_pos += u * d.cap; p.pre += u * d.cap;
+    p.slab += u * d.nblk * d.cap;
+    return p;
+}
+constexpr int kMaxGridY = 65535;
+
+}  // namespace
+
+cudaError_t launch_window_sums(const DecodeArgs &d, bool f32, int D, unsigned long long *launches, cudaStream_t stream)
+{
+    const unsigned grid = (unsigned)(((size_t)d.U * d.cap + 4 * kSumKeys - 1) / (4 * kSumKeys));
+    if (f32) {
+        if (D == 64) window_sums_kernel<float, 64><<<grid, kSumKeys, 0, stream>>>(d);
+        else window_sums_kernel<float, 128><<<grid, kSumKeys, 0, stream>>>(d);
+    } else {
+        if (D == 64) window_sums_kernel<__nv_bfloat16, 64><<<grid, kSumKeys, 0, stream>>>(d);
+        else window_sums_kernel<__nv_bfloat16, 128><<<grid, kSumKeys, 0, stream>>>(d);
+    }
+    ++*launches;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_finish_prompt(const DecodeArgs &d, long long t, int n, int n_states, int *err, unsigned long long *launches,
+                                 cudaStream_t stream)
+{
+    SumArgs a;
+    memset(&a, 0, sizeof(a));
+    a.d = d;
+    a.t = t; a.n = n; a.err = err;
+    a.wait_cycles = kWaitCycles;
+    if (d.nblk <= 1) {
+        a.set_states = n_states;
+        set_states_kernel<<<1, 32, 0, stream>>>(a);
+        ++*launches;
+        return cudaGetLastError();
+    }
+    const int blk_rows = d.bs * d.G, all = d.nblk * blk_rows;
+    a.piece = min(all, 256 / blk_rows * blk_rows);
+    a.stages = a.piece <= 128 ? 2 : 3;
+    a.tmem_cols = 32;
+    while (a.tmem_cols < 2 * a.piece) a.tmem_cols *= 2;
+    const int chunk = kSumMaxRows / a.piece * a.piece;
+    for (int u0 = 0; u0 < d.U; u0 += kMaxGridY) {
+        a.d = unit_range(d, kD, 2, u0, min(kMaxGridY, d.U - u0));
+        a.splits = prefill_tc_splits(a.d.U, n, a.piece);
+        CUtensorMap tm;
+        if (!encode_map(&tm, a.d.K, a.d.U, d.cap, kTile)) return cudaErrorInvalidValue;
+        for (int row0 = (all - 1) / chunk * chunk; row0 >= 0; row0 -= chunk) {
+            a.row0 = row0;
+            a.rows = min(chunk, all - row0);
+            a.last = row0 == 0;
+            a.set_states = a.last && u0 + a.d.U == d.U ? n_states : 0;
+            cudaError_t e;
+            switch (d.G) {
+                case 1: e = launch_sums_g<1>(a, tm, stream); break;
+                case 2: e = launch_sums_g<2>(a, tm, stream); break;
+                case 4: e = launch_sums_g<4>(a, tm, stream); break;
+                case 8: e = launch_sums_g<8>(a, tm, stream); break;
+                case 16: e = launch_sums_g<16>(a, tm, stream); break;
+                default: e = cudaErrorInvalidValue;
+            }
+            ++*launches;
+            if (e != cudaSuccess) return e;
+        }
+    }
+    return cudaSuccess;
+}
+
+}  // namespace mkv
