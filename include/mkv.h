@@ -192,9 +192,8 @@ mkv_status mkv_prefill_static(mkv_ctx *ctx, const void *k, const void *v, const 
  * would leave it (Algorithm 1 once over the row's prompt), and every later decode step appends one token to every
  * row: row b's token of step s has position prompt_len[b] + s, its window, eviction decisions and cache fill are
  * its own.  mkv_view.count is then the largest fill among the rows and mkv_view.next_pos the longest row's
- * position; mkv_row_state reports each row.  Rows are processed one by one with the CUDA-core scoring kernels
- * (set-up speed, not tuned).  Not available (MKV_UNSUPPORTED) together with evict_interval > 1 or with a window
- * of more than 256 ring rows on the tensor-core kernel.  Synchronises the stream before returning. */
+ * position; mkv_row_state reports each row.  Not available (MKV_UNSUPPORTED) together with evict_interval > 1 or
+ * with a window of more than 256 ring rows on the tensor-core kernel.  Synchronises the stream before returning. */
 mkv_status mkv_prefill_ragged(mkv_ctx *ctx, const void *k, const void *v, const void *q_window,
                               const int32_t *prompt_len, int padded_len, void *stream);
 

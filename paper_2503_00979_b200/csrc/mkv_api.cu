@@ -216,12 +216,11 @@ DecodeArgs make_args(const mkv_ctx *c, const void *q, const void *k, const void 
 
 // Arguments of a launch that covers one layer of the context's own: every arena pointer is moved to the layer's
 // first unit, the inputs and `out` are that layer's tensors, and the layer's own step state is used.
-// `row` >= 0 narrows the launch further, to that batch row's units of the layer (prompt phase of a ragged batch).
-DecodeArgs make_args_layer(const mkv_ctx *c, int layer, const void *q, const void *k, const void *v, void *out, int row = -1)
+DecodeArgs make_args_layer(const mkv_ctx *c, int layer, const void *q, const void *k, const void *v, void *out)
 {
     DecodeArgs a = make_args(c, q, k, v, out);
     const Shape &s = c->s;
-    const size_t u0 = (size_t)layer * s.upl + (row >= 0 ? (size_t)row * s.Hkv : 0);
+    const size_t u0 = (size_t)layer * s.upl;
     a.K = (char *)a.K + u0 * s.cap * s.D * s.es; a.V = (char *)a.V + u0 * s.cap * s.D * s.es;
     a.pos += u0 * s.cap;
     a.ring_q = (char *)a.ring_q + u0 * s.R * s.G * s.D * s.es; a.ring_c += u0 * s.R * s.G;
@@ -233,7 +232,7 @@ DecodeArgs make_args_layer(const mkv_ctx *c, int layer, const void *q, const voi
     a.st = a.st + 1 + layer;
     if (a.row_n) a.row_n += (size_t)(1 + layer) * 2 * s.B;
     a.u0 = (int)u0;
-    a.U = row >= 0 ? s.Hkv : s.upl;
+    a.U = s.upl;
     return a;
 }
 
@@ -410,7 +409,7 @@ mkv_status core_prefill(mkv_ctx *ctx, const void *k, const void *v, const void *
     const int n_states = 1 + ctx->s.layers;
     const cudaError_t e = use_static
         ? run_prefill_static(a, f32, ctx->s.D, k, v, q_window, prompt_len, stream, &ctx->launches, ctx->device, n_states)
-        : run_prefill(a, f32, ctx->s.D, k, v, q_window, prompt_len, stream, &ctx->launches, &ctx->prefill_scratch, n_states);
+        : run_prefill(a, f32, ctx->s.D, k, v, q_window, prompt_len, stream, &ctx->launches, &ctx->prefill_scratch, n_states, prompt_len);
     if (e == cudaErrorMemoryAllocation) { cudaGetLastError(); return fail(ctx, MKV_OOM, "%s: no memory for scratch", where); }
     if (e == cudaErrorLaunchTimeout) { cudaGetLastError(); return fail(ctx, MKV_DEVICE_TIMEOUT, "%s: a device-side wait of the prompt phase ran out", where); }
     if (e != cudaSuccess) return fail(ctx, MKV_CUDA, "prompt phase: %s", cudaGetErrorString(e));
@@ -423,8 +422,7 @@ mkv_status core_prefill(mkv_ctx *ctx, const void *k, const void *v, const void *
     return MKV_OK;
 }
 
-// Prompt phase of a batch whose rows have prompts of different lengths (tensors padded to `padded_len` tokens): every
-// row goes through the prompt phase by itself, layer by layer, then the common step state is set.
+// Prompt phase of a batch whose rows have prompts of different lengths (tensors padded to `padded_len` tokens).
 mkv_status core_prefill_ragged(mkv_ctx *ctx, const void *k, const void *v, const void *q_window, const int32_t *prompt_len,
                                int padded_len, cudaStream_t stream)
 {
@@ -435,9 +433,6 @@ mkv_status core_prefill_ragged(mkv_ctx *ctx, const void *k, const void *v, const
     if (ctx->kind == kKindTc && tc_ring_chunks(s.Gq, s.R) > 1) return fail(ctx, MKV_UNSUPPORTED, "mkv_prefill_ragged: not available with a window of more than 256 ring rows on the tensor-core kernel; create the context with the CUDA-core kernel%s");
     int longest = 0;
     for (int b = 0; b < s.B; ++b) longest = std::max(longest, (int)prompt_len[b]);
-    ctx->ragged = true;          // make_args hands the row arrays to the kernels from here on
-    const bool f32 = ctx->p.dtype == MKV_DTYPE_F32;
-    const int qw_stride = padded_len < s.R ? padded_len : s.R;
     int nmax = 0;
     for (int b = 0; b < s.B; ++b) {
         const int P = prompt_len[b], Rw = P < s.R ? P : s.R;
@@ -445,29 +440,22 @@ mkv_status core_prefill_ragged(mkv_ctx *ctx, const void *k, const void *v, const
         ctx->row_shift[b] = longest - P;
         nmax = std::max(nmax, ctx->row_n[b]);
     }
-    for (int layer = 0; layer < s.layers; ++layer) {
-        for (int b = 0; b < s.B; ++b) {
-            const DecodeArgs a = make_args_layer(ctx, layer, nullptr, nullptr, nullptr, nullptr, b);
-            const size_t unit = ((size_t)layer * s.B + b) * s.Hkv;
-            const PrefillRow row = {padded_len, qw_stride, ctx->row_shift[b]};
-            const cudaError_t e = run_prefill(a, f32, s.D, off(k, unit * padded_len * s.D * s.es), off(v, unit * padded_len * s.D * s.es),
-                                              off(q_window, unit * s.Gq * qw_stride * s.D * s.es), prompt_len[b], stream,
-                                              &ctx->launches, &ctx->prefill_scratch, 0, &row);
-            if (e == cudaErrorMemoryAllocation) { cudaGetLastError(); return fail(ctx, MKV_OOM, "mkv_prefill_ragged: no memory for scratch%s"); }
-            if (e != cudaSuccess) return fail(ctx, MKV_CUDA, "prompt phase: %s", cudaGetErrorString(e));
-        }
-    }
-    // the rows' fills for every state and both step parities, their offsets, then the common state
+    ctx->ragged = true;          // make_args hands the row arrays to the kernels from here on
+    // the rows' fills for every state and both step parities, and their offsets
     const int ns = 1 + s.layers;
     int *rows_h = new (std::nothrow) int[(size_t)ns * 2 * s.B];
     if (!rows_h) return fail(ctx, MKV_OOM, "mkv_prefill_ragged: out of host memory%s");
     for (int i = 0; i < ns * 2; ++i) memcpy(rows_h + (size_t)i * s.B, ctx->row_n, sizeof(int) * s.B);
     cudaError_t e = cudaMemcpyAsync(ctx->base + ctx->L.rows, rows_h, sizeof(int) * ns * 2 * s.B, cudaMemcpyHostToDevice, stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->base + ctx->L.row_shift, ctx->row_shift, sizeof(int) * s.B, cudaMemcpyHostToDevice, stream);
-    const DecodeArgs all = make_args(ctx, nullptr, nullptr, nullptr, nullptr);
-    if (e == cudaSuccess) e = launch_finish_prompt(all, longest, nmax, ns, &all.st->err, &ctx->launches, stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+    // every unit of the batch goes through the same launches, each by its own length
+    const DecodeArgs a = make_args(ctx, nullptr, nullptr, nullptr, nullptr);
+    if (e == cudaSuccess)
+        e = run_prefill(a, ctx->p.dtype == MKV_DTYPE_F32, s.D, k, v, q_window, longest, stream, &ctx->launches, &ctx->prefill_scratch, ns,
+                        padded_len);
     delete[] rows_h;
+    if (e == cudaErrorMemoryAllocation) { cudaGetLastError(); return fail(ctx, MKV_OOM, "mkv_prefill_ragged: no memory for scratch%s"); }
+    if (e == cudaErrorLaunchTimeout) { cudaGetLastError(); return fail(ctx, MKV_DEVICE_TIMEOUT, "mkv_prefill_ragged: a device-side wait of the prompt phase ran out%s"); }
     if (e != cudaSuccess) return fail(ctx, MKV_CUDA, "prompt phase: %s", cudaGetErrorString(e));
     ctx->n = nmax;
     ctx->t = longest;

@@ -82,6 +82,14 @@ struct DecodeArgs {
                                // prefetch: a stale value (steps replayed from a CUDA graph) costs time, not results
 };
 
+// How far the prompt of a unit's batch row ends before the longest one (0 everywhere unless the rows' prompts have
+// different lengths): unit u belongs to batch row (u / Hkv) % B.
+struct RowMap {
+    const int *shift;          // [B] or nullptr
+    int Hkv, B;
+    __device__ __forceinline__ int operator()(int u) const { return shift != nullptr ? shift[(u / Hkv) % B] : 0; }
+};
+
 // Fill, position offset and policy decision of one unit on this step.
 struct UnitStep {
     int n, shift;

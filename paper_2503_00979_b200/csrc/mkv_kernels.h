@@ -41,23 +41,18 @@ struct PrefillScratch {
     void *ptr;
     size_t bytes;
 };
-// One batch row of a batch whose prompts have different lengths: `a` covers the row's units of one layer, k / v /
-// q_window point at the row's first unit inside tensors padded to the longest prompt (kv_stride tokens per unit,
-// qw_stride window entries per head), and the row is `shift` positions behind the longest on the context's common
-// time axis, which assigns the ring slots.  Such a call leaves the step state alone and does not synchronise.
-struct PrefillRow {
-    int kv_stride, qw_stride, shift;
-};
+// With prompts of different lengths in the batch (a.row_shift) P is the longest prompt's length; the tensors are padded
+// to padded_len tokens (P otherwise).
 cudaError_t run_prefill(const DecodeArgs &a, bool f32, int D, const void *k, const void *v, const void *q_window,
                         int P, cudaStream_t stream, unsigned long long *launches, PrefillScratch *scratch, int n_states,
-                        const PrefillRow *row = nullptr);
+                        int padded_len);
 
 // Tensor-core scoring of the prompt phase (mkv_prefill_tc.cu): two passes over the prompt keys, window-row
 // normalisers into ring_c and fused scores of the older tokens into Fp [nb][P].
 bool prefill_tc_supported(bool f32, int D, int G, int R, const void *k, int P);
 int prefill_tc_splits(int units_in_batch, int P, int window_rows);
 size_t prefill_tc_floats_per_unit(int P, int Rw, int G, int splits);
-cudaError_t run_prefill_scores_tc(const DecodeArgs &a, const void *k, const void *qwin, int P, int ub0, int nb, int splits,
+cudaError_t run_prefill_scores_tc(const DecodeArgs &a, const void *k, const void *qwin, int P, int Ps, int ub0, int nb, int splits,
                                   float *Fp, float *part, int *err, unsigned long long *launches, cudaStream_t stream);
 
 // The same prompt phase with its scratch in a fixed device array of prefill_static_max_floats()

@@ -46,15 +46,20 @@ __global__ void init_arena_kernel(DecodeArgs a)
 template <typename T, int D>
 __global__ void __launch_bounds__(kPT) prefill_logits_kernel(const T *__restrict__ k, const T *__restrict__ qwin,
                                                              float *__restrict__ S, int ub0, int P, int Rw, int G,
-                                                             float scale2, int Ps, int Rws)
+                                                             float scale2, int Ps, int Rws, RowMap rowmap)
 {
-    // Ps, Rws: tokens per unit in k and entries per head in qwin as laid out by the caller (P and Rw unless the
-    // batch rows' prompts have different lengths and the tensors are padded to the longest)
+    // P, Rw: of the longest prompt, which S is laid out for.  Ps, Rws: tokens per unit in k and entries per head in qwin
+    // as laid out by the caller (P and Rw unless the batch rows' prompts have different lengths and the tensors are
+    // padded)
     extern __shared__ __align__(16) float psm[];
     float *Ks = psm, *Qs = psm + kPK * (D + 4), *Ssm = Qs + kPR * (D + 4);
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const int u = ub0 + blockIdx.y, kt = blockIdx.x * kPK;
+    const int Srows = Rw * G, SP = P;
+    P -= rowmap(u);
+    Rw = min(Rw, P);
     const int rows = Rw * G;
+    if (kt >= P) return;
     constexpr int KS = D + 4, C4 = D / 4;
     const T *Ku = k + (size_t)u * Ps * D;
     for (int idx = tid; idx < kPK * C4; idx += kPT) {
@@ -103,20 +108,24 @@ __global__ void __launch_bounds__(kPT) prefill_logits_kernel(const T *__restrict
             if (j >= P) continue;
             const int row = r0 + rl;
             const int rpos = P - Rw + row / G;           // absolute position of the window row
-            S[((size_t)blockIdx.y * rows + row) * P + j] = (j <= rpos) ? Ssm[key * (kPR + 1) + rl] : -INFINITY;
+            S[((size_t)blockIdx.y * Srows + row) * SP + j] = (j <= rpos) ? Ssm[key * (kPR + 1) + rl] : -INFINITY;
         }
     }
 }
 
 // c = max + log2(sum exp2(s - max)) of one window row; stored in the ring row p % R.
 __global__ void __launch_bounds__(kPT) prefill_rowstats_kernel(const float *__restrict__ S, float *__restrict__ ring_c,
-                                                               int ub0, int P, int Rw, int G, int Gs, int R, int shift)
+                                                               int ub0, int P, int Rw, int G, int Gs, int R, RowMap rowmap)
 {
     __shared__ float red[kPT / 32];
     __shared__ float bc;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int row = blockIdx.x, u = ub0 + blockIdx.y;
     const float *s = S + ((size_t)blockIdx.y * Rw * G + row) * P;
+    const int shift = rowmap(u);
+    P -= shift;
+    Rw = min(Rw, P);
+    if (row >= Rw * G) return;
     float m = -INFINITY;
     for (int j = tid; j < P; j += kPT) m = fmaxf(m, s[j]);
     m = warp_max(m);
@@ -143,10 +152,13 @@ __global__ void __launch_bounds__(kPT) prefill_rowstats_kernel(const float *__re
 // Eq. 4-6 with Algorithm 1's group sum: F[j] for every older prompt token j < P - Rw.
 __global__ void __launch_bounds__(kPT) prefill_fuse_kernel(const float *__restrict__ S, const float *__restrict__ ring_c,
                                                            float *__restrict__ Fp, int ub0, int P, int Rw, int G, int Gs,
-                                                           int R, int fusion, int shift)
+                                                           int R, int fusion, RowMap rowmap)
 {
     extern __shared__ float cs[];   // [Rw * G]
-    const int u = ub0 + blockIdx.y, rows = Rw * G;
+    const int u = ub0 + blockIdx.y, Srows = Rw * G, SP = P, shift = rowmap(u);
+    P -= shift;
+    Rw = min(Rw, P);
+    const int rows = Rw * G;
     for (int row = threadIdx.x; row < rows; row += kPT) {
         const int rslot = (P - Rw + row / G + shift) % R;
         cs[row] = ring_c[((size_t)u * R + rslot) * Gs + row % G];
@@ -154,14 +166,14 @@ __global__ void __launch_bounds__(kPT) prefill_fuse_kernel(const float *__restri
     __syncthreads();
     const int j = blockIdx.x * kPT + threadIdx.x;
     if (j >= P - Rw) return;
-    const float *s = S + (size_t)blockIdx.y * rows * P + j;
+    const float *s = S + (size_t)blockIdx.y * Srows * SP + j;
     float F = 0.f;
     for (int i = 0; i < Rw; ++i) {
         float Sr = 0.f;
-        for (int g = 0; g < G; ++g) Sr += exp2f(s[(size_t)(i * G + g) * P] - cs[i * G + g]);
+        for (int g = 0; g < G; ++g) Sr += exp2f(s[(size_t)(i * G + g) * SP] - cs[i * G + g]);
         F = fuse(fusion, F, Sr);
     }
-    Fp[(size_t)blockIdx.y * P + j] = F;
+    Fp[(size_t)blockIdx.y * SP + j] = F;
 }
 
 // Top-C of the M = P - Rw older tokens by (F descending, position ascending): an 8-pass
@@ -169,16 +181,23 @@ __global__ void __launch_bounds__(kPT) prefill_fuse_kernel(const float *__restri
 // lists the kept positions, followed by the window positions.
 constexpr int kSelT = 1024;  // threads of the selection kernel: a pass is a chain of rounds of kSelT keys
 __global__ void __launch_bounds__(kSelT) prefill_select_kernel(const float *__restrict__ Fp, int *__restrict__ pos, int ub0,
-                                                               int P, int Rw, int C, int cap)
+                                                               int P, int Rw, int C, int cap, RowMap rowmap)
 {
     __shared__ unsigned int hist[256];
     __shared__ unsigned long long prefix_s;
     __shared__ int remaining_s, done_s;
     __shared__ int wtot[kSelT / 32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int u = ub0 + blockIdx.x, M = P - Rw;
+    const int u = ub0 + blockIdx.x;
     const float *F = Fp + (size_t)blockIdx.x * P;
     int *upos = pos + (size_t)u * cap;
+    P -= rowmap(u);
+    Rw = min(Rw, P);
+    const int M = P - Rw;
+    if (M <= C) {               // a shorter row whose whole prompt fits
+        for (int i = tid; i < P; i += kSelT) upos[i] = i;
+        return;
+    }
     unsigned long long prefix = 0;
     int remaining = C;
     constexpr int kSelBatch = 4;                                         // keys per thread in flight
@@ -268,11 +287,11 @@ __global__ void __launch_bounds__(kSelT) prefill_select_kernel(const float *__re
     for (int i = tid; i < Rw; i += kSelT) upos[C + i] = M + i;
 }
 
-__global__ void prefill_identity_pos_kernel(int *pos, int U, int n, int cap)
+__global__ void prefill_identity_pos_kernel(int *pos, int U, int n, int cap, RowMap rowmap)
 {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (size_t)U * n) return;
-    pos[(i / n) * cap + (i % n)] = (int)(i % n);
+    if ((int)(i % n) < n - rowmap((int)(i / n))) pos[(i / n) * cap + (i % n)] = (int)(i % n);
 }
 
 // K/V rows of the kept prompt positions into the arena, 16 bytes per thread.  The free slots n .. cap-1 are cleared: the
@@ -280,13 +299,15 @@ __global__ void prefill_identity_pos_kernel(int *pos, int U, int n, int cap)
 // and written in 80 us for 256 units of 2032 slots.  Clearing the whole arena first, as two memsets, wrote every kept
 // row twice.)
 template <typename T, int D>
-__global__ void prefill_gather_kernel(const T *__restrict__ k, const T *__restrict__ v, DecodeArgs a, int Ps, int n)
+__global__ void prefill_gather_kernel(const T *__restrict__ k, const T *__restrict__ v, DecodeArgs a, int P, int Ps, RowMap rowmap)
 {
     constexpr int CH = D * sizeof(T) / 16;
     const int u = blockIdx.x;
     const int idx = blockIdx.y * blockDim.x + threadIdx.x;
     if (idx >= a.cap * CH) return;
     const int slot = idx / CH, c = idx % CH;
+    P -= rowmap(u);
+    const int n = min(P, a.C + min(P, a.R));
     uint4 *Kd = reinterpret_cast<uint4 *>(static_cast<T *>(a.K) + ((size_t)u * a.cap + slot) * D) + c;
     uint4 *Vd = reinterpret_cast<uint4 *>(static_cast<T *>(a.V) + ((size_t)u * a.cap + slot) * D) + c;
     if (slot >= n) {
@@ -303,9 +324,11 @@ __global__ void prefill_gather_kernel(const T *__restrict__ k, const T *__restri
 
 // window queries into their ring rows (row p % R); the rows that a prompt shorter than the window leaves empty are zero
 template <typename T, int D>
-__global__ void prefill_ring_kernel(const T *__restrict__ qwin, DecodeArgs a, int P, int Rw, int Rws, int shift)
+__global__ void prefill_ring_kernel(const T *__restrict__ qwin, DecodeArgs a, int P, int Rws, RowMap rowmap)
 {
-    const int u = blockIdx.x, G = a.G, Gq = a.Gq;       // heads Gq .. G-1 of a ring slot are padding (zero query)
+    const int u = blockIdx.x, G = a.G, Gq = a.Gq, shift = rowmap(u);
+    P -= shift;
+    const int Rw = min(P, a.R);                         // heads Gq .. G-1 of a ring slot are padding (zero query)
     T *rq = static_cast<T *>(a.ring_q) + (size_t)u * a.R * G * D;
     for (int idx = threadIdx.x; idx < a.R * G * D; idx += blockDim.x) {
         const int dd = idx % D, g = (idx / D) % G, i = idx / (D * G);
@@ -317,12 +340,14 @@ __global__ void prefill_ring_kernel(const T *__restrict__ qwin, DecodeArgs a, in
 
 // the same, 16 bytes per thread (q_window 16-byte aligned)
 template <typename T, int D>
-__global__ void prefill_ring_vec_kernel(const T *__restrict__ qwin, DecodeArgs a, int P, int Rw, int Rws, int shift)
+__global__ void prefill_ring_vec_kernel(const T *__restrict__ qwin, DecodeArgs a, int P, int Rws, RowMap rowmap)
 {
     constexpr int CH = D * sizeof(T) / 16;
-    const int u = blockIdx.x, G = a.G, Gq = a.Gq;
+    const int u = blockIdx.x, G = a.G, Gq = a.Gq, shift = rowmap(u);
     const int idx = blockIdx.y * blockDim.x + threadIdx.x;
     if (idx >= a.R * G * CH) return;
+    P -= shift;
+    const int Rw = min(P, a.R);
     const int c = idx % CH, g = (idx / CH) % G, i = idx / (CH * G);
     const int rslot = (P - Rw + i + shift) % a.R;
     uint4 v = make_uint4(0, 0, 0, 0);
@@ -337,13 +362,16 @@ __global__ void prefill_ring_vec_kernel(const T *__restrict__ qwin, DecodeArgs a
 // tokens that were kept and that the row may see, c = log2 sum exp2(s), from the arena as it stands (kept K rows,
 // their positions, the ring's queries).  One CTA per (window row, unit).
 template <typename T, int D>
-__global__ void __launch_bounds__(kPT) prefill_renorm_kernel(DecodeArgs a, int P, int Rw, int n, int shift)
+__global__ void __launch_bounds__(kPT) prefill_renorm_kernel(DecodeArgs a, int P, RowMap rowmap)
 {
     __shared__ float qs[D];
     __shared__ float red[kPT / 32];
     __shared__ float bc;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int u = blockIdx.y, G = a.G, row = blockIdx.x, i = row / G, g = row % G;
+    const int u = blockIdx.y, G = a.G, row = blockIdx.x, i = row / G, g = row % G, shift = rowmap(u);
+    P -= shift;
+    const int Rw = min(P, a.R), n = a.C + Rw;
+    if (i >= Rw || P <= n) return;                                    // everything was kept
     const int rpos = P - Rw + i, rslot = (rpos + shift) % a.R;
     float *c_out = a.ring_c + ((size_t)u * a.R + rslot) * G + g;
     if (*c_out == INFINITY) return;                                   // padding head
@@ -392,11 +420,12 @@ __global__ void __launch_bounds__(kPT) prefill_renorm_kernel(DecodeArgs a, int P
 
 template <typename T, int D>
 cudaError_t run_prefill_t(const DecodeArgs &a, const T *k, const T *v, const T *qwin, int P, cudaStream_t stream,
-                          unsigned long long *launches, float *S, size_t scratch_floats, int n_states, const PrefillRow *row)
+                          unsigned long long *launches, float *S, size_t scratch_floats, int n_states, int padded_len)
 {
-    // `row`: the units of `a` are one batch row of a ragged batch - the tensors are padded to the longest prompt, the
-    // ring slots follow the common time axis, the caller sets the step state and synchronises after the last row
-    const int Ps = row ? row->kv_stride : P, shift = row ? row->shift : 0;
+    // With prompts of different lengths (a.row_shift) P is the longest one and the tensors are padded to padded_len
+    // tokens; the ring slots follow the common time axis, on which every row ends at P.
+    const RowMap rowmap = {a.row_shift, a.Hkv, a.B};
+    const int Ps = padded_len, Rws = min(Ps, a.R);
     const int U = a.U, G = a.G, R = a.R, C = a.C;
     // the CUDA-core scoring kernels work on the model's Gq heads per window position (rows of S); the ring keeps G
     // heads per slot, the padding heads with normaliser +inf from init_arena_kernel
@@ -407,8 +436,7 @@ cudaError_t run_prefill_t(const DecodeArgs &a, const T *k, const T *v, const T *
     // bf16 / head_dim 128 shapes score on the tensor cores (two passes over the keys, no rows x P table); the
     // others materialise the window-row logits S [rows][P] per unit and reduce them with CUDA-core kernels
     // (the arena's group must be the padded one: a context that runs the CUDA-core decode kernel keeps G as it is)
-    const bool tc = !row && prefill_tc_supported(sizeof(T) == 4, D, a.Gq, R, k, P) && tc_padded_group(a.Gq) == G;
-    const int Rws = row ? row->qw_stride : Rw;
+    const bool tc = prefill_tc_supported(sizeof(T) == 4, D, a.Gq, R, k, P) && tc_padded_group(a.Gq) == G;
     const int tc_splits = tc ? prefill_tc_splits(U, P, Rw * G) : 0;
     const size_t per_unit = tc ? prefill_tc_floats_per_unit(P, Rw, G, tc_splits) : (size_t)rows * P + P;   // floats
     if (per_unit + 1 > scratch_floats) return cudaErrorInvalidConfiguration;
@@ -433,40 +461,39 @@ cudaError_t run_prefill_t(const DecodeArgs &a, const T *k, const T *v, const T *
     for (int ub0 = 0; ub0 < U; ub0 += (int)ub) {
         const int nb = min((int)ub, U - ub0);
         if (tc) {
-            e = run_prefill_scores_tc(a, k, qwin, P, ub0, nb, tc_splits, Fp, part, err_word, launches, stream);
+            e = run_prefill_scores_tc(a, k, qwin, P, Ps, ub0, nb, tc_splits, Fp, part, err_word, launches, stream);
             if (e != cudaSuccess) return e;
         } else {
             prefill_logits_kernel<T, D><<<dim3((P + kPK - 1) / kPK, nb), kPT, logits_smem, stream>>>(k, qwin, S, ub0, P, Rw,
-                                                                                                 a.Gq, a.scale2, Ps, Rws);
-            prefill_rowstats_kernel<<<dim3(rows, nb), kPT, 0, stream>>>(S, a.ring_c, ub0, P, Rw, a.Gq, G, R, shift);
+                                                                                                 a.Gq, a.scale2, Ps, Rws, rowmap);
+            prefill_rowstats_kernel<<<dim3(rows, nb), kPT, 0, stream>>>(S, a.ring_c, ub0, P, Rw, a.Gq, G, R, rowmap);
             *launches += 2;
         }
         if (select) {
             if (!tc) {
                 prefill_fuse_kernel<<<dim3((P - Rw + kPT - 1) / kPT, nb), kPT, rows * sizeof(float), stream>>>(
-                    S, a.ring_c, Fp, ub0, P, Rw, a.Gq, G, R, a.fusion, shift);
+                    S, a.ring_c, Fp, ub0, P, Rw, a.Gq, G, R, a.fusion, rowmap);
                 ++*launches;
             }
-            prefill_select_kernel<<<nb, kSelT, 0, stream>>>(Fp, a.pos, ub0, P, Rw, C, a.cap);
+            prefill_select_kernel<<<nb, kSelT, 0, stream>>>(Fp, a.pos, ub0, P, Rw, C, a.cap, rowmap);
             ++*launches;
         }
     }
     if (!select) {
-        prefill_identity_pos_kernel<<<(unsigned)(((size_t)U * n + 255) / 256), 256, 0, stream>>>(a.pos, U, n, a.cap);
+        prefill_identity_pos_kernel<<<(unsigned)(((size_t)U * n + 255) / 256), 256, 0, stream>>>(a.pos, U, n, a.cap, rowmap);
         ++*launches;
     }
     constexpr int CH = D * sizeof(T) / 16;
-    prefill_gather_kernel<T, D><<<dim3(U, (a.cap * CH + 255) / 256), 256, 0, stream>>>(k, v, a, Ps, n);
+    prefill_gather_kernel<T, D><<<dim3(U, (a.cap * CH + 255) / 256), 256, 0, stream>>>(k, v, a, P, Ps, rowmap);
     if (((uintptr_t)qwin & 15) == 0)
-        prefill_ring_vec_kernel<T, D><<<dim3(U, (R * G * CH + 255) / 256), 256, 0, stream>>>(qwin, a, P, Rw, Rws, shift);
+        prefill_ring_vec_kernel<T, D><<<dim3(U, (R * G * CH + 255) / 256), 256, 0, stream>>>(qwin, a, P, Rws, rowmap);
     else
-        prefill_ring_kernel<T, D><<<U, 256, 0, stream>>>(qwin, a, P, Rw, Rws, shift);
+        prefill_ring_kernel<T, D><<<U, 256, 0, stream>>>(qwin, a, P, Rws, rowmap);
     if (a.norm_current && select) {
-        prefill_renorm_kernel<T, D><<<dim3(Rw * G, U), kPT, 0, stream>>>(a, P, Rw, n, shift);
+        prefill_renorm_kernel<T, D><<<dim3(Rw * G, U), kPT, 0, stream>>>(a, P, rowmap);
         ++*launches;
     }
     *launches += 2;
-    if (row) return cudaGetLastError();
     e = cudaGetLastError();
     if (e == cudaSuccess) e = launch_finish_prompt(a, P, n, n_states, err_word, launches, stream);
     const cudaError_t e2 = cudaStreamSynchronize(stream);
@@ -482,17 +509,17 @@ cudaError_t run_prefill_t(const DecodeArgs &a, const T *k, const T *v, const T *
 
 cudaError_t dispatch_prefill(const DecodeArgs &a, bool f32, int D, const void *k, const void *v, const void *q_window, int P,
                              cudaStream_t stream, unsigned long long *launches, float *S, size_t scratch_floats, int n_states,
-                             const PrefillRow *row = nullptr)
+                             int padded_len)
 {
     if (f32) {
         auto kk = static_cast<const float *>(k), vv = static_cast<const float *>(v), qq = static_cast<const float *>(q_window);
-        return D == 64 ? run_prefill_t<float, 64>(a, kk, vv, qq, P, stream, launches, S, scratch_floats, n_states, row)
-                       : run_prefill_t<float, 128>(a, kk, vv, qq, P, stream, launches, S, scratch_floats, n_states, row);
+        return D == 64 ? run_prefill_t<float, 64>(a, kk, vv, qq, P, stream, launches, S, scratch_floats, n_states, padded_len)
+                       : run_prefill_t<float, 128>(a, kk, vv, qq, P, stream, launches, S, scratch_floats, n_states, padded_len);
     }
     auto kk = static_cast<const __nv_bfloat16 *>(k), vv = static_cast<const __nv_bfloat16 *>(v),
          qq = static_cast<const __nv_bfloat16 *>(q_window);
-    return D == 64 ? run_prefill_t<__nv_bfloat16, 64>(a, kk, vv, qq, P, stream, launches, S, scratch_floats, n_states, row)
-                   : run_prefill_t<__nv_bfloat16, 128>(a, kk, vv, qq, P, stream, launches, S, scratch_floats, n_states, row);
+    return D == 64 ? run_prefill_t<__nv_bfloat16, 64>(a, kk, vv, qq, P, stream, launches, S, scratch_floats, n_states, padded_len)
+                   : run_prefill_t<__nv_bfloat16, 128>(a, kk, vv, qq, P, stream, launches, S, scratch_floats, n_states, padded_len);
 }
 
 // ---- scratch of mkv_prefill_static -------------------------------------------------------------------------
@@ -529,10 +556,10 @@ cudaError_t static_scratch_address(int device, float **out)
 
 cudaError_t run_prefill(const DecodeArgs &a, bool f32, int D, const void *k, const void *v, const void *q_window, int P,
                         cudaStream_t stream, unsigned long long *launches, PrefillScratch *scratch, int n_states,
-                        const PrefillRow *row)
+                        int padded_len)
 {
     const int Rw = P < a.R ? P : a.R;
-    const bool tc = !row && prefill_tc_supported(f32, D, a.Gq, a.R, k, P) && tc_padded_group(a.Gq) == a.G;
+    const bool tc = prefill_tc_supported(f32, D, a.Gq, a.R, k, P) && tc_padded_group(a.Gq) == a.G;
     const size_t per_unit = (tc ? prefill_tc_floats_per_unit(P, Rw, a.G, prefill_tc_splits(a.U, P, Rw * a.G))
                                 : (size_t)Rw * a.G * P + P) * sizeof(float);
     size_t ub = ((size_t)1 << 30) / per_unit;
@@ -552,7 +579,7 @@ cudaError_t run_prefill(const DecodeArgs &a, bool f32, int D, const void *k, con
         scratch->bytes = need;
     }
     return dispatch_prefill(a, f32, D, k, v, q_window, P, stream, launches, static_cast<float *>(scratch->ptr),
-                            scratch->bytes / sizeof(float), n_states, row);
+                            scratch->bytes / sizeof(float), n_states, padded_len);
 }
 
 namespace {
@@ -583,7 +610,7 @@ cudaError_t run_prefill_static(const DecodeArgs &a, bool f32, int D, const void 
     float *S = nullptr;
     const cudaError_t e = static_scratch_address(device, &S);
     if (e != cudaSuccess) return e;
-    return dispatch_prefill(a, f32, D, k, v, q_window, P, stream, launches, S, kStaticScratchFloats, n_states);
+    return dispatch_prefill(a, f32, D, k, v, q_window, P, stream, launches, S, kStaticScratchFloats, n_states, P);
 }
 
 }  // namespace mkv
