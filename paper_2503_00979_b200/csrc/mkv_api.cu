@@ -28,6 +28,7 @@ struct Shape {
     int B, Hkv;             // batch rows and KV heads (upl = B * Hkv)
     int U, G, D, R, C, cap, splits, T, tc_grid_size, tc_grid_layer;
     int Gq;                 // the model's GQA ratio; G is it rounded up to a power of two on the tensor-core path
+    int simt_splits, simt_splits_layer;   // warp-level kernel: CTAs per unit of a whole-stack launch, of a layer's
     int nc;                 // ring chunks of the tensor-core kernel (1 unless CURRENT and the window has more than 256 rows)
     int bs, nblk;           // slots per block of the ring and blocks (DecodeArgs::slab)
     size_t es;
@@ -137,12 +138,17 @@ bool resolve(const mkv_params *p, Shape *s, KernelKind *kind)
     }
     if (stored) return false;
     *kind = kKindSimt;
-    s->bs = s->R;
-    s->nblk = 1;
+    s->bs = current ? 0 : simt_block_slots(p->dtype == MKV_DTYPE_F32, s->G, s->R);
+    if (s->bs == 0) s->bs = s->R;
+    s->nblk = (s->R + s->bs - 1) / s->bs;
     const int max_splits = (s->cap + 31) / 32;
     int sp = p->splits > 0 ? p->splits : simt_default_splits(s->U, s->cap);
     if (sp > max_splits) sp = max_splits;
-    s->splits = sp;
+    int sp_layer = p->splits > 0 ? sp : simt_default_splits(s->upl, s->cap);
+    if (sp_layer > max_splits) sp_layer = max_splits;
+    s->simt_splits = sp;
+    s->simt_splits_layer = sp_layer;
+    s->splits = std::max(sp, sp_layer);
     s->tc_grid_size = 0;
     s->tc_grid_layer = 0;
     return true;
@@ -274,7 +280,8 @@ mkv_status launch_step(mkv_ctx *ctx, int layer, const void *q, const void *k, co
         }
     }
     const cudaError_t e = ctx->kind == kKindTc ? launch_decode_tc(layer < 0 ? ctx->plan : ctx->plan_layer, a, stream)
-                                               : launch_decode_simt(a, ctx->p.dtype == MKV_DTYPE_F32, ctx->s.D, stream);
+                                               : launch_decode_simt(a, layer < 0 ? ctx->s.simt_splits : ctx->s.simt_splits_layer,
+                                                                     ctx->p.dtype == MKV_DTYPE_F32, ctx->s.D, stream);
     if (e != cudaSuccess) return fail(ctx, MKV_CUDA, "decode launch failed: %s", cudaGetErrorString(e));
     ctx->launches += 1;
     const bool ev = step_scores(ctx->t, ctx->n, ctx->steps, ctx->s.R, ctx->s.C, ctx->s.T);

@@ -14,8 +14,7 @@ constexpr int kFusionSum = 0;
 constexpr int kFusionMax = 1;
 
 // Device-resident step state.  Kernels read it at entry and one CTA of each launch advances it
-// (the last one to finish in the CUDA-core kernel, the last one to have read it in the
-// tensor-core kernel), so consecutive launches need no host-side step index.
+// (the last one to have read it), so consecutive launches need no host-side step index.
 struct DevState {
     long long t;          // absolute position of the token being decoded
     int n;                // tokens cached per unit before this step
@@ -209,6 +208,19 @@ __host__ __device__ inline int open_block(long long t, int R, int bs) { return (
 __host__ __device__ inline bool step_opens_block(long long t, int R, int bs, int nblk)
 {
     return nblk > 1 && (int)(t % R) % bs == 0;
+}
+
+// The fused score S of ring block j joins the sums of one key; blocks come in descending order, acc and pre run along.
+__device__ __forceinline__ void take_block(float S, int j, int open, int fusion, float *slab, size_t cap, bool valid,
+                                           float &acc, float &pre)
+{
+    if (j > open) {
+        acc = fuse(fusion, acc, S);
+        if (valid) slab[(size_t)j * cap] = acc;
+    } else if (j < open) {
+        pre = fuse(fusion, pre, S);
+        if (valid) slab[(size_t)j * cap] = S;
+    }
 }
 
 // CURRENT normalisation (the reading of Eq. 4 in which a window row's weights are taken over the tokens that are
@@ -432,22 +444,6 @@ __device__ void finalize_unit(const DecodeArgs &a, int u, long long t, int n, in
         if (a.nblk > 1) a.sum_pos[(size_t)u * a.cap + e_slot] = (int)(t - shift);
         a.evicted_pos[u] = e_pos;
         a.ticket[u] = 0;
-    }
-}
-
-// Last action of every CTA of a decode launch: the CTA that finishes last advances the
-// device-resident step state.  Must be called by all CTAs, after all their other work,
-// so that no CTA can still be about to read the state when it changes.
-__device__ __forceinline__ void finish_cta(const DecodeArgs &a, long long t, int n, bool evict)
-{
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        const unsigned int total = gridDim.x * gridDim.y * gridDim.z;
-        if (atomicAdd(&a.st->done, 1u) == total - 1) {
-            advance_state(a, t, n, a.st->steps, evict);
-            __threadfence();
-        }
     }
 }
 

@@ -5,8 +5,9 @@
 
 namespace mkv {
 
-// CUDA-core decode step (any supported shape).  `a.splits` CTAs per unit.
-cudaError_t launch_decode_simt(const DecodeArgs &a, bool f32, int D, cudaStream_t stream);
+// Warp-level decode step (any supported shape).  `nsplit` CTAs per unit, at most a.splits.
+cudaError_t launch_decode_simt(const DecodeArgs &a, int nsplit, bool f32, int D, cudaStream_t stream);
+int simt_block_slots(bool f32, int G, int R);      // slots per block of the ring (DecodeArgs::bs), 0: no sums are kept
 int simt_default_splits(int U, int cap);
 
 // Coarse-grained eviction (evict_interval > 1): drops everything beyond the top C after a step that scored and
@@ -65,10 +66,10 @@ cudaError_t run_prefill_static(const DecodeArgs &a, bool f32, int D, const void 
 // The window sums (DecodeArgs::slab) of the slots whose token is no longer the one in sum_pos, for the step that a.st
 // holds.  *launches counts the launches.
 cudaError_t launch_window_sums(const DecodeArgs &a, bool f32, int D, unsigned long long *launches, cudaStream_t stream);
-// Last launch(es) of the prompt phase: the window sums of every slot, where the context keeps them, for the step at
-// position t of n cached tokens, and the n_states step states at a.st.  `err`: word in which a wait that runs out is
+// Last launch(es) of the prompt phase: if `sums`, the window sums of every slot, where the context keeps them, for the
+// step at position t of n cached tokens, and the n_states step states at a.st.  `err`: word in which a wait that runs out is
 // reported.
-cudaError_t launch_finish_prompt(const DecodeArgs &a, long long t, int n, int n_states, int *err, unsigned long long *launches,
+cudaError_t launch_finish_prompt(const DecodeArgs &a, bool sums, long long t, int n, int n_states, int *err, unsigned long long *launches,
                                  cudaStream_t stream);
 
 // Copies one step state over n_dst others (the whole-stack state and the per-layer states are brought level when

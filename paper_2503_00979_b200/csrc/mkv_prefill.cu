@@ -287,6 +287,39 @@ __global__ void __launch_bounds__(kSelT) prefill_select_kernel(const float *__re
     for (int i = tid; i < Rw; i += kSelT) upos[C + i] = M + i;
 }
 
+// The window sums (DecodeArgs::slab) of the kept slots from the window-row logits S, which the scoring without the tensor
+// cores leaves behind: one slot per thread.
+__global__ void __launch_bounds__(kPT) prefill_sums_kernel(const float *__restrict__ S, DecodeArgs a, int ub0, int P, int Rw, int Gs,
+                                                           RowMap rowmap)
+{
+    extern __shared__ float cs[];   // [R * Gq]
+    const int u = ub0 + blockIdx.y, G = a.Gq, Srows = Rw * G, SP = P, shift = rowmap(u), open = open_block(P, a.R, a.bs);
+    P -= shift;
+    Rw = min(Rw, P);
+    for (int i = threadIdx.x; i < a.R * G; i += kPT) cs[i] = a.ring_c[((size_t)u * a.R + i / G) * Gs + i % G];
+    __syncthreads();
+    const int k = blockIdx.x * kPT + threadIdx.x;
+    if (k >= a.cap) return;
+    const size_t at = (size_t)u * a.cap + k;
+    const int p = a.pos[at];
+    a.sum_pos[at] = p;
+    if (p < 0) return;                                                    // free
+    const float *s = S + (size_t)blockIdx.y * Srows * SP + p;
+    float acc = 0.f, pre = 0.f;
+    for (int j = a.nblk - 1; j >= 0; --j) {
+        float F = 0.f;
+        for (int r = j * a.bs; r < min(a.R, (j + 1) * a.bs); ++r) {
+            const int i = ((r - (P - Rw + shift)) % a.R + a.R) % a.R;     // window row in ring slot r
+            if (i >= Rw) continue;
+            float Sr = 0.f;
+            for (int g = 0; g < G; ++g) Sr += exp2f(s[(size_t)(i * G + g) * SP] - cs[r * G + g]);
+            F = fuse(a.fusion, F, Sr);
+        }
+        take_block(F, j, open, a.fusion, a.slab + (size_t)u * a.nblk * a.cap + k, a.cap, true, acc, pre);
+    }
+    a.pre[at] = pre;
+}
+
 __global__ void prefill_identity_pos_kernel(int *pos, int U, int n, int cap, RowMap rowmap)
 {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -458,6 +491,12 @@ cudaError_t run_prefill_t(const DecodeArgs &a, const T *k, const T *v, const T *
         e = cudaMemsetAsync(err_word, 0, sizeof(int), stream);
         if (e != cudaSuccess) return e;
     }
+    if (!select) {
+        prefill_identity_pos_kernel<<<(unsigned)(((size_t)U * n + 255) / 256), 256, 0, stream>>>(a.pos, U, n, a.cap, rowmap);
+        ++*launches;
+    }
+    // the window sums: on the tensor cores at the end, or from the logits S where there are any
+    const bool sums_tc = sizeof(T) == 2 && D == 128 && tc_padded_group(a.Gq) == G;
     for (int ub0 = 0; ub0 < U; ub0 += (int)ub) {
         const int nb = min((int)ub, U - ub0);
         if (tc) {
@@ -478,10 +517,10 @@ cudaError_t run_prefill_t(const DecodeArgs &a, const T *k, const T *v, const T *
             prefill_select_kernel<<<nb, kSelT, 0, stream>>>(Fp, a.pos, ub0, P, Rw, C, a.cap, rowmap);
             ++*launches;
         }
-    }
-    if (!select) {
-        prefill_identity_pos_kernel<<<(unsigned)(((size_t)U * n + 255) / 256), 256, 0, stream>>>(a.pos, U, n, a.cap, rowmap);
-        ++*launches;
+        if (a.nblk > 1 && !sums_tc) {
+            prefill_sums_kernel<<<dim3((a.cap + kPT - 1) / kPT, nb), kPT, R * a.Gq * sizeof(float), stream>>>(S, a, ub0, P, Rw, G, rowmap);
+            ++*launches;
+        }
     }
     constexpr int CH = D * sizeof(T) / 16;
     prefill_gather_kernel<T, D><<<dim3(U, (a.cap * CH + 255) / 256), 256, 0, stream>>>(k, v, a, P, Ps, rowmap);
@@ -495,7 +534,7 @@ cudaError_t run_prefill_t(const DecodeArgs &a, const T *k, const T *v, const T *
     }
     *launches += 2;
     e = cudaGetLastError();
-    if (e == cudaSuccess) e = launch_finish_prompt(a, P, n, n_states, err_word, launches, stream);
+    if (e == cudaSuccess) e = launch_finish_prompt(a, sums_tc, P, n, n_states, err_word, launches, stream);
     const cudaError_t e2 = cudaStreamSynchronize(stream);
     if (e != cudaSuccess || e2 != cudaSuccess) return e != cudaSuccess ? e : e2;
     if (waits) {    // a bounded wait that ran out

@@ -47,19 +47,6 @@ __device__ __forceinline__ void set_states(const SumArgs &a)
     }
 }
 
-// The fused score S of ring block j joins the sums of one key; blocks come in descending order, acc and pre run along.
-__device__ __forceinline__ void take_block(float S, int j, int open, int fusion, float *slab, size_t cap, bool valid,
-                                           float &acc, float &pre)
-{
-    if (j > open) {
-        acc = fuse(fusion, acc, S);
-        if (valid) slab[(size_t)j * cap] = acc;
-    } else if (j < open) {
-        pre = fuse(fusion, pre, S);
-        if (valid) slab[(size_t)j * cap] = S;
-    }
-}
-
 template <int G, int FUSION>
 __global__ void __launch_bounds__(kSumThreads, 2)
 window_sums_tc_kernel(const __grid_constant__ SumArgs a, const __grid_constant__ CUtensorMap tmK)
@@ -300,7 +287,7 @@ cudaError_t launch_window_sums(const DecodeArgs &d, bool f32, int D, unsigned lo
     return cudaGetLastError();
 }
 
-cudaError_t launch_finish_prompt(const DecodeArgs &d, long long t, int n, int n_states, int *err, unsigned long long *launches,
+cudaError_t launch_finish_prompt(const DecodeArgs &d, bool sums, long long t, int n, int n_states, int *err, unsigned long long *launches,
                                  cudaStream_t stream)
 {
     SumArgs a;
@@ -308,7 +295,7 @@ cudaError_t launch_finish_prompt(const DecodeArgs &d, long long t, int n, int n_
     a.d = d;
     a.t = t; a.n = n; a.err = err;
     a.wait_cycles = kWaitCycles;
-    if (d.nblk <= 1) {
+    if (d.nblk <= 1 || !sums) {
         a.set_states = n_states;
         set_states_kernel<<<1, 32, 0, stream>>>(a);
         ++*launches;
