@@ -28,7 +28,7 @@ struct Shape {
     int B, Hkv;             // batch rows and KV heads (upl = B * Hkv)
     int U, G, D, R, C, cap, splits, T, tc_grid_size, tc_grid_layer;
     int Gq;                 // the model's GQA ratio; G is it rounded up to a power of two on the tensor-core path
-    int simt_splits, simt_splits_layer;   // warp-level kernel: CTAs per unit of a whole-stack launch, of a layer's
+    int simt_splits, simt_splits_layer;   // warp-level kernel: CTAs per unit of a whole-stack launch, of a layer's (0: not used)
     int nc;                 // ring chunks of the tensor-core kernel (1 unless CURRENT and the window has more than 256 rows)
     int bs, nblk;           // slots per block of the ring and blocks (DecodeArgs::slab)
     size_t es;
@@ -134,6 +134,9 @@ bool resolve(const mkv_params *p, Shape *s, KernelKind *kind)
         const int sp_layer = std::max(tc_partials_per_unit(s->upl * nc, s->cap, s->tc_grid_layer),
                                       tc_partials_per_unit(s->upl, s->cap, s->tc_grid_layer));
         s->splits = sp_all > sp_layer ? sp_all : sp_layer;
+        const bool may = p->kernel == MKV_KERNEL_AUTO && !current;
+        s->simt_splits = may ? simt_small_splits(s->U, s->Gq, s->R, s->bs, s->nblk, s->cap) : 0;
+        s->simt_splits_layer = may ? simt_small_splits(s->upl, s->Gq, s->R, s->bs, s->nblk, s->cap) : 0;
         return true;
     }
     if (stored) return false;
@@ -141,7 +144,7 @@ bool resolve(const mkv_params *p, Shape *s, KernelKind *kind)
     s->bs = current ? 0 : simt_block_slots(p->dtype == MKV_DTYPE_F32, s->G, s->R);
     if (s->bs == 0) s->bs = s->R;
     s->nblk = (s->R + s->bs - 1) / s->bs;
-    const int max_splits = (s->cap + 31) / 32;
+    const int max_splits = std::min(16, (s->cap + 31) / 32);
     int sp = p->splits > 0 ? p->splits : simt_default_splits(s->U, s->cap);
     if (sp > max_splits) sp = max_splits;
     int sp_layer = p->splits > 0 ? sp : simt_default_splits(s->upl, s->cap);
@@ -279,9 +282,11 @@ mkv_status launch_step(mkv_ctx *ctx, int layer, const void *q, const void *k, co
             if (ef != cudaSuccess) return fail(ctx, MKV_CUDA, "window sums launch failed: %s", cudaGetErrorString(ef));
         }
     }
-    const cudaError_t e = ctx->kind == kKindTc ? launch_decode_tc(layer < 0 ? ctx->plan : ctx->plan_layer, a, stream)
-                                               : launch_decode_simt(a, layer < 0 ? ctx->s.simt_splits : ctx->s.simt_splits_layer,
-                                                                     ctx->p.dtype == MKV_DTYPE_F32, ctx->s.D, stream);
+    const int nsplit = layer < 0 ? ctx->s.simt_splits : ctx->s.simt_splits_layer;
+    // (of two layers or more, the launch before a layer's is another layer's, or no programmatic predecessor at all)
+    const bool early = layer >= 0 && ctx->s.layers > 1;
+    const cudaError_t e = nsplit > 0 ? launch_decode_simt(a, nsplit, early, ctx->p.dtype == MKV_DTYPE_F32, ctx->s.D, stream)
+                                     : launch_decode_tc(layer < 0 ? ctx->plan : ctx->plan_layer, a, stream);
     if (e != cudaSuccess) return fail(ctx, MKV_CUDA, "decode launch failed: %s", cudaGetErrorString(e));
     ctx->launches += 1;
     const bool ev = step_scores(ctx->t, ctx->n, ctx->steps, ctx->s.R, ctx->s.C, ctx->s.T);
