@@ -125,9 +125,7 @@ bool resolve(const mkv_params *p, Shape *s, KernelKind *kind)
         s->nblk = current ? 1 : (s->R + s->bs - 1) / s->bs;
         // the persistent grid (148 SMs on B200; correctness does not depend on the count)
         s->tc_grid_size = tc_grid(s->U * nc, s->cap, p->splits, 148);
-        // a per-layer call sees only a layer's units: ranges of about an eighth of a unit's tiles, so that a layer
-        // of few units still spreads over the SMs while a unit stays within eight CTAs
-        s->tc_grid_layer = tc_grid(s->upl * nc, s->cap, p->splits > 0 ? p->splits : 8, 148);
+        s->tc_grid_layer = tc_grid(s->upl * nc, s->cap, p->splits, 148);      // a per-layer call sees only a layer's units
         // on a step without a policy decision only the main chunks are walked: take the worse of both schedules
         const int sp_all = std::max(tc_partials_per_unit(s->U * nc, s->cap, s->tc_grid_size),
                                     tc_partials_per_unit(s->U, s->cap, s->tc_grid_size));

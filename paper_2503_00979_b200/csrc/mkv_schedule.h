@@ -25,7 +25,24 @@ struct Item {
 // A unit cut by a range boundary is then worked on early by both CTAs that hold a piece of it (the one before the
 // boundary starts with it, the one after it takes it first or second), so its cross-CTA merge runs while tiles
 // still stream, and the item a CTA ends with is a unit all of its own, whose epilogue needs no other CTA.
-struct Walk {
+//
+// Whole units: where the ranges can be cut between units at the price of less than kMergeTiles tiles on the busiest CTA,
+// they are.  A unit that two CTAs share costs a partial, a ticket and a second epilogue in global memory, a chain of
+// round trips of about 5 us at the end of the launch; a tile costs about 1.26 us.  (112 units x 8 heads of 600 / 1030 /
+// 2030 slots on 112 CTAs against 148 in equal shares: 21.1 / 29.7 / 43.3 us per step against 26.4 / 36.3 / 43.1, shares
+// longer by 1.2 / 2.2 / 3.9 tiles; 256 units of 512 slots on 128 CTAs 20.7 against 29.3, 8192 of them 443 against 493.)
+constexpr int kMergeTiles = 4;
+
+// Whether whole units pay for a context of this capacity, and then at every fill.  (WHOLE is a template parameter because the
+// other kind of walk, with a run-time switch in it, cost the flagship's step 0.4 us.)
+inline bool sched_whole(int U, int cap, int grid)
+{
+    const long long nt = (cap + kSchedTile - 1) / kSchedTile;
+    return U > grid && ((U + grid - 1) / grid * (long long)grid - U) * nt < (long long)kMergeTiles * grid;
+}
+
+template <bool WHOLE>
+struct WalkT {
     int tile, tile_begin, tile_end;   // the host keeps U * tiles per unit below 2^31
     int nat_end;      // end of the part of the range that is handed out in tile order
     int lead_nk;      // tiles of the piece handed out first (0: none, or already handed out)
@@ -36,15 +53,20 @@ struct Walk {
     int eff;          // working CTAs
     int cta;          // this CTA
     long long total;
-    MKV_HD Walk(int U, int n, int grid, int cta_index)
+    MKV_HD WalkT(int U, int n, int grid, int cta_index)
     {
         nt = (n + kSchedTile - 1) / kSchedTile;
         total = (long long)U * nt;
         eff = (int)(total < (long long)grid ? total : (long long)grid);
         cta = cta_index;
         if (cta < eff) {
-            tile = (int)(total * cta / eff);
-            tile_end = (int)(total * (cta + 1) / eff);
+            if (WHOLE) {
+                tile = (int)((unsigned)U * cta / eff) * nt;           // (at most 2^24 units)
+                tile_end = (int)((unsigned)U * (cta + 1) / eff) * nt;
+            } else {
+                tile = (int)(total * cta / eff);
+                tile_end = (int)(total * (cta + 1) / eff);
+            }
         } else {
             tile = tile_end = 0;
         }
@@ -87,10 +109,15 @@ struct Walk {
         ++nitems;
     }
     // the CTA that owns global tile i: the largest c with c * T / E <= i
-    MKV_HD int owner(long long i) const { return (int)(((i + 1) * eff - 1) / total); }
+    MKV_HD int owner(long long i) const
+    {
+        if (WHOLE) i = i / nt * nt + nt - 1;            // the unit's last tile: (u + 1) * nt * E / T = (u + 1) * E / U
+        return (int)(((i + 1) * eff - 1) / total);
+    }
     // How many CTAs hold tiles of unit u, and this CTA's index among them.
     MKV_HD int ctas_of_unit(int u, int &my_index) const
     {
+        if (WHOLE) { my_index = 0; return 1; }
         const long long i0 = (long long)u * nt;
         const int c0 = owner(i0), c1 = owner(i0 + nt - 1);
         my_index = cta - c0;
@@ -98,8 +125,13 @@ struct Walk {
     }
 };
 
-// Grid of the persistent kernel.  `splits_hint` > 0 asks for about that many CTAs per unit
-// (ranges of cap_tiles / splits_hint tiles); otherwise one CTA per SM.
+using Walk = WalkT<false>;
+
+// Grid of the persistent kernel.  `splits_hint` > 0 asks for about that many CTAs per unit (ranges of
+// cap_tiles / splits_hint tiles).  Otherwise one CTA per SM, or a multiple of the units where that leaves the shares less
+// than kMergeTiles / 2 tiles longer: every unit is then cut into equal parts of its own and never shared by more CTAs than
+// it has parts (8 at most, what the fast epilogue merges), or is one CTA's alone, for which kMergeTiles are paid.
+// (64 units of 8 tiles in 128 parts 17.4 us per step against 21.1; 32 units of 16 tiles in 128 parts 18.8 against 22.9.)
 inline int sched_grid(int U, int cap, int splits_hint, int n_sm)
 {
     const long long ntiles = (cap + kSchedTile - 1) / kSchedTile, total = (long long)U * ntiles;
@@ -108,6 +140,13 @@ inline int sched_grid(int U, int cap, int splits_hint, int n_sm)
         const long long chunk = (ntiles + splits_hint - 1) / splits_hint;
         grid = (total + chunk - 1) / chunk;
         if (grid > n_sm) grid = n_sm;
+    } else if (U <= n_sm) {
+        long long parts = n_sm / U;
+        if (parts > 8) parts = 8;
+        if (parts > ntiles) parts = ntiles;
+        if (ntiles * n_sm - total < (long long)kMergeTiles * n_sm) grid = U;
+        else if (parts > 1 && 2 * (((ntiles + parts - 1) / parts) * n_sm - total) < (long long)kMergeTiles * n_sm) grid = U * parts;
+        else if (parts == 8) grid = U * parts;
     }
     if (grid > total) grid = total;
     return (int)(grid < 1 ? 1 : grid);

@@ -95,15 +95,15 @@ __host__ __device__ inline SmemLayout tc_smem_layout(const TcGeom &g, int G)
 struct TcPlan {
     CUtensorMap tmK, tmV, tmQ;
     TcGeom geo;
-    bool attr_set[3][2];      // [mode][ragged]: the instantiation's shared-memory limit has been raised
+    bool attr_set[4][2];      // [mode][ragged]: the instantiation's shared-memory limit has been raised
 };
 
 // Which ring rows a step of the kernel scores.
 //   kTcBlocks  the block of slots that is being filled; the rest of the window comes from kept sums (FROZEN
-//              normalisation: every step of every window)
+//              normalisation: every step of every window).  kTcBlocksWhole: and no unit is cut between CTAs
 //   kTcFull    all rows as one operand, kTcChunks all rows in chunks of up to 256 (CURRENT normalisation, whose
 //              weights all change with every eviction)
-enum TcMode { kTcFull = 0, kTcChunks = 1, kTcBlocks = 2 };
+enum TcMode { kTcFull = 0, kTcChunks = 1, kTcBlocks = 2, kTcBlocksWhole = 3 };
 
 namespace {
 
@@ -323,7 +323,7 @@ decode_tc_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ C
                  const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmQ,
                  const __grid_constant__ TcGeom geo)
 {
-    constexpr bool MC = MODE == kTcChunks, BLOCKS = MODE == kTcBlocks;
+    constexpr bool MC = MODE == kTcChunks, BLOCKS = MODE >= kTcBlocks, WHOLE = MODE == kTcBlocksWhole;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     // the swizzled operand tiles need a 1024-byte aligned base; the launch asks for 1 KB of slack
     unsigned char *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -378,7 +378,7 @@ decode_tc_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ C
     if constexpr (!MC && !RAGGED) {
         if ((tid == 0 || tid == 64) && a.n_hint > 0 && geo.prefetch_tiles > 0) {
             const CUtensorMap *pm = tid == 0 ? &tmK : &tmV;
-            Walk w(a.U, a.n_hint, (int)gridDim.x, (int)blockIdx.x);
+            WalkT<WHOLE> w(a.U, a.n_hint, (int)gridDim.x, (int)blockIdx.x);
             Item x;
             int left = geo.prefetch_tiles;
             while (left > 0 && w.next(x)) {
@@ -434,7 +434,7 @@ decode_tc_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ C
     if (warp == 0) {
         // ------------------------------------------------ TMA producer: query ring and K tiles (one lane)
         if (lane == 0) {
-            Walk w(a.U * NCe, n, (int)gridDim.x, (int)blockIdx.x);
+            WalkT<WHOLE> w(a.U * NCe, n, (int)gridDim.x, (int)blockIdx.x);
             Item x;
             int issued = 0, rings = 0;
             bool ok = true;
@@ -478,7 +478,7 @@ decode_tc_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ C
     } else if (warp == 2) {
         // ------------------------------------------------ TMA producer: V tiles (one lane)
         if (lane == 0) {
-            Walk w(a.U * NCe, n, (int)gridDim.x, (int)blockIdx.x);
+            WalkT<WHOLE> w(a.U * NCe, n, (int)gridDim.x, (int)blockIdx.x);
             Item x;
             int issued = 0;                                 // V tiles loaded so far (only main chunks read V)
             bool ok = true;
@@ -508,7 +508,7 @@ decode_tc_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ C
         __syncwarp();       // see the K producer
     } else if (warp == 1) {
         // ------------------------------------------------ new-query substitution + MMA issue
-        Walk w(a.U * NCe, n, (int)gridDim.x, (int)blockIdx.x);
+        WalkT<WHOLE> w(a.U * NCe, n, (int)gridDim.x, (int)blockIdx.x);
         Item x;
         const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NR >> 3) << 17) | ((uint32_t)(kTile >> 4) << 24);
         bool ok = true;
@@ -600,7 +600,7 @@ decode_tc_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ C
         int seg_tiles = 0;
         int npub = 0;                                  // partials this warp has handed to the epilogue group
 
-        Walk w(a.U * NCe, n, (int)gridDim.x, (int)blockIdx.x);
+        WalkT<WHOLE> w(a.U * NCe, n, (int)gridDim.x, (int)blockIdx.x);
         Item x;
         bool ok = true;
         int Tn = grp;                                  // next tile of this group
@@ -871,7 +871,7 @@ decode_tc_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ C
         int *flag = reinterpret_cast<int *>(epi + kFinFloats);
         float *cml = epi + kFinFloats + 8;                            // merged (m, l) [g][2]
         float *sc = cml + 2 * kMaxGroup;                              // [warp][g] scale to the merged reference
-        Walk w(a.U * NCe, n, (int)gridDim.x, (int)blockIdx.x);
+        WalkT<WHOLE> w(a.U * NCe, n, (int)gridDim.x, (int)blockIdx.x);
         Item x;
         bool ok = true;
         int k = 0;                                                    // units finished so far
@@ -1020,6 +1020,8 @@ template <int G, int FUSION>
 cudaError_t launch_gf(TcPlan *plan, const DecodeArgs &a, cudaStream_t stream)
 {
     constexpr int NG = kComputeGroups;
+    if (!a.norm_current && sched_whole(a.U, a.cap, plan->geo.grid))
+        return a.row_n ? launch_gfn<G, FUSION, NG, kTcBlocksWhole, true>(plan, a, stream) : launch_gfn<G, FUSION, NG, kTcBlocksWhole, false>(plan, a, stream);
     if (a.nblk > 1)
         return a.row_n ? launch_gfn<G, FUSION, NG, kTcBlocks, true>(plan, a, stream) : launch_gfn<G, FUSION, NG, kTcBlocks, false>(plan, a, stream);
     if (plan->geo.nc > 1) return a.row_n ? cudaErrorInvalidValue : launch_gfn<G, FUSION, NG, kTcChunks, false>(plan, a, stream);

@@ -46,3 +46,14 @@ def test_other_sm_counts(replay):
     for n_sm in (1, 2, 7, 132, 160):
         replay(40, 900, 0, n_sm)
         replay(40, 900, 3, n_sm)
+
+
+# shares cut between units: the same replay with the other kind of walk
+@pytest.mark.parametrize("U,cap", [(149, 129), (256, 1152), (300, 257), (1024, 1000), (295, 4000)])
+def test_whole_units(tmp_path, U, cap):
+    exe = str(tmp_path / "replay_whole")
+    with open(os.path.join(HERE, "schedule_replay.cpp")) as f:
+        src = f.read().replace("Walk w(", "WalkT<true> w(").replace("Walk any(", "WalkT<true> any(")
+    subprocess.run(["g++", "-O2", "-std=c++17", "-I", CSRC, "-x", "c++", "-", "-o", exe], input=src, text=True, check=True)
+    r = subprocess.run([exe, str(U), str(cap), "0", "148"], capture_output=True, text=True)
+    assert r.returncode == 0 and r.stdout.startswith("ok 148"), r.stdout + r.stderr
