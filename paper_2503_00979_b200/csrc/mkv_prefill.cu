@@ -176,17 +176,26 @@ __global__ void __launch_bounds__(kPT) prefill_fuse_kernel(const float *__restri
     Fp[(size_t)blockIdx.y * SP + j] = F;
 }
 
-// Top-C of the M = P - Rw older tokens by (F descending, position ascending): an 8-pass
-// radix select finds the C-th best 64-bit rank key, then an order-preserving compaction
-// lists the kept positions, followed by the window positions.
-constexpr int kSelT = 1024;  // threads of the selection kernel: a pass is a chain of rounds of kSelT keys
-__global__ void __launch_bounds__(kSelT) prefill_select_kernel(const float *__restrict__ Fp, int *__restrict__ pos, int ub0,
-                                                               int P, int Rw, int C, int cap, RowMap rowmap)
+// Top-C of the M = P - Rw older tokens by (F descending, position ascending): a radix select on the 64-bit rank keys finds
+// the C-th best, then an order-preserving compaction lists the kept positions, followed by the window positions.
+//
+// One CTA per unit; a warp owns a run of the keys, so that the compaction needs one scan over the warps and no barrier per
+// round.  The digits are 12 bits wide: the first takes sign, exponent and three bits of the mantissa, after which a bucket mostly holds a few hundredths of the keys; those move to a list in shared memory, on which the other digits
+// work.  The keys are read from memory once if a warp's run fits in its registers (up to 8192 keys), else three times.
+// Bound by latency for short prompts, by L2 for long ones.  With 8-bit digits, every one of them over all keys, and a
+// compaction of 1024 keys per round between barriers: 31 us for 256 units of 6112 keys and 306 us for 131040, now 17 and 101.
+constexpr int kSelT = 1024;      // threads of the selection kernel
+constexpr int kSelRun = 8;       // keys a lane holds at a time
+constexpr int kSelList = 3072;   // keys of a bucket that fit the list
+__global__ void __launch_bounds__(kSelT, 2) prefill_select_kernel(const float *__restrict__ Fp, int *__restrict__ pos, int ub0,
+                                                                  int P, int Rw, int C, int cap, RowMap rowmap)
 {
-    __shared__ unsigned int hist[256];
+    constexpr int kW = kSelT / 32, kChunk = 32 * kSelRun, kBins = 4096, kPer = kBins / kSelT;
+    __shared__ unsigned int hist[kBins];
+    __shared__ unsigned long long list[kSelList];
+    __shared__ int wtot[kW], wkeep[kW];
     __shared__ unsigned long long prefix_s;
-    __shared__ int remaining_s, done_s;
-    __shared__ int wtot[kSelT / 32];
+    __shared__ int remaining_s, count_s, n_list;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int u = ub0 + blockIdx.x;
     const float *F = Fp + (size_t)blockIdx.x * P;
@@ -198,91 +207,133 @@ __global__ void __launch_bounds__(kSelT) prefill_select_kernel(const float *__re
         for (int i = tid; i < P; i += kSelT) upos[i] = i;
         return;
     }
-    unsigned long long prefix = 0;
-    int remaining = C;
-    constexpr int kSelBatch = 4;                                         // keys per thread in flight
-    for (int pass = 7; pass >= 0; --pass) {
-        if (tid < 256) hist[tid] = 0;
+    const int run = (M + kW * kChunk - 1) / (kW * kChunk) * kChunk;      // keys of a warp
+    const int j0 = warp * run, j1 = min(M, j0 + run);
+    const bool held = run == kChunk;
+    unsigned int v[kSelRun];
+    auto load = [&](int c0) {                                            // lane l holds keys c0 + 32 i + l
+#pragma unroll
+        for (int i = 0; i < kSelRun; ++i) {
+            const int j = c0 + 32 * i + lane;
+            v[i] = j < j1 ? __float_as_uint(F[j]) : 0u;
+        }
+    };
+    if (held) load(j0);
+    if (tid == 0) n_list = 0;
+    unsigned long long prefix = 0;       // the key bits found so far, at their place
+    int remaining = C, hi = 64, shift = 52;      // the bits from `hi` up are known, the digit is hi - 1 .. shift
+    bool listed = false, exact = false;
+    while (true) {
+        // ---- histogram of the digit among the keys that share the prefix
+        for (int i = tid; i < kBins; i += kSelT) hist[i] = 0;
         __syncthreads();
-        const int shift = 8 * pass;
-        for (int c0 = 0; c0 < M; c0 += kSelT * kSelBatch) {
-            // the loads of a batch are issued together: a pass is a chain of L2 round trips otherwise
-            unsigned int fb[kSelBatch];
+        const unsigned int mask = (1u << (hi - shift)) - 1u;
+        if (listed) {
+            for (int i = tid; i < n_list; i += kSelT)
+                if ((list[i] ^ prefix) >> hi == 0) atomicAdd(&hist[(unsigned)(list[i] >> shift) & mask], 1u);
+        } else {
+            for (int c0 = j0; c0 < j1; c0 += kChunk) {
+                if (!held) load(c0);
 #pragma unroll
-            for (int i = 0; i < kSelBatch; ++i) {
-                const int j = c0 + i * kSelT + tid;
-                fb[i] = j < M ? __float_as_uint(F[j]) : 0u;
-            }
-#pragma unroll
-            for (int i = 0; i < kSelBatch; ++i) {
-                if (c0 + i * kSelT >= M) break;                          // uniform over the CTA
-                const int j = c0 + i * kSelT + tid;
-                unsigned int bin = 256u;                                 // 256: not counted in this pass
-                if (j < M) {
-                    const unsigned long long key = rank_key(fb[i], j);
-                    if (pass == 7 || (key >> (shift + 8)) == prefix) bin = (unsigned)(key >> shift) & 255u;
+                for (int i = 0; i < kSelRun; ++i) {
+                    const int j = c0 + 32 * i + lane;
+                    const unsigned long long key = rank_key(v[i], j);
+                    if (j < j1 && (hi == 64 || (key ^ prefix) >> hi == 0)) atomicAdd(&hist[(unsigned)(key >> shift) & mask], 1u);
                 }
-                // one shared-memory atomic per warp and distinct bucket: the high bytes of the keys (sign and
-                // exponent of the score) fall into a few buckets, and 32 atomics on one word would be serialised
-                const unsigned int peers = __match_any_sync(0xffffffffu, bin);
-                if (bin < 256u && lane == __ffs(peers) - 1) atomicAdd(&hist[bin], (unsigned)__popc(peers));
             }
         }
         __syncthreads();
-        // the bucket b that holds the `remaining`-th best key: above(b) < remaining <= above(b) + hist[b], with
-        // above(b) the number of keys in higher buckets.  Thread b < 256 owns bucket b; exactly one qualifies.
-        int h = 0, incl = 0;
-        if (tid < 256) {                                                 // whole warps 0..7
-            h = (int)hist[tid];
-            incl = h;                                                    // sum over this warp's buckets >= tid
+        // ---- the bucket that holds the `remaining`-th best key: above < remaining <= above + its count, with `above` the
+        // keys in higher buckets.  A thread owns kPer adjacent buckets; exactly one bucket qualifies.
+        int own = 0;
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int up = __shfl_down_sync(0xffffffffu, incl, o);
-                if (lane + o < 32) incl += up;
-            }
-            if (lane == 0) wtot[warp] = incl;
+        for (int b = 0; b < kPer; ++b) own += (int)hist[tid * kPer + b];
+        int incl = own;                                                  // sum over this warp's threads >= tid
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int up = __shfl_down_sync(0xffffffffu, incl, o);
+            if (lane + o < 32) incl += up;
         }
+        if (lane == 0) wtot[warp] = incl;
         __syncthreads();
-        if (tid < 256) {
-            int above = incl - h;
-            for (int w = warp + 1; w < 8; ++w) above += wtot[w];
-            if (h > 0 && above < remaining && remaining <= above + h) {
-                const unsigned long long np = (prefix << 8) | (unsigned long long)tid;
-                // the bucket fills the remaining places exactly: every key in it is kept, so the smallest key with
-                // this prefix is the threshold and the finer passes (mostly tie-breaking position bits) are not
-                // needed
-                const bool exact = above + h == remaining;
-                remaining_s = remaining - above;
-                prefix_s = exact ? np << shift : np;
-                done_s = exact ? 1 : 0;
+        int wsum = lane > warp ? wtot[lane] : 0;                         // (as many warps as lanes)
+        wsum = (int)__reduce_add_sync(0xffffffffu, (unsigned)wsum);
+        int above = wsum + incl - own;
+        if (above < remaining && remaining <= above + own) {
+#pragma unroll
+            for (int b = kPer - 1; b >= 0; --b) {
+                const int h = (int)hist[tid * kPer + b];
+                if (above < remaining && remaining <= above + h) {
+                    prefix_s = prefix | (unsigned long long)(tid * kPer + b) << shift;
+                    remaining_s = remaining - above;
+                    count_s = h;
+                }
+                above += h;
             }
         }
         __syncthreads();
         prefix = prefix_s;
         remaining = remaining_s;
-        const bool done = done_s != 0;
+        const int count = count_s;
         __syncthreads();
-        if (done) break;
-    }
-    // order-preserving compaction of the kept positions, kSelT keys per round
-    int base = 0;
-    for (int c0 = 0; c0 < M; c0 += kSelT) {
-        const int j = c0 + tid;
-        const bool keep = j < M && rank_key(__float_as_uint(F[j]), j) >= prefix;
-        const unsigned int bal = __ballot_sync(0xffffffffu, keep);
-        if (lane == 0) wtot[warp] = __popc(bal);
-        __syncthreads();
-        int incl = wtot[lane];                                           // every warp scans the 32 warp totals
+        // the bucket fills the remaining places exactly: all of it is kept, the finer digits are not needed
+        exact = count == remaining;
+        if (exact || shift == 0) break;
+        if (!listed && count <= kSelList) {
+            // ---- the bucket moves to the list; what lies above it is kept
+            int keep = 0;
+            for (int c0 = j0; c0 < j1; c0 += kChunk) {
+                if (!held) load(c0);
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int dn = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += dn;
+                for (int i = 0; i < kSelRun; ++i) {
+                    const int j = c0 + 32 * i + lane;
+                    const unsigned long long key = rank_key(v[i], j);
+                    const bool in = j < j1;
+                    keep += __popc(__ballot_sync(0xffffffffu, in && key >> shift > prefix >> shift));
+                    const unsigned int bal = __ballot_sync(0xffffffffu, in && key >> shift == prefix >> shift);
+                    if (bal != 0) {
+                        int at = 0;
+                        if (lane == 0) at = atomicAdd(&n_list, __popc(bal));
+                        at = __shfl_sync(0xffffffffu, at, 0);
+                        if (bal >> lane & 1) list[at + __popc(bal & ((1u << lane) - 1u))] = key;
+                    }
+                }
+            }
+            if (lane == 0) wkeep[warp] = keep;
+            listed = true;
+            __syncthreads();
         }
-        const int before = warp == 0 ? 0 : __shfl_sync(0xffffffffu, incl, warp - 1);
-        const int total = __shfl_sync(0xffffffffu, incl, 31);
-        if (keep) upos[base + before + __popc(bal & ((1u << lane) - 1u))] = j;
-        base += total;
-        __syncthreads();
+        hi = shift;
+        shift = max(0, shift - 12);
+    }
+    // every key >= prefix is kept (the bits below the last digit are zero in it): how many of each warp's
+    if (listed) {
+        for (int i = tid; i < n_list; i += kSelT)
+            if (list[i] >= prefix) atomicAdd(&wkeep[(0xFFFFFFFFu - (unsigned)list[i]) / (unsigned)run], 1);
+    } else {
+        int keep = 0;
+        for (int c0 = j0; c0 < j1; c0 += kChunk) {
+            if (!held) load(c0);
+#pragma unroll
+            for (int i = 0; i < kSelRun; ++i) {
+                const int j = c0 + 32 * i + lane;
+                keep += __popc(__ballot_sync(0xffffffffu, j < j1 && rank_key(v[i], j) >= prefix));
+            }
+        }
+        if (lane == 0) wkeep[warp] = keep;
+    }
+    __syncthreads();
+    int base = (int)__reduce_add_sync(0xffffffffu, lane < warp ? (unsigned)wkeep[lane] : 0u);
+    for (int c0 = j0; c0 < j1; c0 += kChunk) {
+        if (!held) load(c0);
+#pragma unroll
+        for (int i = 0; i < kSelRun; ++i) {
+            const int j = c0 + 32 * i + lane;
+            const bool keep = j < j1 && rank_key(v[i], j) >= prefix;
+            const unsigned int bal = __ballot_sync(0xffffffffu, keep);
+            if (keep) upos[base + __popc(bal & ((1u << lane) - 1u))] = j;
+            base += __popc(bal);
+        }
     }
     for (int i = tid; i < Rw; i += kSelT) upos[C + i] = M + i;
 }
