@@ -68,6 +68,10 @@ cudaError_t run_prefill_static(const DecodeArgs &a, bool f32, int D, const void 
 // The window sums (DecodeArgs::slab) of the slots whose token is no longer the one in sum_pos, for the step that a.st
 // holds.  *launches counts the launches.
 cudaError_t launch_window_sums(const DecodeArgs &a, bool f32, int D, unsigned long long *launches, cudaStream_t stream);
+// The gather of the kept prompt rows into the arena and the window sums in one launch (windows of up to 256 ring rows on the
+// tensor cores); a.pos and the ring are there.
+bool gather_sums_supported(const DecodeArgs &a, const void *k, const void *v);
+cudaError_t launch_gather_sums(const DecodeArgs &a, const void *k, const void *v, int P, int Ps, int n, int *err, cudaStream_t stream);
 // Last launch(es) of the prompt phase: if `sums`, the window sums of every slot, where the context keeps them, for the
 // step at position t of n cached tokens, and the n_states step states at a.st.  `err`: word in which a wait that runs out is
 // reported.

@@ -574,18 +574,23 @@ cudaError_t run_prefill_t(const DecodeArgs &a, const T *k, const T *v, const T *
         }
     }
     constexpr int CH = D * sizeof(T) / 16;
-    prefill_gather_kernel<T, D><<<dim3(U, (a.cap * CH + 255) / 256), 256, 0, stream>>>(k, v, a, P, Ps, rowmap);
     if (((uintptr_t)qwin & 15) == 0)
         prefill_ring_vec_kernel<T, D><<<dim3(U, (R * G * CH + 255) / 256), 256, 0, stream>>>(qwin, a, P, Rws, rowmap);
     else
         prefill_ring_kernel<T, D><<<U, 256, 0, stream>>>(qwin, a, P, Rws, rowmap);
+    // (the gather may take the window sums along, for which it needs the ring)
+    const bool sums_along = sums_tc && gather_sums_supported(a, k, v);
+    e = cudaSuccess;
+    if (sums_along) e = launch_gather_sums(a, k, v, P, Ps, n, err_word, stream);
+    else prefill_gather_kernel<T, D><<<dim3(U, (a.cap * CH + 255) / 256), 256, 0, stream>>>(k, v, a, P, Ps, rowmap);
+    if (e != cudaSuccess) return e;
     if (a.norm_current && select) {
         prefill_renorm_kernel<T, D><<<dim3(Rw * G, U), kPT, 0, stream>>>(a, P, rowmap);
         ++*launches;
     }
     *launches += 2;
     e = cudaGetLastError();
-    if (e == cudaSuccess) e = launch_finish_prompt(a, sums_tc, P, n, n_states, err_word, launches, stream);
+    if (e == cudaSuccess) e = launch_finish_prompt(a, sums_tc && !sums_along, P, n, n_states, err_word, launches, stream);
     const cudaError_t e2 = cudaStreamSynchronize(stream);
     if (e != cudaSuccess || e2 != cudaSuccess) return e != cudaSuccess ? e : e2;
     if (waits) {    // a bounded wait that ran out

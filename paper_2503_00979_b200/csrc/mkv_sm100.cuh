@@ -111,6 +111,13 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *map
         ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(z), "r"(bar), "l"(policy) : "memory");
 }
 
+// Shared memory to the box at (x, y, z); rows beyond the tensor are left out.  Joins the thread's current bulk group.
+__device__ __forceinline__ void tma_store_3d(const CUtensorMap *map, uint32_t src, int x, int y, int z)
+{
+    asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.tile.bulk_group [%0, {%1, %2, %3}], [%4];"
+                 ::"l"(map), "r"(x), "r"(y), "r"(z), "r"(src) : "memory");
+}
+
 // Asks for the box at (x, y, z) to be brought into L2; no data reaches the SM and no barrier is involved.  The same
 // coordinate rules as for the load: x * element size a multiple of 16 bytes, out-of-range parts are skipped.
 __device__ __forceinline__ void tma_prefetch_l2_3d(const CUtensorMap *map, int x, int y, int z)
@@ -226,12 +233,13 @@ __device__ __forceinline__ void split_bf16x2(float x, float y, uint32_t &hi, uin
 }
 
 // group barrier that also ORs a predicate over the group (uniform bail-out decisions)
+template <int N = kGroupThreads>
 __device__ __forceinline__ bool group_any(int bar_id, bool pred)
 {
     uint32_t r;
     asm volatile(
         "{\n.reg .pred p, q;\nsetp.ne.b32 p, %1, 0;\nbarrier.red.or.pred q, %2, %3, p;\nselp.u32 %0, 1, 0, q;\n}"
-        : "=r"(r) : "r"((uint32_t)pred), "r"(bar_id), "r"(kGroupThreads) : "memory");
+        : "=r"(r) : "r"((uint32_t)pred), "r"(bar_id), "r"(N) : "memory");
     return r != 0;
 }
 
