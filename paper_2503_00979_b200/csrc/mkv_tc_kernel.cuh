@@ -127,10 +127,25 @@ struct RingPos {
 // evict the minimum, append (Eq. 1 merge, Eq. 4-7).  All loads of a phase are issued together, so
 // the whole epilogue costs a few L2 round trips.  Requires nseg <= 8 and nseg*G*2 <= 256.
 // LOCAL: the single partial is this CTA's own: l_o[g] is the thread's column of the merged output,
-// l_ml [G][2] sits in shared memory.
+// l_ml [G][2] sits in shared memory.  `x`: the new token's rows, which the group loads while the unit's tiles still stream
+// (read here they added a round trip to the end of the step, and over the interconnect where they lie in host memory).
+template <int G> struct NewRows {
+    static constexpr int chunks = (G * 16 + kGroupThreads - 1) / kGroupThreads;    // 16-byte chunks of q per thread
+    uint4 q[chunks], k, v;       // chunks tid + 128 i of the queries, chunk tid % 16 of the key and the value
+    __device__ __forceinline__ void load(const DecodeArgs &a, int u, int tid)
+    {
+        const uint4 *qs = reinterpret_cast<const uint4 *>(static_cast<const __nv_bfloat16 *>(a.q) + (size_t)u * a.Gq * kD);
+#pragma unroll
+        for (int i = 0; i < chunks; ++i)
+            q[i] = tid + i * kGroupThreads < a.Gq * 16 ? qs[tid + i * kGroupThreads] : make_uint4(0, 0, 0, 0);
+        k = reinterpret_cast<const uint4 *>(static_cast<const __nv_bfloat16 *>(a.k_new) + (size_t)u * kD)[tid & 15];
+        v = reinterpret_cast<const uint4 *>(static_cast<const __nv_bfloat16 *>(a.v_new) + (size_t)u * kD)[tid & 15];
+    }
+};
+
 template <int G, bool LOCAL>
 __device__ void finalize_fast(const DecodeArgs &a, int u, long long t, int n, int nseg, bool evict, float *sm, int tid,
-                              int bar_id, const float (&l_o)[G], const float *l_ml, int shift)
+                              int bar_id, const float (&l_o)[G], const float *l_ml, int shift, const NewRows<G> &x)
 {
     constexpr int NT_ = kGroupThreads;
     const int lane = tid & 31, warp = tid >> 5;
@@ -141,25 +156,11 @@ __device__ void finalize_fast(const DecodeArgs &a, int u, long long t, int n, in
     int *red_slot = reinterpret_cast<int *>(pml_s + 256 + 64);                           // [32]
 
     const int Gq = a.Gq;      // heads Gq .. G-1 are padding: zero query, normaliser +inf, no output
-    const __nv_bfloat16 *q = static_cast<const __nv_bfloat16 *>(a.q) + (size_t)u * Gq * kD;
-    const __nv_bfloat16 *kn = static_cast<const __nv_bfloat16 *>(a.k_new) + (size_t)u * kD;
-    const __nv_bfloat16 *vn = static_cast<const __nv_bfloat16 *>(a.v_new) + (size_t)u * kD;
     const float *pml = a.part_ml + (size_t)u * a.splits * G * 2;
     const float *po = a.part_o + (size_t)u * a.splits * G * kD;
 
     // ---- phase A: every load that does not depend on another one
-    constexpr int QCH = (G * 16 + NT_ - 1) / NT_;          // 16-byte chunks of q per thread
-    uint4 qv[QCH], kv[QCH];
-#pragma unroll
-    for (int i = 0; i < QCH; ++i) {
-        const int c = tid + i * NT_;
-        if (c < G * 16) {
-            qv[i] = c < Gq * 16 ? reinterpret_cast<const uint4 *>(q)[c] : make_uint4(0, 0, 0, 0);
-            kv[i] = reinterpret_cast<const uint4 *>(kn)[c & 15];
-        }
-    }
-    uint4 vv = make_uint4(0, 0, 0, 0);
-    if (tid < 16) vv = reinterpret_cast<const uint4 *>(vn)[tid];
+    constexpr int QCH = NewRows<G>::chunks;
     for (int i = tid; i < nseg * G * 2; i += NT_) pml_s[i] = LOCAL ? l_ml[i] : __ldcg(pml + i);
     float pov[G][8];
 #pragma unroll
@@ -174,7 +175,7 @@ __device__ void finalize_fast(const DecodeArgs &a, int u, long long t, int n, in
         const int c = tid + i * NT_;
         float acc = 0.f;
         if (c < G * 16) {
-            const uint32_t *qa = reinterpret_cast<const uint32_t *>(&qv[i]), *ka = reinterpret_cast<const uint32_t *>(&kv[i]);
+            const uint32_t *qa = reinterpret_cast<const uint32_t *>(&x.q[i]), *ka = reinterpret_cast<const uint32_t *>(&x.k);
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 acc += __uint_as_float(qa[e] << 16) * __uint_as_float(ka[e] << 16);
@@ -186,7 +187,7 @@ __device__ void finalize_fast(const DecodeArgs &a, int u, long long t, int n, in
         if (c < G * 16 && (c & 15) == 0) s_self[c >> 4] = acc * a.scale2;
     }
     if (tid < 16) {
-        const uint32_t *va = reinterpret_cast<const uint32_t *>(&vv);
+        const uint32_t *va = reinterpret_cast<const uint32_t *>(&x.v);
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
             vsm[tid * 8 + 2 * e] = __uint_as_float(va[e] << 16);
@@ -236,14 +237,14 @@ __device__ void finalize_fast(const DecodeArgs &a, int u, long long t, int n, in
         constexpr int B = 8;          // slots per thread and round, all their loads in flight together
         for (int kb = tid; kb < n; kb += B * NT_) {
             int p[B];
-            float f0[B], x[G][B];
+            float f0[B], xs[G][B];
 #pragma unroll
             for (int b = 0; b < B; ++b) {
                 const int k = kb + b * NT_;
                 p[b] = k < n ? pos[k] : 0x7fffffff;
                 f0[b] = k < n ? __ldcg(F + k) : 0.f;
 #pragma unroll
-                for (int g = 0; g < G; ++g) x[g][b] = k < n ? __ldcg(sn + (size_t)g * a.cap + k) : -INFINITY;
+                for (int g = 0; g < G; ++g) xs[g][b] = k < n ? __ldcg(sn + (size_t)g * a.cap + k) : -INFINITY;
             }
 #pragma unroll
             for (int b = 0; b < B; ++b) {
@@ -252,7 +253,7 @@ __device__ void finalize_fast(const DecodeArgs &a, int u, long long t, int n, in
                 if ((long long)p[b] <= thr) {
                     float s = 0.f;
 #pragma unroll
-                    for (int g = 0; g < G; ++g) s += exp2f(x[g][b] - cn[g]);
+                    for (int g = 0; g < G; ++g) s += exp2f(xs[g][b] - cn[g]);
                     const float f = fuse(a.fusion, f0[b], s);
                     F[k] = f;
                     const unsigned long long key = rank_key(__float_as_uint(f), p[b]);
@@ -296,15 +297,15 @@ __device__ void finalize_fast(const DecodeArgs &a, int u, long long t, int n, in
     __nv_bfloat16 *Kd = static_cast<__nv_bfloat16 *>(a.K) + ((size_t)u * a.cap + e_slot) * kD;
     __nv_bfloat16 *Vd = static_cast<__nv_bfloat16 *>(a.V) + ((size_t)u * a.cap + e_slot) * kD;
     if (tid < 16) {
-        reinterpret_cast<uint4 *>(Kd)[tid] = kv[0];
-        reinterpret_cast<uint4 *>(Vd)[tid] = vv;
+        reinterpret_cast<uint4 *>(Kd)[tid] = x.k;
+        reinterpret_cast<uint4 *>(Vd)[tid] = x.v;
     }
     const int rs = (int)(t % a.R);
     __nv_bfloat16 *rq = static_cast<__nv_bfloat16 *>(a.ring_q) + ((size_t)u * a.R + rs) * G * kD;
 #pragma unroll
     for (int i = 0; i < QCH; ++i) {
         const int c = tid + i * NT_;
-        if (c < G * 16) reinterpret_cast<uint4 *>(rq)[c] = qv[i];
+        if (c < G * 16) reinterpret_cast<uint4 *>(rq)[c] = x.q[i];
     }
     if (tid < G) a.ring_c[((size_t)u * a.R + rs) * G + tid] = cnew[tid];
     if (tid == 0) {
@@ -880,6 +881,8 @@ decode_tc_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ C
                 const int u = MC ? x.unit / NCe : x.unit;
                 const bool main_item = MC ? (NCe == 1 || x.unit - u * NCe == c_main) : true;
                 const UnitStep us = RAGGED ? unit_step(a, u, t, n, steps_done, evict) : UnitStep{n, 0, evict};
+                NewRows<G> rows;
+                if constexpr (!MC) rows.load(a, u, etid);
                 if (group_any(kEpiBar, !mbar_wait(bar_udone, (uint32_t)(k & 1), abort_flag, kWaitUDone, WL))) { ok = false; break; }
                 // merge the compute warps' partials: common reference = max of theirs
                 if (etid < G && main_item) {
@@ -946,7 +949,7 @@ decode_tc_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ C
                                                                   kEpiBar, RAGGED ? us.shift : 0);
                     }
                 } else if (ncta == 1) {
-                    finalize_fast<G, true>(a, u, t, us.n, 1, us.evict, fin_sm, etid, kEpiBar, o, cml, RAGGED ? us.shift : 0);
+                    finalize_fast<G, true>(a, u, t, us.n, 1, us.evict, fin_sm, etid, kEpiBar, o, cml, RAGGED ? us.shift : 0, rows);
                 } else {
                     // the unit is shared: publish this CTA's partial; the last CTA to do so finishes the unit.
                     // The group barrier orders every thread's writes (and, through the mbarrier above, the compute
@@ -968,7 +971,7 @@ decode_tc_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ C
                     group_sync(kEpiBar, kGroupThreads);
                     if (*flag) {
                         if (ncta <= 8 && ncta * G * 2 <= 256)
-                            finalize_fast<G, false>(a, u, t, us.n, ncta, us.evict, fin_sm, etid, kEpiBar, o, nullptr, RAGGED ? us.shift : 0);
+                            finalize_fast<G, false>(a, u, t, us.n, ncta, us.evict, fin_sm, etid, kEpiBar, o, nullptr, RAGGED ? us.shift : 0, rows);
                         else
                             finalize_unit<__nv_bfloat16, kD, G>(a, u, t, us.n, ncta, us.evict, fin_sm, etid, kGroupThreads, kEpiBar,
                                                                 RAGGED ? us.shift : 0);
