@@ -387,6 +387,7 @@ void core_destroy(mkv_ctx *ctx)
     if (ctx->plan) tc_plan_destroy(ctx->plan);
     if (ctx->plan_layer) tc_plan_destroy(ctx->plan_layer);
     if (ctx->prefill_scratch.ptr) cudaFree(ctx->prefill_scratch.ptr);
+    if (ctx->prefill_scratch.host_err) cudaFreeHost(ctx->prefill_scratch.host_err);
     if (ctx->owns_workspace && ctx->base) cudaFree(ctx->base);
     delete[] ctx->row_n;
     delete[] ctx->viewed;

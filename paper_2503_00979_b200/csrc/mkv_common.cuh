@@ -127,6 +127,31 @@ __host__ __device__ __forceinline__ unsigned long long rank_key(unsigned int F_b
     return ((unsigned long long)F_bits << 32) | (unsigned long long)(0xFFFFFFFFu - (unsigned)pos);
 }
 
+// Programmatic stream serialisation, by the protocol that every kernel launched with launch_chained follows: it may start
+// while the kernel before it in the stream still runs, waits for that kernel's end before it touches anything another kernel
+// writes or reads, and only then lets the next one start.  So the kernel before the one before it is complete when it starts.
+__device__ __forceinline__ void chain_wait()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <typename... Params, typename... Args>
+inline cudaError_t launch_chained(void (*kern)(Params...), dim3 grid, unsigned block, size_t smem, cudaStream_t stream, Args &&...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...);
+}
+
 // How a unit's n cached tokens are divided among `splits` CTAs: contiguous ranges whose
 // length is a multiple of `tile`.  Returns the per-split length; *active = splits with work.
 __host__ __device__ inline int split_len(int n, int splits, int tile, int *active)

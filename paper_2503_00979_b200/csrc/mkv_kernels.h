@@ -43,6 +43,7 @@ cudaError_t launch_decode_tc(TcPlan *plan, const DecodeArgs &a, cudaStream_t str
 struct PrefillScratch {
     void *ptr;
     size_t bytes;
+    int *host_err;       // pinned word (nullptr: none could be had)
 };
 // With prompts of different lengths in the batch (a.row_shift) P is the longest prompt's length; the tensors are padded
 // to padded_len tokens (P otherwise).

@@ -31,9 +31,12 @@ __device__ __forceinline__ void ld4(const __nv_bfloat16 *p, float (&o)[4])
     o[2] = __uint_as_float(v.y << 16); o[3] = __uint_as_float(v.y & 0xffff0000u);
 }
 
-__global__ void init_arena_kernel(DecodeArgs a)
+// (launched in full stream order: what it waits for is complete for the kernels behind it too)
+__global__ void init_arena_kernel(DecodeArgs a, int *err)
 {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0) *err = 0;
     const size_t ncap = (size_t)a.U * a.cap;
     if (i < ncap) { a.pos[i] = -1; a.F[i] = 0.f; }
     if (i < ncap && a.nblk > 1) a.sum_pos[i] = -1;
@@ -196,6 +199,7 @@ __global__ void __launch_bounds__(kSelT, 2) prefill_select_kernel(const float *_
     __shared__ int wtot[kW], wkeep[kW];
     __shared__ unsigned long long prefix_s;
     __shared__ int remaining_s, count_s, n_list;
+    chain_wait();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int u = ub0 + blockIdx.x;
     const float *F = Fp + (size_t)blockIdx.x * P;
@@ -373,6 +377,7 @@ __global__ void __launch_bounds__(kPT) prefill_sums_kernel(const float *__restri
 
 __global__ void prefill_identity_pos_kernel(int *pos, int U, int n, int cap, RowMap rowmap)
 {
+    chain_wait();
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (size_t)U * n) return;
     if ((int)(i % n) < n - rowmap((int)(i / n))) pos[(i / n) * cap + (i % n)] = (int)(i % n);
@@ -410,6 +415,7 @@ __global__ void prefill_gather_kernel(const T *__restrict__ k, const T *__restri
 template <typename T, int D>
 __global__ void prefill_ring_kernel(const T *__restrict__ qwin, DecodeArgs a, int P, int Rws, RowMap rowmap)
 {
+    chain_wait();
     const int u = blockIdx.x, G = a.G, Gq = a.Gq, shift = rowmap(u);
     P -= shift;
     const int Rw = min(P, a.R);                         // heads Gq .. G-1 of a ring slot are padding (zero query)
@@ -426,6 +432,7 @@ __global__ void prefill_ring_kernel(const T *__restrict__ qwin, DecodeArgs a, in
 template <typename T, int D>
 __global__ void prefill_ring_vec_kernel(const T *__restrict__ qwin, DecodeArgs a, int P, int Rws, RowMap rowmap)
 {
+    chain_wait();
     constexpr int CH = D * sizeof(T) / 16;
     const int u = blockIdx.x, G = a.G, Gq = a.Gq, shift = rowmap(u);
     const int idx = blockIdx.y * blockDim.x + threadIdx.x;
@@ -504,7 +511,7 @@ __global__ void __launch_bounds__(kPT) prefill_renorm_kernel(DecodeArgs a, int P
 
 template <typename T, int D>
 cudaError_t run_prefill_t(const DecodeArgs &a, const T *k, const T *v, const T *qwin, int P, cudaStream_t stream,
-                          unsigned long long *launches, float *S, size_t scratch_floats, int n_states, int padded_len)
+                          unsigned long long *launches, float *S, size_t scratch_floats, int *host_err, int n_states, int padded_len)
 {
     // With prompts of different lengths (a.row_shift) P is the longest one and the tensors are padded to padded_len
     // tokens; the ring slots follow the common time axis, on which every row ends at P.
@@ -535,15 +542,19 @@ cudaError_t run_prefill_t(const DecodeArgs &a, const T *k, const T *v, const T *
     cudaError_t e = cudaFuncSetAttribute(prefill_logits_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)logits_smem);
     if (e != cudaSuccess) return e;
     const size_t init_n = max((size_t)U * a.cap, (size_t)U * R * G);
-    init_arena_kernel<<<(unsigned)((init_n + 255) / 256), 256, 0, stream>>>(a);
-    ++*launches;
+    init_arena_kernel<<<(unsigned)((init_n + 255) / 256), 256, 0, stream>>>(a, err_word);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
     const bool waits = tc || a.nblk > 1;            // kernels with bounded waits are launched
-    if (waits) {
-        e = cudaMemsetAsync(err_word, 0, sizeof(int), stream);
-        if (e != cudaSuccess) return e;
-    }
+    constexpr int CH = D * sizeof(T) / 16;
+    e = ((uintptr_t)qwin & 15) == 0
+        ? launch_chained(prefill_ring_vec_kernel<T, D>, dim3(U, (R * G * CH + 255) / 256), 256, 0, stream, qwin, a, P, Rws, rowmap)
+        : launch_chained(prefill_ring_kernel<T, D>, dim3(U), 256, 0, stream, qwin, a, P, Rws, rowmap);
+    if (e != cudaSuccess) return e;
+    *launches += 2;
     if (!select) {
-        prefill_identity_pos_kernel<<<(unsigned)(((size_t)U * n + 255) / 256), 256, 0, stream>>>(a.pos, U, n, a.cap, rowmap);
+        e = launch_chained(prefill_identity_pos_kernel, dim3((unsigned)(((size_t)U * n + 255) / 256)), 256, 0, stream, a.pos, U, n, a.cap, rowmap);
+        if (e != cudaSuccess) return e;
         ++*launches;
     }
     // the window sums: on the tensor cores at the end, or from the logits S where there are any
@@ -565,7 +576,8 @@ cudaError_t run_prefill_t(const DecodeArgs &a, const T *k, const T *v, const T *
                     S, a.ring_c, Fp, ub0, P, Rw, a.Gq, G, R, a.fusion, rowmap);
                 ++*launches;
             }
-            prefill_select_kernel<<<nb, kSelT, 0, stream>>>(Fp, a.pos, ub0, P, Rw, C, a.cap, rowmap);
+            e = launch_chained(prefill_select_kernel, dim3(nb), kSelT, 0, stream, Fp, a.pos, ub0, P, Rw, C, a.cap, rowmap);
+            if (e != cudaSuccess) return e;
             ++*launches;
         }
         if (a.nblk > 1 && !sums_tc) {
@@ -573,11 +585,6 @@ cudaError_t run_prefill_t(const DecodeArgs &a, const T *k, const T *v, const T *
             ++*launches;
         }
     }
-    constexpr int CH = D * sizeof(T) / 16;
-    if (((uintptr_t)qwin & 15) == 0)
-        prefill_ring_vec_kernel<T, D><<<dim3(U, (R * G * CH + 255) / 256), 256, 0, stream>>>(qwin, a, P, Rws, rowmap);
-    else
-        prefill_ring_kernel<T, D><<<U, 256, 0, stream>>>(qwin, a, P, Rws, rowmap);
     // (the gather may take the window sums along, for which it needs the ring)
     const bool sums_along = sums_tc && gather_sums_supported(a, k, v);
     e = cudaSuccess;
@@ -588,14 +595,17 @@ cudaError_t run_prefill_t(const DecodeArgs &a, const T *k, const T *v, const T *
         prefill_renorm_kernel<T, D><<<dim3(Rw * G, U), kPT, 0, stream>>>(a, P, rowmap);
         ++*launches;
     }
-    *launches += 2;
+    ++*launches;
     e = cudaGetLastError();
     if (e == cudaSuccess) e = launch_finish_prompt(a, sums_tc && !sums_along, P, n, n_states, err_word, launches, stream);
+    // a bounded wait that ran out: the word comes back with the stream's end if there is pinned memory for it
+    int werr = 0;
+    if (waits && host_err != nullptr && e == cudaSuccess) e = cudaMemcpyAsync(host_err, err_word, sizeof(int), cudaMemcpyDeviceToHost, stream);
     const cudaError_t e2 = cudaStreamSynchronize(stream);
     if (e != cudaSuccess || e2 != cudaSuccess) return e != cudaSuccess ? e : e2;
-    if (waits) {    // a bounded wait that ran out
-        int werr = 0;
-        e = cudaMemcpy(&werr, err_word, sizeof(int), cudaMemcpyDeviceToHost);
+    if (waits) {
+        if (host_err != nullptr) werr = *host_err;
+        else e = cudaMemcpy(&werr, err_word, sizeof(int), cudaMemcpyDeviceToHost);
         if (e != cudaSuccess) return e;
         if (werr != 0) return cudaErrorLaunchTimeout;
     }
@@ -603,18 +613,18 @@ cudaError_t run_prefill_t(const DecodeArgs &a, const T *k, const T *v, const T *
 }
 
 cudaError_t dispatch_prefill(const DecodeArgs &a, bool f32, int D, const void *k, const void *v, const void *q_window, int P,
-                             cudaStream_t stream, unsigned long long *launches, float *S, size_t scratch_floats, int n_states,
+                             cudaStream_t stream, unsigned long long *launches, float *S, size_t scratch_floats, int *host_err, int n_states,
                              int padded_len)
 {
     if (f32) {
         auto kk = static_cast<const float *>(k), vv = static_cast<const float *>(v), qq = static_cast<const float *>(q_window);
-        return D == 64 ? run_prefill_t<float, 64>(a, kk, vv, qq, P, stream, launches, S, scratch_floats, n_states, padded_len)
-                       : run_prefill_t<float, 128>(a, kk, vv, qq, P, stream, launches, S, scratch_floats, n_states, padded_len);
+        return D == 64 ? run_prefill_t<float, 64>(a, kk, vv, qq, P, stream, launches, S, scratch_floats, host_err, n_states, padded_len)
+                       : run_prefill_t<float, 128>(a, kk, vv, qq, P, stream, launches, S, scratch_floats, host_err, n_states, padded_len);
     }
     auto kk = static_cast<const __nv_bfloat16 *>(k), vv = static_cast<const __nv_bfloat16 *>(v),
          qq = static_cast<const __nv_bfloat16 *>(q_window);
-    return D == 64 ? run_prefill_t<__nv_bfloat16, 64>(a, kk, vv, qq, P, stream, launches, S, scratch_floats, n_states, padded_len)
-                   : run_prefill_t<__nv_bfloat16, 128>(a, kk, vv, qq, P, stream, launches, S, scratch_floats, n_states, padded_len);
+    return D == 64 ? run_prefill_t<__nv_bfloat16, 64>(a, kk, vv, qq, P, stream, launches, S, scratch_floats, host_err, n_states, padded_len)
+                   : run_prefill_t<__nv_bfloat16, 128>(a, kk, vv, qq, P, stream, launches, S, scratch_floats, host_err, n_states, padded_len);
 }
 
 // ---- scratch of mkv_prefill_static -------------------------------------------------------------------------
@@ -673,8 +683,12 @@ cudaError_t run_prefill(const DecodeArgs &a, bool f32, int D, const void *k, con
         if (e != cudaSuccess) { scratch->ptr = nullptr; return e; }
         scratch->bytes = need;
     }
+    if (!scratch->host_err && cudaMallocHost(reinterpret_cast<void **>(&scratch->host_err), sizeof(int)) != cudaSuccess) {
+        cudaGetLastError();
+        scratch->host_err = nullptr;
+    }
     return dispatch_prefill(a, f32, D, k, v, q_window, P, stream, launches, static_cast<float *>(scratch->ptr),
-                            scratch->bytes / sizeof(float), n_states, padded_len);
+                            scratch->bytes / sizeof(float), scratch->host_err, n_states, padded_len);
 }
 
 namespace {
@@ -705,7 +719,7 @@ cudaError_t run_prefill_static(const DecodeArgs &a, bool f32, int D, const void 
     float *S = nullptr;
     const cudaError_t e = static_scratch_address(device, &S);
     if (e != cudaSuccess) return e;
-    return dispatch_prefill(a, f32, D, k, v, q_window, P, stream, launches, S, kStaticScratchFloats, n_states, P);
+    return dispatch_prefill(a, f32, D, k, v, q_window, P, stream, launches, S, kStaticScratchFloats, nullptr, n_states, P);
 }
 
 }  // namespace mkv

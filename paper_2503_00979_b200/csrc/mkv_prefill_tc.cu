@@ -110,6 +110,7 @@ prefill_tc_kernel(const __grid_constant__ PfArgs a, const __grid_constant__ CUte
         const uint32_t off = (uint32_t)((ch >> 3) * (QR * 128) + row * 128 + (((ch & 7) ^ (row & 7)) << 4));
         *reinterpret_cast<uint4 *>(smem + off) = v;
     }
+    chain_wait();           // (the prompt is complete: the chain of launches starts behind it in full stream order)
     if (PASS == 2) {
         // merge the pass-1 partials of this unit's key splits into each row's normaliser c = max + log2(sum)
         for (int row = tid; row < 256; row += kPfThreads) {
@@ -327,8 +328,7 @@ cudaError_t launch_pass(const PfArgs &a, const CUtensorMap &tm, int nb, int fusi
     const int cols = 2 * (PASS == 1 ? a.qrows : a.rpad);
     b.tmem_cols = 32;
     while (b.tmem_cols < cols) b.tmem_cols *= 2;
-    kern<<<dim3(a.splits, nb), kPfThreads, smem, stream>>>(b, tm);
-    return cudaGetLastError();
+    return launch_chained(kern, dim3(a.splits, nb), kPfThreads, smem, stream, b, tm);
 }
 
 template <int PASS>

@@ -70,6 +70,7 @@ window_sums_tc_kernel(const __grid_constant__ SumArgs a, const __grid_constant__
 
     const int n = a.n, nt = (n + kTile - 1) / kTile, per = (nt + a.splits - 1) / a.splits;
     const int t0 = sp * per, t1 = min(nt, t0 + per), ntile = max(0, t1 - t0);
+    chain_wait();
     if (sp == 0 && u == 0) set_states(a);
     const int blk_rows = d.bs * G, RG = d.R * G, open = open_block(a.t, d.R, d.bs);
     const int npiece = (a.rows + PR - 1) / PR;
@@ -263,6 +264,7 @@ gather_sums_tc_kernel(const __grid_constant__ GatherArgs ga, const __grid_consta
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    chain_wait();
 
     if (warp >= 10) {
         // ------------------------------------------------ fetch: a warp takes 32 rows of a tile, half a warp a row
@@ -444,8 +446,7 @@ cudaError_t launch_gather_g(const GatherArgs &a, const CUtensorMap &tmK, const C
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     const long long tiles = (long long)s.d.U * ((s.d.cap + kTile - 1) / kTile);
-    kern<<<(unsigned)(tiles < 148 ? tiles : 148), kGsThreads, smem, stream>>>(a, tmK, tmV);
-    return cudaGetLastError();
+    return launch_chained(kern, dim3((unsigned)(tiles < 148 ? tiles : 148)), kGsThreads, smem, stream, a, tmK, tmV);
 }
 
 // What is timed is the comparison, 8 bytes per slot in 16-byte loads; a slot that was moved is redone by one thread.
@@ -486,7 +487,11 @@ __global__ void __launch_bounds__(kSumKeys) window_sums_kernel(const __grid_cons
     }
 }
 
-__global__ void set_states_kernel(const __grid_constant__ SumArgs a) { set_states(a); }
+__global__ void set_states_kernel(const __grid_constant__ SumArgs a)
+{
+    chain_wait();
+    set_states(a);
+}
 
 template <int G>
 cudaError_t launch_sums_g(const SumArgs &a, const CUtensorMap &tm, cudaStream_t stream)
@@ -495,8 +500,7 @@ cudaError_t launch_sums_g(const SumArgs &a, const CUtensorMap &tm, cudaStream_t 
     const int smem = a.piece * 256 + a.stages * kStageBytes + kSumMaxRows * 4 + 256 + 1024;
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    kern<<<dim3(a.splits, a.d.U), kSumThreads, smem, stream>>>(a, tm);
-    return cudaGetLastError();
+    return launch_chained(kern, dim3(a.splits, a.d.U), kSumThreads, smem, stream, a, tm);
 }
 
 // `d` for a launch over its units u0 .. u0 + count - 1 (grid.y takes 65535 units at most)
@@ -571,9 +575,8 @@ cudaError_t launch_finish_prompt(const DecodeArgs &d, bool sums, long long t, in
     a.wait_cycles = kWaitCycles;
     if (d.nblk <= 1 || !sums) {
         a.set_states = n_states;
-        set_states_kernel<<<1, 32, 0, stream>>>(a);
         ++*launches;
-        return cudaGetLastError();
+        return launch_chained(set_states_kernel, dim3(1), 32, 0, stream, a);
     }
     const int blk_rows = d.bs * d.G, all = d.nblk * blk_rows;
     a.piece = min(all, 256 / blk_rows * blk_rows);
