@@ -229,10 +229,13 @@ __device__ __forceinline__ void group_sync(int bar_id, int nthr)
 
 // The block of the ring that is open before the step at position t, and whether that step opens the next one (it then
 // scores block `open` for good: see DecodeArgs::slab).
-__host__ __device__ inline int open_block(long long t, int R, int bs) { return (int)((t - 1) % R) / bs; }
+// (Positions fit in 32 bits and start at 1, a prompt's length; 64-bit divisions would take most of a microsecond at the start
+// of every launch.)
+__host__ __device__ inline int ring_slot(long long t, int R) { return (int)((unsigned)t % (unsigned)R); }
+__host__ __device__ inline int open_block(long long t, int R, int bs) { return ring_slot(t - 1, R) / bs; }
 __host__ __device__ inline bool step_opens_block(long long t, int R, int bs, int nblk)
 {
-    return nblk > 1 && (int)(t % R) % bs == 0;
+    return nblk > 1 && ring_slot(t, R) % bs == 0;
 }
 
 // The fused score S of ring block j joins the sums of one key; blocks come in descending order, acc and pre run along.
@@ -447,7 +450,7 @@ __device__ void finalize_unit(const DecodeArgs &a, int u, long long t, int n, in
             e_pos = -1;
             if (tid == 0 && n < a.cap) F[n] = -1.f;
         } else if (a.norm_current) {
-            renormalise_after_eviction<T, D>(a, u, e_slot, (int)(t % a.R), cnew, sm + 4 * kMaxGroup + 3 * 32, tid, nthr, bar_id);
+            renormalise_after_eviction<T, D>(a, u, e_slot, ring_slot(t, a.R), cnew, sm + 4 * kMaxGroup + 3 * 32, tid, nthr, bar_id);
         }
     }
 
@@ -460,7 +463,7 @@ __device__ void finalize_unit(const DecodeArgs &a, int u, long long t, int n, in
     T *Kd = static_cast<T *>(a.K) + ((size_t)u * a.cap + e_slot) * D;
     T *Vd = static_cast<T *>(a.V) + ((size_t)u * a.cap + e_slot) * D;
     for (int i = tid; i < D; i += nthr) { Kd[i] = kn[i]; Vd[i] = vn[i]; }
-    const int rs = (int)(t % a.R);
+    const int rs = ring_slot(t, a.R);
     T *rq = static_cast<T *>(a.ring_q) + ((size_t)u * a.R + rs) * G * D;
     for (int i = tid; i < G * D; i += nthr) stf(rq + i, i < Gq * D ? ldf(q + i) : 0.f);
     if (tid < G) a.ring_c[((size_t)u * a.R + rs) * G + tid] = cnew[tid];

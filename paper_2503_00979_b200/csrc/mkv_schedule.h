@@ -63,6 +63,9 @@ struct WalkT {
             if (WHOLE) {
                 tile = (int)((unsigned)U * cta / eff) * nt;           // (at most 2^24 units)
                 tile_end = (int)((unsigned)U * (cta + 1) / eff) * nt;
+            } else if (narrow()) {
+                tile = (int)((unsigned)total * cta / eff);
+                tile_end = (int)((unsigned)total * (cta + 1) / eff);
             } else {
                 tile = (int)(total * cta / eff);
                 tile_end = (int)(total * (cta + 1) / eff);
@@ -112,8 +115,11 @@ struct WalkT {
     MKV_HD int owner(long long i) const
     {
         if (WHOLE) i = i / nt * nt + nt - 1;            // the unit's last tile: (u + 1) * nt * E / T = (u + 1) * E / U
+        if (narrow()) return (int)((((unsigned)i + 1) * eff - 1) / (unsigned)total);
         return (int)(((i + 1) * eff - 1) / total);
     }
+    // products of a tile and a CTA index fit in 32 bits (64-bit divisions are slow, and stand at the start of every launch)
+    MKV_HD bool narrow() const { return total < (1ll << 24) && eff < 256; }
     // How many CTAs hold tiles of unit u, and this CTA's index among them.
     MKV_HD int ctas_of_unit(int u, int &my_index) const
     {

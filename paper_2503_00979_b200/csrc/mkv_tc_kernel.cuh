@@ -285,7 +285,7 @@ __device__ void finalize_fast(const DecodeArgs &a, int u, long long t, int n, in
             if (tid == 0 && n < a.cap) F[n] = -1.f;
         } else if (a.norm_current) {
             // vsm (the new value row as floats) was last read for the attention output: free to hold the evicted key
-            renormalise_after_eviction<__nv_bfloat16, kD>(a, u, e_slot, (int)(t % a.R), cnew, vsm, tid, NT_, bar_id);
+            renormalise_after_eviction<__nv_bfloat16, kD>(a, u, e_slot, ring_slot(t, a.R), cnew, vsm, tid, NT_, bar_id);
         }
     }
 
@@ -300,7 +300,7 @@ __device__ void finalize_fast(const DecodeArgs &a, int u, long long t, int n, in
         reinterpret_cast<uint4 *>(Kd)[tid] = x.k;
         reinterpret_cast<uint4 *>(Vd)[tid] = x.v;
     }
-    const int rs = (int)(t % a.R);
+    const int rs = ring_slot(t, a.R);
     __nv_bfloat16 *rq = static_cast<__nv_bfloat16 *>(a.ring_q) + ((size_t)u * a.R + rs) * G * kD;
 #pragma unroll
     for (int i = 0; i < QCH; ++i) {
@@ -399,7 +399,7 @@ decode_tc_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ C
     __syncthreads();
 
     const bool evict = step_scores(t, n, steps_done, a.R, a.C, a.T);
-    const int rs_new = (int)(t % a.R);
+    const int rs_new = ring_slot(t, a.R);
     // MC (a window of more than 256 ring rows): the ring is cut into geo.nc chunks of RGP rows = RGP / G ring
     // slots, and the schedule walks U * nc "virtual units": virtual unit v is chunk v % nc of unit v / nc.  The
     // chunk that holds the slot of the new query (the main chunk) does everything a unit does otherwise; the
@@ -410,14 +410,16 @@ decode_tc_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ C
     const int NCe = MC ? (evict ? geo.nc : 1) : 1;               // chunks walked per unit on this step
     const int c_main = MC || BLOCKS ? rs_new / a.bs : 0;
     const int rs_loc = MC || BLOCKS ? rs_new - c_main * a.bs : rs_new;   // the new query's slot inside its chunk or block
-    const bool fold = BLOCKS && step_opens_block(t, a.R, a.bs, a.nblk);
-    const int j_old = BLOCKS ? open_block(t, a.R, a.bs) : 0;     // fold: the finished block
+    const bool fold = BLOCKS && a.nblk > 1 && rs_loc == 0;       // step_opens_block()
+    const int j_old = c_main > 0 ? c_main - 1 : a.nblk - 1;      // fold: the finished block, open_block()
     const int QB = BLOCKS ? geo.qbox : RGP;                      // ring rows per operand box
     const int NR = fold ? 2 * QB : QB;                           // ring rows of this step's operand (MMA N)
     // Every thread of this CTA holds its copy of the step state (the barrier above orders their reads
     // before this point), so the CTA can be counted now: the last CTA of the launch to get here advances
-    // the state for the next launch while the tiles stream, instead of at the tail of the kernel.
-    if (tid == 0) {
+    // the state for the next launch while the tiles stream, instead of at the tail of the kernel.  (By a thread of the
+    // epilogue group, which has nothing to do yet: the fence and the ticket are round trips, which the thread that issues the
+    // first copies used to wait for.)
+    if (tid == 32 * (kFirstComputeWarp + 4 * NG)) {
         __threadfence();
         if (atomicAdd(&a.st->done, 1u) == gridDim.x - 1) {
             if constexpr (RAGGED) {
