@@ -234,7 +234,8 @@ mkv_status mkv_decode_step_host(mkv_ctx *ctx, const void *q_host, const void *k_
 /* Device pointers into one layer of the cache.  Valid until the context is destroyed;
  * contents change with every decode step.  Reading them needs a stream synchronisation.
  * The view is for reading, with one exception: slot order is free, so rows of K, V and pos may be
- * moved together between two steps, by whoever has called this function since the earlier one. */
+ * moved together between two steps, by whoever has called this function since the earlier one, and
+ * between any two replays of recorded steps. */
 mkv_status mkv_cache_view(mkv_ctx *ctx, int layer, mkv_view *view);
 
 /* Waits for `stream` and reports device-side errors (MKV_DEVICE_TIMEOUT) recorded so far. */

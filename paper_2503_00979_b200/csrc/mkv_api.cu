@@ -218,6 +218,7 @@ DecodeArgs make_args(const mkv_ctx *c, const void *q, const void *k, const void 
     a.row_shift = c->ragged ? (const int *)(b + c->L.row_shift) : nullptr;
     a.B = c->s.B; a.Hkv = c->s.Hkv;
     a.n_hint = c->prefilled ? c->n : 0;
+    a.check_moved = 0;
     return a;
 }
 
@@ -260,24 +261,30 @@ mkv_status level_states(mkv_ctx *ctx, int want, cudaStream_t stream)
     return MKV_OK;
 }
 
+// (The default stream cannot be recorded; the query costs 0.3 us of a launch.)
+bool is_capturing(cudaStream_t stream)
+{
+    if (stream == nullptr) return false;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &cs) == cudaSuccess) return cs == cudaStreamCaptureStatusActive;
+    cudaGetLastError();
+    return false;
+}
+
 // One decode step of the whole stack (layer < 0) or of one layer of this context's own.
 mkv_status launch_step(mkv_ctx *ctx, int layer, const void *q, const void *k, const void *v, void *out, cudaStream_t stream)
 {
     const mkv_status ls = level_states(ctx, layer < 0 ? 1 : 2, stream);
     if (ls != MKV_OK) return ls;
-    const DecodeArgs a = layer < 0 ? make_args(ctx, q, k, v, out) : make_args_layer(ctx, layer, q, k, v, out);
+    DecodeArgs a = layer < 0 ? make_args(ctx, q, k, v, out) : make_args_layer(ctx, layer, q, k, v, out);
     // A view of the cache has been handed out since the last step, and its holder may have rearranged the slots (their
-    // order is free): the window sums of slots whose token has changed are taken again.  At the start of a step that
-    // is looked after for all layers at once, within a step for the layer concerned.
+    // order is free).  A step that is being recorded does not know when it will be replayed, and always looks.
+    const bool capturing = is_capturing(stream);
     if (ctx->viewed) {
-        const bool start = layer <= 0;
-        bool any = false;
-        for (int l = start ? 0 : layer; l < (start ? ctx->s.layers : layer + 1); ++l) { any |= ctx->viewed[l] != 0; ctx->viewed[l] = 0; }
-        if (any) {
-            DecodeArgs w = a;
-            if (layer == 0) { w = make_args(ctx, q, k, v, out); w.st = a.st; }
-            const cudaError_t ef = launch_window_sums(w, ctx->p.dtype == MKV_DTYPE_F32, ctx->s.D, &ctx->launches, stream);
-            if (ef != cudaSuccess) return fail(ctx, MKV_CUDA, "window sums launch failed: %s", cudaGetErrorString(ef));
+        a.check_moved = capturing;
+        for (int l = layer < 0 ? 0 : layer; l < (layer < 0 ? ctx->s.layers : layer + 1) && !capturing; ++l) {
+            a.check_moved |= ctx->viewed[l];
+            ctx->viewed[l] = 0;
         }
     }
     const int nsplit = layer < 0 ? ctx->s.simt_splits : ctx->s.simt_splits_layer;
@@ -292,12 +299,6 @@ mkv_status launch_step(mkv_ctx *ctx, int layer, const void *q, const void *k, co
     // device state and does nothing if no compaction is pending)
     // (While the stream is being captured the launch is recorded after every step, so that the recorded sequence
     // stays valid when it is replayed in another phase of the eviction period.)
-    bool capturing = false;
-    if (ctx->s.T > 1 && !ev) {
-        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-        capturing = cudaStreamIsCapturing(stream, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusActive;
-        cudaGetLastError();
-    }
     if (ctx->s.T > 1 && (ev || capturing)) {
         const cudaError_t e2 = launch_compact(a, ctx->p.dtype == MKV_DTYPE_F32, ctx->s.D, stream);
         if (e2 != cudaSuccess) return fail(ctx, MKV_CUDA, "compaction launch failed: %s", cudaGetErrorString(e2));

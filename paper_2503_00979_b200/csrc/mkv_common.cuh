@@ -76,6 +76,9 @@ struct DecodeArgs {
     float *pre;                // [U][cap]
     int *sum_pos;              // [U][cap]  position of the token a slot's entries belong to (= pos, unless a holder of a
                                // cache view has rearranged the slots)
+    int check_moved;           // 1: look for slots that hold another token than their entries belong to, and take their
+                               // sums again (resum_moved).  (On every launch it would cost 2 to 3 %: 57.6 to 58.9 us for 256
+                               // units x 2032 slots, 844 to 870 for 8192 x 1056.)
     int bs, nblk;
     int n_hint;                // the host's view of st->n when the launch was enqueued (0: none).  Only used to
                                // prefetch: a stale value (steps replayed from a CUDA graph) costs time, not results
@@ -250,6 +253,60 @@ __device__ __forceinline__ void take_block(float S, int j, int open, int fusion,
         if (valid) slab[(size_t)j * cap] = S;
     }
 }
+// The window sums of slot k of unit u from its key and the ring as they stand, by one warp.  Leaves slab and pre as the step
+// that puts its query into ring slot rs_new leaves them, and returns the fused score over all rows of the window but that one.
+template <typename T, int D>
+__device__ float resum_slot(const DecodeArgs &a, int u, int k, int rs_new, int lane)
+{
+    const size_t at = (size_t)u * a.cap + k;
+    const T *kr = static_cast<const T *>(a.K) + at * D;
+    float kv[D / 32];
+#pragma unroll
+    for (int i = 0; i < D / 32; ++i) kv[i] = ldf(kr + lane + 32 * i);
+    float *slab = a.slab + (size_t)u * a.nblk * a.cap + k;
+    float F = 0.f, acc = 0.f, pre = 0.f;
+    for (int j = a.nblk - 1; j >= 0; --j) {
+        float S = 0.f;
+        for (int s = j * a.bs; s < min(a.R, (j + 1) * a.bs); ++s) {
+            if (s == rs_new) continue;
+            float Sr = 0.f;
+            for (int g = 0; g < a.G; ++g) {
+                const size_t row = ((size_t)u * a.R + s) * a.G + g;
+                const float c = a.ring_c[row];
+                if (c == INFINITY) continue;                  // empty row, padding head
+                const T *qr = static_cast<const T *>(a.ring_q) + row * D;
+                float x = 0.f;
+#pragma unroll
+                for (int i = 0; i < D / 32; ++i) x += kv[i] * ldf(qr + lane + 32 * i);
+                Sr += exp2f(warp_sum(x) * a.scale2 - c);
+            }
+            S = fuse(a.fusion, S, Sr);
+        }
+        F = fuse(a.fusion, F, S);
+        take_block(S, j, rs_new / a.bs, a.fusion, slab, a.cap, lane == 0, acc, pre);
+    }
+    if (lane == 0) { a.pre[at] = pre; a.sum_pos[at] = a.pos[at]; }
+    return F;
+}
+
+// The slots k0 .. k1 - 1 of unit u whose token is not the one that their sums belong to, by `nwarp` warps; F[k - k0] receives
+// what resum_slot returns.  Nothing has moved as a rule, and then this is not called.
+template <typename T, int D>
+__device__ __noinline__ void resum_moved(const DecodeArgs &a, int u, int k0, int k1, int rs_new, float *F, int warp, int nwarp, int lane)
+{
+    const int *pos = a.pos + (size_t)u * a.cap, *sum_pos = a.sum_pos + (size_t)u * a.cap;
+    for (int kb = k0 + 32 * warp; kb < k1; kb += 32 * nwarp) {
+        const int k = kb + lane;
+        unsigned todo = __ballot_sync(0xffffffffu, k < k1 && pos[k] != sum_pos[k]);
+        while (todo != 0) {
+            const int b = __ffs(todo) - 1;
+            todo &= todo - 1;
+            const float f = resum_slot<T, D>(a, u, kb + b, rs_new, lane);
+            if (lane == 0) F[kb + b - k0] = f;
+        }
+    }
+}
+
 
 // CURRENT normalisation (the reading of Eq. 4 in which a window row's weights are taken over the tokens that are
 // still cached): the token in `e_slot` is about to be evicted, so every window row loses the weight w it had on it
@@ -300,10 +357,10 @@ __device__ void renormalise_after_eviction(const DecodeArgs &a, int u, int e_slo
 // `sm` needs kFinalizeSmemFloats floats of shared memory, 8-byte aligned.  GT is the GQA
 // group size when known at compile time (0: use a.G); it lets the loads of a round be
 // issued together.  Loads are batched so that the whole epilogue costs a handful of L2
-// round trips.
+// round trips.  `moved`: a slot of the unit holds another token than its window sums belong to.
 template <typename T, int D, int GT>
 __device__ void finalize_unit(const DecodeArgs &a, int u, long long t, int n, int active, bool evict, float *sm,
-                              int tid, int nthr, int bar_id, int shift = 0)
+                              int tid, int nthr, int bar_id, int shift = 0, bool moved = false)
 {
     const int lane = tid & 31, warp = tid >> 5, nwarp = nthr >> 5;
     const int G = GT > 0 ? GT : a.G;
@@ -378,6 +435,10 @@ __device__ void finalize_unit(const DecodeArgs &a, int u, long long t, int n, in
     int *pos = a.pos + (size_t)u * a.cap;
     float *F = a.F + (size_t)u * a.cap;
     int e_slot = n, e_pos = -1;
+    if (moved) {
+        resum_moved<T, D>(a, u, 0, n, ring_slot(t, a.R), F, warp, nwarp, lane);
+        group_sync(bar_id, nthr);
+    }
     if (evict) {
         const float *sn = a.s_new + (size_t)u * G * a.cap;
         const long long thr = t - shift - a.R;        // positions are the row's own; ring slots follow t

@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(kCT, KPT <= 4 ? 2 : 1) compact_kernel(DecodeAr
                 float *row = j < a.nblk ? slab + (size_t)j * a.cap : pre;
                 row[holes[i]] = row[movers[i]];
             }
-            if (tid < nh) a.sum_pos[(size_t)u * a.cap + holes[tid]] = pos[movers[tid]];
+            if (tid < nh) a.sum_pos[(size_t)u * a.cap + holes[tid]] = a.sum_pos[(size_t)u * a.cap + movers[tid]];
         }
         __syncthreads();
         for (int k = keep + tid; k < n; k += kCT) {

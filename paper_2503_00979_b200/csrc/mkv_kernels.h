@@ -66,9 +66,6 @@ size_t prefill_static_max_floats();
 cudaError_t run_prefill_static(const DecodeArgs &a, bool f32, int D, const void *k, const void *v, const void *q_window,
                                int P, cudaStream_t stream, unsigned long long *launches, int device, int n_states);
 
-// The window sums (DecodeArgs::slab) of the slots whose token is no longer the one in sum_pos, for the step that a.st
-// holds.  *launches counts the launches.
-cudaError_t launch_window_sums(const DecodeArgs &a, bool f32, int D, unsigned long long *launches, cudaStream_t stream);
 // The gather of the kept prompt rows into the arena and the window sums in one launch (windows of up to 256 ring rows on the
 // tensor cores); a.pos and the ring are there.
 bool gather_sums_supported(const DecodeArgs &a, const void *k, const void *v);

@@ -182,6 +182,7 @@ decode_simt_kernel(const __grid_constant__ DecodeArgs a, const int nsplit, const
     const T *Ku = static_cast<const T *>(a.K) + (size_t)u * a.cap * D, *Vu = static_cast<const T *>(a.V) + (size_t)u * a.cap * D;
     const int *pos = a.pos + (size_t)u * a.cap;
     float *slab = kept ? a.slab + (size_t)u * a.nblk * a.cap : nullptr, *pre = kept ? a.pre + (size_t)u * a.cap : nullptr;
+    bool moved = false;                                         // a slot holds another token than its window sums belong to
     // scores, logits and positions of this CTA's keys: in shared memory if they fit (index key - k0), else in the arena
     // (CURRENT normalisation reads the logits there)
     const bool local = per <= L::keys && !a.norm_current;
@@ -257,6 +258,7 @@ decode_simt_kernel(const __grid_constant__ DecodeArgs a, const int nsplit, const
                     f_rest = fuse(a.fusion, f_rest, f_pre);
                 }
                 if (local && evict && valid) pk[kl] = pos[key];
+                if (a.check_moved && valid) moved |= pos[key] != __ldcg(a.sum_pos + (size_t)u * a.cap + key);
                 cp_async_wait<1>();
                 __syncwarp();
                 // ---------------- fused scores over the resident rows
@@ -688,6 +690,10 @@ decode_simt_kernel(const __grid_constant__ DecodeArgs a, const int nsplit, const
         for (int r = 0; r < kMaxCluster; ++r)
             if (r < nsplit) o += co[r * slice + i] * cml[(r * GP + g) * 2];
         stf(out + idx, o / fin.l[g]);
+    }
+    if (a.check_moved && __syncthreads_or(moved)) {
+        resum_moved<T, D>(a, u, k0, k1, rs_new, Fk, warp, kWarps, lane);
+        __syncthreads();
     }
     // ---------------- Algorithm 1 / Eq. 7: add the new row's term to the scores of this CTA's keys, evict the minimum
     int e_slot = us.n, e_pos = -1;

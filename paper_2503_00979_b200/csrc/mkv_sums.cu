@@ -7,10 +7,6 @@
 // up to 256 at a time) and the CTA layout of the prompt phase's scoring passes: warps 0-3 and 6-9 are two consumer
 // groups on alternate key tiles and accumulator buffers, warp 4 feeds K tiles with TMA, warp 5 issues the MMAs.
 // Bound by the kept keys' bytes and R*G exponentials per key (256 units of 2048 slots, 128 rows: 38 us).
-//
-// window_sums_kernel does the same on the CUDA cores for the slots whose token is no longer the one their sums belong
-// to: a holder of a cache view may rearrange the slots, so the first step after a view has been handed out runs it (as cheap as reading 8 bytes per slot).
-// Nothing has moved as a rule, and it ends after comparing two positions per slot.
 #include <string.h>
 
 #include "mkv_common.cuh"
@@ -449,44 +445,6 @@ cudaError_t launch_gather_g(const GatherArgs &a, const CUtensorMap &tmK, const C
     return launch_chained(kern, dim3((unsigned)(tiles < 148 ? tiles : 148)), kGsThreads, smem, stream, a, tmK, tmV);
 }
 
-// What is timed is the comparison, 8 bytes per slot in 16-byte loads; a slot that was moved is redone by one thread.
-constexpr int kSumKeys = 256;
-template <typename T, int D>
-__global__ void __launch_bounds__(kSumKeys) window_sums_kernel(const __grid_constant__ DecodeArgs d)
-{
-    const size_t total = (size_t)d.U * d.cap, i4 = ((size_t)blockIdx.x * kSumKeys + threadIdx.x) * 4;
-    if (i4 >= total) return;
-    // (a layer's arrays need not start on a 16-byte boundary)
-    if (i4 + 4 <= total && (((uintptr_t)d.pos | (uintptr_t)d.sum_pos) & 15) == 0) {
-        const int4 x = *reinterpret_cast<const int4 *>(d.pos + i4), y = *reinterpret_cast<const int4 *>(d.sum_pos + i4);
-        if (x.x == y.x && x.y == y.y && x.z == y.z && x.w == y.w) return;
-    }
-    for (size_t at = i4; at < total && at < i4 + 4; ++at) {
-        if (d.pos[at] == d.sum_pos[at] || d.pos[at] < 0) continue;
-        const size_t u = at / d.cap;
-        const int key = (int)(at % d.cap), G = d.G, open = open_block(d.st->t, d.R, d.bs);
-        const T *kr = static_cast<const T *>(d.K) + at * D;
-        float acc = 0.f, pre = 0.f;
-        for (int j = d.nblk - 1; j >= 0; --j) {
-            float S = 0.f;
-            for (int s = j * d.bs; s < min(d.R, (j + 1) * d.bs); ++s) {
-                float Sr = 0.f;
-                for (int g = 0; g < G; ++g) {
-                    const size_t row = (u * d.R + s) * G + g;
-                    const T *qr = static_cast<const T *>(d.ring_q) + row * D;
-                    float x = 0.f;
-                    for (int i = 0; i < D; ++i) x += ldf(qr + i) * ldf(kr + i);
-                    Sr += exp2f(x * d.scale2 - d.ring_c[row]);
-                }
-                S = fuse(d.fusion, S, Sr);
-            }
-            take_block(S, j, open, d.fusion, d.slab + u * d.nblk * d.cap + key, d.cap, true, acc, pre);
-        }
-        d.pre[at] = pre;
-        d.sum_pos[at] = d.pos[at];
-    }
-}
-
 __global__ void set_states_kernel(const __grid_constant__ SumArgs a)
 {
     chain_wait();
@@ -519,20 +477,6 @@ DecodeArgs unit_range(const DecodeArgs &d, int D, size_t es, int u0, int count)
 constexpr int kMaxGridY = 65535;
 
 }  // namespace
-
-cudaError_t launch_window_sums(const DecodeArgs &d, bool f32, int D, unsigned long long *launches, cudaStream_t stream)
-{
-    const unsigned grid = (unsigned)(((size_t)d.U * d.cap + 4 * kSumKeys - 1) / (4 * kSumKeys));
-    if (f32) {
-        if (D == 64) window_sums_kernel<float, 64><<<grid, kSumKeys, 0, stream>>>(d);
-        else window_sums_kernel<float, 128><<<grid, kSumKeys, 0, stream>>>(d);
-    } else {
-        if (D == 64) window_sums_kernel<__nv_bfloat16, 64><<<grid, kSumKeys, 0, stream>>>(d);
-        else window_sums_kernel<__nv_bfloat16, 128><<<grid, kSumKeys, 0, stream>>>(d);
-    }
-    ++*launches;
-    return cudaGetLastError();
-}
 
 bool gather_sums_supported(const DecodeArgs &d, const void *k, const void *v)
 {

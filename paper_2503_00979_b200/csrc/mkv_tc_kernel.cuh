@@ -145,7 +145,7 @@ template <int G> struct NewRows {
 
 template <int G, bool LOCAL>
 __device__ void finalize_fast(const DecodeArgs &a, int u, long long t, int n, int nseg, bool evict, float *sm, int tid,
-                              int bar_id, const float (&l_o)[G], const float *l_ml, int shift, const NewRows<G> &x)
+                              int bar_id, const float (&l_o)[G], const float *l_ml, int shift, const NewRows<G> &x, bool moved)
 {
     constexpr int NT_ = kGroupThreads;
     const int lane = tid & 31, warp = tid >> 5;
@@ -222,6 +222,10 @@ __device__ void finalize_fast(const DecodeArgs &a, int u, long long t, int n, in
     int *pos = a.pos + (size_t)u * a.cap;
     float *F = a.F + (size_t)u * a.cap;
     int e_slot = n, e_pos = -1;
+    if (moved) {      // (rare)
+        resum_moved<__nv_bfloat16, kD>(a, u, 0, n, ring_slot(t, a.R), F, warp, NT_ / 32, lane);
+        group_sync(bar_id, NT_);
+    }
     if (!evict) {
         // no selection on this step (cache still filling, or between two runs of a coarse-grained policy):
         // the new token takes the next free slot
@@ -872,21 +876,44 @@ decode_tc_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ C
         const float *wml = reinterpret_cast<const float *>(smem + L.wml);
         float *epi = reinterpret_cast<float *>(smem + L.epi);
         float *fin_sm = epi;                                          // kFinFloats
-        int *flag = reinterpret_cast<int *>(epi + kFinFloats);
+        int *flag = reinterpret_cast<int *>(epi + kFinFloats), *moved_flag = flag + 1;
         float *cml = epi + kFinFloats + 8;                            // merged (m, l) [g][2]
         float *sc = cml + 2 * kMaxGroup;                              // [warp][g] scale to the merged reference
         WalkT<WHOLE> w(a.U * NCe, n, (int)gridDim.x, (int)blockIdx.x);
         Item x;
         bool ok = true;
         int k = 0;                                                    // units finished so far
+        if (etid == 0) *moved_flag = 0;
+        group_sync(kEpiBar, kGroupThreads);
         while (ok && w.next(x)) {
             {
                 const int u = MC ? x.unit / NCe : x.unit;
                 const bool main_item = MC ? (NCe == 1 || x.unit - u * NCe == c_main) : true;
                 const UnitStep us = RAGGED ? unit_step(a, u, t, n, steps_done, evict) : UnitStep{n, 0, evict};
+                // do the kept sums belong to the tokens in this item's slots?
+                if constexpr (BLOCKS) {
+                    if (a.check_moved) {
+                        const int *pos = a.pos + (size_t)u * a.cap, *sum_pos = a.sum_pos + (size_t)u * a.cap;
+                        const int k1 = min(us.n, (x.tile0 + x.nk) * kTile);
+                        for (int kb = x.tile0 * kTile + etid; kb < k1; kb += 8 * kGroupThreads) {
+                            int p[8], ps[8];
+#pragma unroll
+                            for (int b = 0; b < 8; ++b) {          // (unconditional: all in flight together)
+                                const int key = min(kb + b * kGroupThreads, k1 - 1);
+                                p[b] = __ldcg(pos + key);
+                                ps[b] = __ldcg(sum_pos + key);
+                            }
+                            bool diff = false;
+#pragma unroll
+                            for (int b = 0; b < 8; ++b) diff |= p[b] != ps[b];
+                            if (diff) *moved_flag = 1;
+                        }
+                    }
+                }
                 NewRows<G> rows;
                 if constexpr (!MC) rows.load(a, u, etid);
                 if (group_any(kEpiBar, !mbar_wait(bar_udone, (uint32_t)(k & 1), abort_flag, kWaitUDone, WL))) { ok = false; break; }
+                bool moved = BLOCKS && *moved_flag != 0;
                 // merge the compute warps' partials: common reference = max of theirs
                 if (etid < G && main_item) {
                     float m = -INFINITY;
@@ -952,7 +979,7 @@ decode_tc_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ C
                                                                   kEpiBar, RAGGED ? us.shift : 0);
                     }
                 } else if (ncta == 1) {
-                    finalize_fast<G, true>(a, u, t, us.n, 1, us.evict, fin_sm, etid, kEpiBar, o, cml, RAGGED ? us.shift : 0, rows);
+                    finalize_fast<G, true>(a, u, t, us.n, 1, us.evict, fin_sm, etid, kEpiBar, o, cml, RAGGED ? us.shift : 0, rows, moved);
                 } else {
                     // the unit is shared: publish this CTA's partial; the last CTA to do so finishes the unit.
                     // The group barrier orders every thread's writes (and, through the mbarrier above, the compute
@@ -967,19 +994,22 @@ decode_tc_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ C
                     if (etid == 0) {
                         // release: the group's writes above (ordered before this thread by the barrier) become visible
                         // to whoever observes the ticket; acquire: the last arriver's reads below see the others'
+                        // (the upper half of the ticket counts the CTAs that have seen a moved slot)
                         int old;
-                        asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;" : "=r"(old) : "l"(a.ticket + u) : "memory");
-                        *flag = old == ncta - 1;
+                        asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], %2;" : "=r"(old) : "l"(a.ticket + u), "r"(moved ? 0x10001 : 1) : "memory");
+                        *flag = (old & 0xffff) == ncta - 1 ? 1 + (old >> 16) : 0;
                     }
                     group_sync(kEpiBar, kGroupThreads);
                     if (*flag) {
+                        moved |= *flag > 1;
                         if (ncta <= 8 && ncta * G * 2 <= 256)
-                            finalize_fast<G, false>(a, u, t, us.n, ncta, us.evict, fin_sm, etid, kEpiBar, o, nullptr, RAGGED ? us.shift : 0, rows);
+                            finalize_fast<G, false>(a, u, t, us.n, ncta, us.evict, fin_sm, etid, kEpiBar, o, nullptr, RAGGED ? us.shift : 0, rows, moved);
                         else
                             finalize_unit<__nv_bfloat16, kD, G>(a, u, t, us.n, ncta, us.evict, fin_sm, etid, kGroupThreads, kEpiBar,
-                                                                RAGGED ? us.shift : 0);
+                                                                RAGGED ? us.shift : 0, moved);
                     }
                 }
+                if (BLOCKS && etid == 0) *moved_flag = 0;
                 group_sync(kEpiBar, kGroupThreads);
                 ++k;
             }
