@@ -131,8 +131,8 @@ __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 // GP: the group padded to a power of two (padding heads: zero query, weight 0).  `early`: the launch before this one
-// does not touch this launch's units.
-template <typename T, int D, int GP>
+// does not touch this launch's units.  CHECK: DecodeArgs::check_moved (compiled apart, as it costs a layer's call 0.4 us).
+template <typename T, int D, int GP, bool CHECK>
 __global__ void __launch_bounds__(SimtSmem<T, D, GP>::threads, GP > 8 ? 1 : SimtSmem<T, D, GP>::ctas)
 decode_simt_kernel(const __grid_constant__ DecodeArgs a, const int nsplit, const int early)
 {
@@ -258,7 +258,7 @@ decode_simt_kernel(const __grid_constant__ DecodeArgs a, const int nsplit, const
                     f_rest = fuse(a.fusion, f_rest, f_pre);
                 }
                 if (local && evict && valid) pk[kl] = pos[key];
-                if (a.check_moved && valid) moved |= pos[key] != __ldcg(a.sum_pos + (size_t)u * a.cap + key);
+                if (CHECK && valid) moved |= pos[key] != __ldcg(a.sum_pos + (size_t)u * a.cap + key);
                 cp_async_wait<1>();
                 __syncwarp();
                 // ---------------- fused scores over the resident rows
@@ -691,7 +691,7 @@ decode_simt_kernel(const __grid_constant__ DecodeArgs a, const int nsplit, const
             if (r < nsplit) o += co[r * slice + i] * cml[(r * GP + g) * 2];
         stf(out + idx, o / fin.l[g]);
     }
-    if (a.check_moved && __syncthreads_or(moved)) {
+    if (CHECK && __syncthreads_or(moved)) {
         resum_moved<T, D>(a, u, k0, k1, rs_new, Fk, warp, kWarps, lane);
         __syncthreads();
     }
@@ -793,10 +793,10 @@ decode_simt_kernel(const __grid_constant__ DecodeArgs a, const int nsplit, const
     }
 }
 
-template <typename T, int D, int GP>
+template <typename T, int D, int GP, bool CHECK>
 cudaError_t launch_simt_g(const DecodeArgs &a, int nsplit, bool early, cudaStream_t stream)
 {
-    auto kern = decode_simt_kernel<T, D, GP>;
+    auto kern = decode_simt_kernel<T, D, GP, CHECK>;
     const int smem = SimtSmem<T, D, GP>::total;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess && nsplit > 8) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -817,17 +817,24 @@ cudaError_t launch_simt_g(const DecodeArgs &a, int nsplit, bool early, cudaStrea
     return cudaLaunchKernelEx(&cfg, kern, a, nsplit, early ? 1 : 0);
 }
 
-template <typename T, int D>
+template <typename T, int D, bool CHECK>
 cudaError_t launch_simt_t(const DecodeArgs &a, int nsplit, bool early, cudaStream_t stream)
 {
     switch (tc_padded_group(a.G)) {
-        case 1: return launch_simt_g<T, D, 1>(a, nsplit, early, stream);
-        case 2: return launch_simt_g<T, D, 2>(a, nsplit, early, stream);
-        case 4: return launch_simt_g<T, D, 4>(a, nsplit, early, stream);
-        case 8: return launch_simt_g<T, D, 8>(a, nsplit, early, stream);
-        case 16: return launch_simt_g<T, D, 16>(a, nsplit, early, stream);
+        case 1: return launch_simt_g<T, D, 1, CHECK>(a, nsplit, early, stream);
+        case 2: return launch_simt_g<T, D, 2, CHECK>(a, nsplit, early, stream);
+        case 4: return launch_simt_g<T, D, 4, CHECK>(a, nsplit, early, stream);
+        case 8: return launch_simt_g<T, D, 8, CHECK>(a, nsplit, early, stream);
+        case 16: return launch_simt_g<T, D, 16, CHECK>(a, nsplit, early, stream);
     }
     return cudaErrorInvalidValue;
+}
+
+template <bool CHECK>
+cudaError_t launch_simt_c(const DecodeArgs &a, int nsplit, bool early, bool f32, int D, cudaStream_t stream)
+{
+    if (f32) return D == 64 ? launch_simt_t<float, 64, CHECK>(a, nsplit, early, stream) : launch_simt_t<float, 128, CHECK>(a, nsplit, early, stream);
+    return D == 64 ? launch_simt_t<__nv_bfloat16, 64, CHECK>(a, nsplit, early, stream) : launch_simt_t<__nv_bfloat16, 128, CHECK>(a, nsplit, early, stream);
 }
 
 }  // namespace
@@ -835,8 +842,7 @@ cudaError_t launch_simt_t(const DecodeArgs &a, int nsplit, bool early, cudaStrea
 cudaError_t launch_decode_simt(const DecodeArgs &a, int nsplit, bool early, bool f32, int D, cudaStream_t stream)
 {
     if (nsplit > kMaxCluster) return cudaErrorInvalidValue;
-    if (f32) return D == 64 ? launch_simt_t<float, 64>(a, nsplit, early, stream) : launch_simt_t<float, 128>(a, nsplit, early, stream);
-    return D == 64 ? launch_simt_t<__nv_bfloat16, 64>(a, nsplit, early, stream) : launch_simt_t<__nv_bfloat16, 128>(a, nsplit, early, stream);
+    return a.check_moved ? launch_simt_c<true>(a, nsplit, early, f32, D, stream) : launch_simt_c<false>(a, nsplit, early, f32, D, stream);
 }
 
 // Rows of a block are scored on every step and once more when it is finished: 16 where they cost scalar FMAs, 32 on the
