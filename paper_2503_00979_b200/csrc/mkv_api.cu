@@ -176,8 +176,11 @@ struct mkv_ctx {
     int steps;
     int next_layer;   // per-layer calls: the layer (of this context's own) expected next; 0 at a step boundary
     int cursor;       // per-layer calls: the layer of the whole model expected next (kept by the outer context)
+    int last_layer;   // what this context launched last: layer (-1: something else), on which stream, while it was recorded or not
+    cudaStream_t last_stream;
+    bool last_capturing;
     int state_ahead;  // 0: whole-stack and per-layer device states level, 1: whole-stack ahead, 2: per-layer ahead
-    unsigned char *viewed;       // [layers] (contexts that keep window sums): a view has been handed out since the last step
+    unsigned char *viewed;       // [layers]: a view has been handed out since the last step
     unsigned long long launches;
     PrefillScratch prefill_scratch;
     char err[256];
@@ -274,22 +277,29 @@ bool is_capturing(cudaStream_t stream)
 // One decode step of the whole stack (layer < 0) or of one layer of this context's own.
 mkv_status launch_step(mkv_ctx *ctx, int layer, const void *q, const void *k, const void *v, void *out, cudaStream_t stream)
 {
+    const unsigned long long before = ctx->launches;
     const mkv_status ls = level_states(ctx, layer < 0 ? 1 : 2, stream);
     if (ls != MKV_OK) return ls;
     DecodeArgs a = layer < 0 ? make_args(ctx, q, k, v, out) : make_args_layer(ctx, layer, q, k, v, out);
     // A view of the cache has been handed out since the last step, and its holder may have rearranged the slots (their
     // order is free).  A step that is being recorded does not know when it will be replayed, and always looks.
     const bool capturing = is_capturing(stream);
-    if (ctx->viewed) {
-        a.check_moved = capturing;
-        for (int l = layer < 0 ? 0 : layer; l < (layer < 0 ? ctx->s.layers : layer + 1) && !capturing; ++l) {
-            a.check_moved |= ctx->viewed[l];
-            ctx->viewed[l] = 0;
-        }
+    bool viewed = false;
+    for (int l = layer < 0 ? 0 : layer; l < (layer < 0 ? ctx->s.layers : layer + 1); ++l) {
+        viewed |= ctx->viewed[l] != 0;
+        if (!capturing) ctx->viewed[l] = 0;
     }
+    a.check_moved = a.nblk > 1 && (capturing || viewed);
     const int nsplit = layer < 0 ? ctx->s.simt_splits : ctx->s.simt_splits_layer;
-    // (of two layers or more, the launch before a layer's is another layer's, or no programmatic predecessor at all)
-    const bool early = layer >= 0 && ctx->s.layers > 1;
+    // A launch may run ahead of the end of the one before it in its stream if that belongs to another layer: what this layer
+    // holds was then written before that one let this one start.  Not so behind a launch of the same layer (layers on streams of
+    // their own), behind the state copy above, or behind a view's holder's own work on the slots.  (cudaStreamPerThread names
+    // another stream in every thread.)
+    const bool early = layer >= 0 && ctx->last_layer >= 0 && ctx->last_layer != layer && ctx->last_stream == stream &&
+                       stream != cudaStreamPerThread && ctx->last_capturing == capturing && ctx->launches == before && !viewed;
+    ctx->last_layer = layer;
+    ctx->last_stream = stream;
+    ctx->last_capturing = capturing;
     const cudaError_t e = nsplit > 0 ? launch_decode_simt(a, nsplit, early, ctx->p.dtype == MKV_DTYPE_F32, ctx->s.D, stream)
                                      : launch_decode_tc(layer < 0 ? ctx->plan : ctx->plan_layer, a, stream);
     if (e != cudaSuccess) return fail(ctx, MKV_CUDA, "decode launch failed: %s", cudaGetErrorString(e));
@@ -344,10 +354,9 @@ mkv_status core_create(mkv_ctx **out, const mkv_params *p, void *workspace, size
     c->row_n = new (std::nothrow) int[2 * (size_t)s.B];
     if (!c->row_n) { delete c; return MKV_OOM; }
     c->row_shift = c->row_n + s.B;
-    if (s.nblk > 1) {
-        c->viewed = new (std::nothrow) unsigned char[s.layers]();
-        if (!c->viewed) { delete[] c->row_n; delete c; return MKV_OOM; }
-    }
+    c->viewed = new (std::nothrow) unsigned char[s.layers]();
+    if (!c->viewed) { delete[] c->row_n; delete c; return MKV_OOM; }
+    c->last_layer = -1;
     if (cudaGetDevice(&c->device) != cudaSuccess) { cudaGetLastError(); delete[] c->row_n; delete[] c->viewed; delete c; return MKV_CUDA; }
     if (workspace) {
         c->base = (char *)workspace;
@@ -529,7 +538,7 @@ void core_view(mkv_ctx *ctx, int layer, mkv_view *view)
     const size_t u0 = (size_t)ctx->s.upl * layer;
     const Shape &s = ctx->s;
     char *b = ctx->base;
-    if (ctx->viewed) ctx->viewed[layer] = 1;
+    ctx->viewed[layer] = 1;
     view->K = b + ctx->L.K + u0 * s.cap * s.D * s.es;
     view->V = b + ctx->L.V + u0 * s.cap * s.D * s.es;
     view->pos = (int32_t *)(b + ctx->L.pos) + u0 * s.cap;
@@ -673,7 +682,7 @@ mkv_status mkv_reset(mkv_ctx *ctx)
         if (!c) continue;
         c->prefilled = false;
         c->ragged = false;
-        c->t = 0; c->n = 0; c->steps = 0; c->next_layer = 0; c->state_ahead = 0; c->cursor = 0;
+        c->t = 0; c->n = 0; c->steps = 0; c->next_layer = 0; c->state_ahead = 0; c->cursor = 0; c->last_layer = -1;
     }
     return MKV_OK;
 }

@@ -21,7 +21,7 @@
 //
 // Bound by HBM for bf16 and, nearly, by FMA issue for f32; small launches by their chain of latencies.  Of those
 // everything that does not need the new query (state, tiles, ring rows, their scoring) may run before the launch before
-// this one has ended, when that launch works on other layers (`early`).
+// this one has ended, when that launch works on another layer (`early`).
 //
 // Measured: 512 units x 1056 slots, bf16, d = 64, R*G = 128: 65 us per step (all rows scored with scalar FMAs, CTA barriers
 // per tile: 838).  2 units x 80 slots, f32, d = 64: 10.6 us (30.6).  One layer of 8 units x 2032 slots, bf16, d = 128, as a

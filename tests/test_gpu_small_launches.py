@@ -1,10 +1,12 @@
 """Launches of a tcgen05 context too small to fill the chip, which the warp-level kernel takes (a cluster per unit): the
 cluster sizes, ranges and blocks at which it can go wrong, steps that alternate between layer calls and whole-stack calls,
-two layers back to back (a layer's launch starts before the one before it has ended), and the neighbours that stay with
+layers back to back (a layer's launch starts before the one before it has ended), and the neighbours that stay with
 the tcgen05 kernel.  Tolerances are those of the lock-step comparison with the oracle."""
+import numpy as np
 import pytest
+import torch
 
-from paper_2503_00979_b200 import synth
+from paper_2503_00979_b200 import binding, synth
 from tests.parity import run_parity, run_parity_coarse, run_parity_ragged
 
 pytestmark = pytest.mark.gpu
@@ -32,3 +34,45 @@ def test_coarse_grained_and_ragged():
     assert run_parity_coarse(w, T=5, steps=23, n_units=2).evictions > 0
     w = synth.Workload("small_ragged", 2, 3, 8, 2, 128, "bf16", 0, 40, 250, 20, "sum", 6)
     assert run_parity_ragged(w, [400, 262, 5], steps=40, per_layer=1).evictions > 0
+
+
+# Layer calls with nothing between them, so that a layer's launch does start before the one before it has ended: outputs,
+# positions and normalisers bit for bit those of the same calls with a synchronisation after each.  `order`: all layers on one
+# stream, a stream for each layer (two launches of a layer are then neighbours in their stream; nothing orders the layers
+# against one another), or layer calls alternating with whole-stack steps (a state copy goes ahead of the layer's launch; both
+# contexts take the same calls).
+@pytest.mark.parametrize("order", ["one stream", "a stream per layer", "alternating"])
+@pytest.mark.parametrize("layers,C,kernel,dtype,T", [(2, 90, "auto", "bf16", 1), (3, 500, "auto", "bf16", 1), (2, 90, "auto", "bf16", 5),
+                                                     (2, 90, "tc", "bf16", 1), (3, 70, "simt", "f32", 1)])
+def test_layer_calls_back_to_back(layers, C, kernel, dtype, T, order):
+    w = synth.Workload("back_to_back", layers, 1, 8, 2, 128, dtype, C + 16, 200, C, 16, "max", 8)
+    dev, tdt = torch.device("cuda:0"), synth.torch_dtype(dtype)
+    st = synth.Stream(w, dev)
+    P = w.prompt_len
+    k, v = st.kv(np.arange(P))
+    qw = st.q(np.arange(P - w.R, P))
+    kk, vv = st.kv(np.arange(P, P + w.steps))
+    q1, k1, v1 = (x.permute(3, 0, 1, 2, 4).to(tdt).contiguous() for x in (st.q(np.arange(P, P + w.steps)), kk, vv))
+    got = []
+    for wait in (True, False):
+        mk = binding.MorphKV(layers, 1, 8, 2, 128, C, w.R, w.fusion, dtype, kernel=kernel, evict_interval=T)
+        mk.prefill(*(x.to(tdt).contiguous() for x in (k, v, qw)))
+        streams = [torch.cuda.Stream() for _ in range(layers if order == "a stream per layer" else 1)]
+        out = torch.empty_like(q1)
+        calls = [(i, l, (q1[i, l], k1[i, l], v1[i, l], out[i, l])) for i in range(w.steps) for l in range(layers)]
+        torch.cuda.synchronize()
+        for i, l, x in calls:
+            s = streams[l % len(streams)]
+            if order == "alternating" and i % 3 == 2:
+                if l == 0:
+                    mk.decode_step(q1[i], k1[i], v1[i], out[i], stream=s)
+            else:
+                mk.decode_step_layer(l, *x, stream=s)
+            if wait:
+                torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        mk.sync()
+        views = [mk.view(l) for l in range(layers)]
+        got.append([out] + [vw[name].clone() for vw in views for name in ("pos", "ring_c", "F")])
+        mk.close()
+    assert all(torch.equal(a, b) for a, b in zip(*got))
