@@ -20,7 +20,8 @@
  *   - Every `const void*` / `void*` tensor argument is a DEVICE pointer unless the name of
  *     the function ends in `_host`.  Tensors are contiguous, row-major, in the context's
  *     dtype (bf16 or f32).  The library applies no positional encoding: q and k are used
- *     as given.
+ *     as given.  A prompt's k and v start at a multiple of 16 bytes, its q_window at one of
+ *     four elements (MKV_INVALID_ARG otherwise); other tensors may start at any element.
  *   - `stream` is a `cudaStream_t` passed as `void*` (NULL = the default stream).  Calls
  *     enqueue work on it and return without synchronising unless stated otherwise.
  *   - No call throws or aborts across this boundary.  Every call returns an `mkv_status`;

@@ -291,6 +291,17 @@ mkv_status launch_step(mkv_ctx *ctx, int layer, const void *q, const void *k, co
     }
     a.check_moved = a.nblk > 1 && (capturing || viewed);
     const int nsplit = layer < 0 ? ctx->s.simt_splits : ctx->s.simt_splits_layer;
+    // the tcgen05 kernel reads its inputs 16 bytes at a time: tensors that start elsewhere go through the staging buffers
+    if (nsplit == 0 && (((uintptr_t)q | (uintptr_t)k | (uintptr_t)v) & 15) != 0) {
+        const size_t row = ctx->s.D * ctx->s.es, u0 = layer < 0 ? 0 : (size_t)layer * ctx->s.upl;
+        const size_t kb = (size_t)a.U * row, qb = kb * ctx->s.Gq;
+        char *sq = ctx->base + ctx->L.stage_q + u0 * row * ctx->s.Gq, *sk = ctx->base + ctx->L.stage_k + u0 * row, *sv = ctx->base + ctx->L.stage_v + u0 * row;
+        cudaError_t ec = cudaMemcpyAsync(sq, q, qb, cudaMemcpyDefault, stream);
+        if (ec == cudaSuccess) ec = cudaMemcpyAsync(sk, k, kb, cudaMemcpyDefault, stream);
+        if (ec == cudaSuccess) ec = cudaMemcpyAsync(sv, v, kb, cudaMemcpyDefault, stream);
+        if (ec != cudaSuccess) return fail(ctx, MKV_CUDA, "decode inputs: %s", cudaGetErrorString(ec));
+        a.q = sq; a.k_new = sk; a.v_new = sv;
+    }
     // A launch may run ahead of the end of the one before it in its stream if that belongs to another layer: what this layer
     // holds was then written before that one let this one start.  Not so behind a launch of the same layer (layers on streams of
     // their own), behind the state copy above, or behind a view's holder's own work on the slots.  (cudaStreamPerThread names
@@ -656,11 +667,18 @@ void mkv_destroy(mkv_ctx *ctx)
     core_destroy(ctx);
 }
 
+// k and v are read 16 bytes at a time, the queries at least four elements at a time
+static bool prompt_aligned(const mkv_ctx *ctx, const void *k, const void *v, const void *q_window)
+{
+    return (((uintptr_t)k | (uintptr_t)v) & 15) == 0 && ((uintptr_t)q_window & (4 * ctx->s.es - 1)) == 0;
+}
+
 static mkv_status prefill_any(mkv_ctx *ctx, const void *k, const void *v, const void *q_window, int prompt_len, void *stream,
                               bool use_static, const char *who)
 {
     if (!ctx) return MKV_INVALID_ARG;
     if (!k || !v || !q_window) return fail(ctx, MKV_INVALID_ARG, "%s: NULL tensor", who);
+    if (!prompt_aligned(ctx, k, v, q_window)) return fail(ctx, MKV_INVALID_ARG, "%s: k and v must be 16-byte aligned, q_window to four elements", who);
     if (prompt_len < 1 || prompt_len > (1 << 24)) return fail(ctx, MKV_INVALID_ARG, "%s: prompt_len out of range", who);
     if (ctx->prefilled) return fail(ctx, MKV_BAD_STATE, "%s: context already holds a sequence", who);
     const int Rw = prompt_len < ctx->s.R ? prompt_len : ctx->s.R;
@@ -702,6 +720,7 @@ mkv_status mkv_prefill_ragged(mkv_ctx *ctx, const void *k, const void *v, const 
 {
     if (!ctx) return MKV_INVALID_ARG;
     if (!k || !v || !q_window || !prompt_len) return fail(ctx, MKV_INVALID_ARG, "mkv_prefill_ragged: NULL argument%s");
+    if (!prompt_aligned(ctx, k, v, q_window)) return fail(ctx, MKV_INVALID_ARG, "mkv_prefill_ragged: k and v must be 16-byte aligned, q_window to four elements%s");
     if (padded_len < 1 || padded_len > (1 << 24)) return fail(ctx, MKV_INVALID_ARG, "mkv_prefill_ragged: padded_len out of range%s");
     for (int b = 0; b < ctx->p.batch; ++b)
         if (prompt_len[b] < 1 || prompt_len[b] > padded_len)

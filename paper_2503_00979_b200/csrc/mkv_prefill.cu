@@ -527,7 +527,7 @@ cudaError_t run_prefill_t(const DecodeArgs &a, const T *k, const T *v, const T *
     // bf16 / head_dim 128 shapes score on the tensor cores (two passes over the keys, no rows x P table); the
     // others materialise the window-row logits S [rows][P] per unit and reduce them with CUDA-core kernels
     // (the arena's group must be the padded one: a context that runs the CUDA-core decode kernel keeps G as it is)
-    const bool tc = prefill_tc_supported(sizeof(T) == 4, D, a.Gq, R, k, P) && tc_padded_group(a.Gq) == G;
+    const bool tc = prefill_tc_supported(sizeof(T) == 4, D, a.Gq, R, k, qwin, P) && tc_padded_group(a.Gq) == G;
     const int tc_splits = tc ? prefill_tc_splits(U, P, Rw * G) : 0;
     const size_t per_unit = tc ? prefill_tc_floats_per_unit(P, Rw, G, tc_splits) : (size_t)rows * P + P;   // floats
     if (per_unit + 1 > scratch_floats) return cudaErrorInvalidConfiguration;
@@ -664,7 +664,7 @@ cudaError_t run_prefill(const DecodeArgs &a, bool f32, int D, const void *k, con
                         int padded_len)
 {
     const int Rw = P < a.R ? P : a.R;
-    const bool tc = prefill_tc_supported(f32, D, a.Gq, a.R, k, P) && tc_padded_group(a.Gq) == a.G;
+    const bool tc = prefill_tc_supported(f32, D, a.Gq, a.R, k, q_window, P) && tc_padded_group(a.Gq) == a.G;
     const size_t per_unit = (tc ? prefill_tc_floats_per_unit(P, Rw, a.G, prefill_tc_splits(a.U, P, Rw * a.G))
                                 : (size_t)Rw * a.G * P + P) * sizeof(float);
     size_t ub = ((size_t)1 << 30) / per_unit;
