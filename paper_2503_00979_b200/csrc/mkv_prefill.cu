@@ -387,28 +387,29 @@ __global__ void prefill_identity_pos_kernel(int *pos, int U, int n, int cap, Row
 // decode kernels read whole tiles and mask afterwards, so a row must hold finite numbers.  (Bound by HBM: 266 MB read
 // and written in 80 us for 256 units of 2032 slots.  Clearing the whole arena first, as two memsets, wrote every kept
 // row twice.)
+constexpr int kMaxGridY = 65535;
 template <typename T, int D>
 __global__ void prefill_gather_kernel(const T *__restrict__ k, const T *__restrict__ v, DecodeArgs a, int P, int Ps, RowMap rowmap)
 {
     constexpr int CH = D * sizeof(T) / 16;
     const int u = blockIdx.x;
-    const int idx = blockIdx.y * blockDim.x + threadIdx.x;
-    if (idx >= a.cap * CH) return;
-    const int slot = idx / CH, c = idx % CH;
     P -= rowmap(u);
     const int n = min(P, a.C + min(P, a.R));
-    uint4 *Kd = reinterpret_cast<uint4 *>(static_cast<T *>(a.K) + ((size_t)u * a.cap + slot) * D) + c;
-    uint4 *Vd = reinterpret_cast<uint4 *>(static_cast<T *>(a.V) + ((size_t)u * a.cap + slot) * D) + c;
-    if (slot >= n) {
-        *Kd = make_uint4(0, 0, 0, 0);
-        *Vd = make_uint4(0, 0, 0, 0);
-        return;
+    for (int idx = blockIdx.y * blockDim.x + threadIdx.x; idx < a.cap * CH; idx += gridDim.y * blockDim.x) {   // (more than once beyond kMaxGridY only)
+        const int slot = idx / CH, c = idx % CH;
+        uint4 *Kd = reinterpret_cast<uint4 *>(static_cast<T *>(a.K) + ((size_t)u * a.cap + slot) * D) + c;
+        uint4 *Vd = reinterpret_cast<uint4 *>(static_cast<T *>(a.V) + ((size_t)u * a.cap + slot) * D) + c;
+        if (slot >= n) {
+            *Kd = make_uint4(0, 0, 0, 0);
+            *Vd = make_uint4(0, 0, 0, 0);
+            continue;
+        }
+        const int p = a.pos[(size_t)u * a.cap + slot];
+        const uint4 *ks = reinterpret_cast<const uint4 *>(k + ((size_t)u * Ps + p) * D) + c;
+        const uint4 *vs = reinterpret_cast<const uint4 *>(v + ((size_t)u * Ps + p) * D) + c;
+        *Kd = *ks;
+        *Vd = *vs;
     }
-    const int p = a.pos[(size_t)u * a.cap + slot];
-    const uint4 *ks = reinterpret_cast<const uint4 *>(k + ((size_t)u * Ps + p) * D) + c;
-    const uint4 *vs = reinterpret_cast<const uint4 *>(v + ((size_t)u * Ps + p) * D) + c;
-    *Kd = *ks;
-    *Vd = *vs;
 }
 
 // window queries into their ring rows (row p % R); the rows that a prompt shorter than the window leaves empty are zero
@@ -435,15 +436,15 @@ __global__ void prefill_ring_vec_kernel(const T *__restrict__ qwin, DecodeArgs a
     chain_wait();
     constexpr int CH = D * sizeof(T) / 16;
     const int u = blockIdx.x, G = a.G, Gq = a.Gq, shift = rowmap(u);
-    const int idx = blockIdx.y * blockDim.x + threadIdx.x;
-    if (idx >= a.R * G * CH) return;
     P -= shift;
     const int Rw = min(P, a.R);
-    const int c = idx % CH, g = (idx / CH) % G, i = idx / (CH * G);
-    const int rslot = (P - Rw + i + shift) % a.R;
-    uint4 v = make_uint4(0, 0, 0, 0);
-    if (g < Gq && i < Rw) v = reinterpret_cast<const uint4 *>(qwin + (((size_t)u * Gq + g) * Rws + i) * D)[c];
-    reinterpret_cast<uint4 *>(static_cast<T *>(a.ring_q) + (((size_t)u * a.R + rslot) * G + g) * D)[c] = v;
+    for (int idx = blockIdx.y * blockDim.x + threadIdx.x; idx < a.R * G * CH; idx += gridDim.y * blockDim.x) {
+        const int c = idx % CH, g = (idx / CH) % G, i = idx / (CH * G);
+        const int rslot = (P - Rw + i + shift) % a.R;
+        uint4 v = make_uint4(0, 0, 0, 0);
+        if (g < Gq && i < Rw) v = reinterpret_cast<const uint4 *>(qwin + (((size_t)u * Gq + g) * Rws + i) * D)[c];
+        reinterpret_cast<uint4 *>(static_cast<T *>(a.ring_q) + (((size_t)u * a.R + rslot) * G + g) * D)[c] = v;
+    }
 }
 
 // The prompt phase on a scratch area of `scratch_floats` floats (the window-row logits S and the fused scores of
@@ -548,7 +549,7 @@ cudaError_t run_prefill_t(const DecodeArgs &a, const T *k, const T *v, const T *
     const bool waits = tc || a.nblk > 1;            // kernels with bounded waits are launched
     constexpr int CH = D * sizeof(T) / 16;
     e = ((uintptr_t)qwin & 15) == 0
-        ? launch_chained(prefill_ring_vec_kernel<T, D>, dim3(U, (R * G * CH + 255) / 256), 256, 0, stream, qwin, a, P, Rws, rowmap)
+        ? launch_chained(prefill_ring_vec_kernel<T, D>, dim3(U, min(kMaxGridY, (R * G * CH + 255) / 256)), 256, 0, stream, qwin, a, P, Rws, rowmap)
         : launch_chained(prefill_ring_kernel<T, D>, dim3(U), 256, 0, stream, qwin, a, P, Rws, rowmap);
     if (e != cudaSuccess) return e;
     *launches += 2;
@@ -589,7 +590,7 @@ cudaError_t run_prefill_t(const DecodeArgs &a, const T *k, const T *v, const T *
     const bool sums_along = sums_tc && gather_sums_supported(a, k, v);
     e = cudaSuccess;
     if (sums_along) e = launch_gather_sums(a, k, v, P, Ps, n, err_word, stream);
-    else prefill_gather_kernel<T, D><<<dim3(U, (a.cap * CH + 255) / 256), 256, 0, stream>>>(k, v, a, P, Ps, rowmap);
+    else prefill_gather_kernel<T, D><<<dim3(U, min(kMaxGridY, (a.cap * CH + 255) / 256)), 256, 0, stream>>>(k, v, a, P, Ps, rowmap);
     if (e != cudaSuccess) return e;
     if (a.norm_current && select) {
         prefill_renorm_kernel<T, D><<<dim3(Rw * G, U), kPT, 0, stream>>>(a, P, rowmap);
