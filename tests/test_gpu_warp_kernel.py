@@ -3,8 +3,9 @@ cache lengths around a 32-key tile and around a CTA's round of eight, blocks of 
 padded group, windows whose sums are not kept (they pass through the kernel 64 rows at a time), CURRENT normalisation,
 several CTAs per unit.  Tolerances are those of the lock-step comparison with the oracle."""
 import pytest
+import torch
 
-from paper_2503_00979_b200 import synth
+from paper_2503_00979_b200 import binding, synth
 from tests.parity import run_parity
 
 pytestmark = pytest.mark.gpu
@@ -34,3 +35,23 @@ def test_windows_that_pass_through_in_pieces(dtype, d, q_heads, R, norm):
 @pytest.mark.parametrize("splits", [3, 40])
 def test_several_ctas_per_unit(splits):
     _run("bf16", 64, 8, 2, 700, 20, 730, "max", splits=splits)
+
+
+# keys that are not numbers: attention over them is not a number either, wherever they lie among a warp's tiles (one key, a tile
+# and more, all of a warp's tiles, all)
+@pytest.mark.parametrize("kernel,dtype,d", [("simt", "f32", 64), ("simt", "f32", 128), ("simt", "bf16", 64), ("simt", "bf16", 128),
+                                            ("tc", "bf16", 128)])
+@pytest.mark.parametrize("C", [300, 1500])
+@pytest.mark.parametrize("first,last", [(5, 5), (64, 95), (0, 127), (0, 199)])
+def test_keys_that_are_not_numbers(kernel, dtype, d, C, first, last):
+    gen = torch.Generator(device="cuda:0")
+    gen.manual_seed(1)
+    k, v, q, q1, k1, v1 = (torch.randn(s, generator=gen, device="cuda:0").to(synth.torch_dtype(dtype))
+                           for s in ((1, 1, 1, 200, d), (1, 1, 1, 200, d), (1, 1, 4, 16, d), (1, 1, 4, d), (1, 1, 1, d), (1, 1, 1, d)))
+    k[:, :, :, first:last + 1] = float("nan")
+    mk = binding.MorphKV(1, 1, 4, 1, d, C, 16, "sum", dtype, kernel=kernel)
+    mk.prefill(k, v, q)
+    out = mk.decode_step(q1, k1, v1)
+    mk.sync()
+    assert out.isnan().all()
+    mk.close()
