@@ -343,35 +343,44 @@ __global__ void __launch_bounds__(kSelT, 2) prefill_select_kernel(const float *_
 }
 
 // The window sums (DecodeArgs::slab) of the kept slots from the window-row logits S, which the scoring without the tensor
-// cores leaves behind: one slot per thread.
-__global__ void __launch_bounds__(kPT) prefill_sums_kernel(const float *__restrict__ S, DecodeArgs a, int ub0, int P, int Rw, int Gs,
-                                                           RowMap rowmap)
+// cores leaves behind: 32 slots per CTA, the ring's blocks shared out among its warps and then run along by one of them.
+// Bound by latency and exponentials.  (One thread per slot for all blocks: FIGURES)
+constexpr int kSumSlots = 32, kSumWarps = 8, kMaxSumBlocks = 64;
+__global__ void __launch_bounds__(32 * kSumWarps) prefill_sums_kernel(const float *__restrict__ S, DecodeArgs a, int ub0, int P, int Rw, int Gs,
+                                                                      RowMap rowmap)
 {
     extern __shared__ float cs[];   // [R * Gq]
+    __shared__ float blk[kMaxSumBlocks][kSumSlots];
     const int u = ub0 + blockIdx.y, G = a.Gq, Srows = Rw * G, SP = P, shift = rowmap(u), open = open_block(P, a.R, a.bs);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     P -= shift;
     Rw = min(Rw, P);
-    for (int i = threadIdx.x; i < a.R * G; i += kPT) cs[i] = a.ring_c[((size_t)u * a.R + i / G) * Gs + i % G];
+    for (int i = threadIdx.x; i < a.R * G; i += blockDim.x) cs[i] = a.ring_c[((size_t)u * a.R + i / G) * Gs + i % G];
     __syncthreads();
-    const int k = blockIdx.x * kPT + threadIdx.x;
-    if (k >= a.cap) return;
+    const int k = blockIdx.x * kSumSlots + lane;
     const size_t at = (size_t)u * a.cap + k;
-    const int p = a.pos[at];
+    const int p = k < a.cap ? a.pos[at] : -1;
+    const int r0 = (P - Rw + shift) % a.R;                                // ring slot of the first window row
+    if (p >= 0) {
+        const float *s = S + (size_t)blockIdx.y * Srows * SP + p;
+        for (int j = warp; j < a.nblk; j += kSumWarps) {
+            float F = 0.f;
+            for (int r = j * a.bs; r < min(a.R, (j + 1) * a.bs); ++r) {
+                const int i = r - r0 + (r < r0 ? a.R : 0);                // window row in ring slot r
+                if (i >= Rw) continue;
+                float Sr = 0.f;
+                for (int g = 0; g < G; ++g) Sr += exp2f(s[(size_t)(i * G + g) * SP] - cs[r * G + g]);
+                F = fuse(a.fusion, F, Sr);
+            }
+            blk[j][lane] = F;
+        }
+    }
+    __syncthreads();
+    if (warp != 0 || k >= a.cap) return;
     a.sum_pos[at] = p;
     if (p < 0) return;                                                    // free
-    const float *s = S + (size_t)blockIdx.y * Srows * SP + p;
     float acc = 0.f, pre = 0.f;
-    for (int j = a.nblk - 1; j >= 0; --j) {
-        float F = 0.f;
-        for (int r = j * a.bs; r < min(a.R, (j + 1) * a.bs); ++r) {
-            const int i = ((r - (P - Rw + shift)) % a.R + a.R) % a.R;     // window row in ring slot r
-            if (i >= Rw) continue;
-            float Sr = 0.f;
-            for (int g = 0; g < G; ++g) Sr += exp2f(s[(size_t)(i * G + g) * SP] - cs[r * G + g]);
-            F = fuse(a.fusion, F, Sr);
-        }
-        take_block(F, j, open, a.fusion, a.slab + (size_t)u * a.nblk * a.cap + k, a.cap, true, acc, pre);
-    }
+    for (int j = a.nblk - 1; j >= 0; --j) take_block(blk[j][lane], j, open, a.fusion, a.slab + (size_t)u * a.nblk * a.cap + k, a.cap, true, acc, pre);
     a.pre[at] = pre;
 }
 
@@ -582,7 +591,8 @@ cudaError_t run_prefill_t(const DecodeArgs &a, const T *k, const T *v, const T *
             ++*launches;
         }
         if (a.nblk > 1 && !sums_tc) {
-            prefill_sums_kernel<<<dim3((a.cap + kPT - 1) / kPT, nb), kPT, R * a.Gq * sizeof(float), stream>>>(S, a, ub0, P, Rw, G, rowmap);
+            if (a.nblk > kMaxSumBlocks) return cudaErrorInvalidValue;
+            prefill_sums_kernel<<<dim3((a.cap + kSumSlots - 1) / kSumSlots, nb), 32 * kSumWarps, R * a.Gq * sizeof(float), stream>>>(S, a, ub0, P, Rw, G, rowmap);
             ++*launches;
         }
     }
