@@ -65,8 +65,8 @@ typedef enum mkv_norm { MKV_NORM_FROZEN = 0, MKV_NORM_CURRENT = 1 } mkv_norm;
 typedef enum mkv_profile { MKV_PROFILE_RECOMPUTE = 0, MKV_PROFILE_STORED = 1 } mkv_profile;
 /* which decode kernel to use: AUTO picks the tensor-core kernel when the shape allows it (bf16, head_dim 128, a
  * window of at most 2048 ring rows R * G', G' the GQA ratio rounded up to a power of two; any window with
- * MKV_PROFILE_STORED), the warp-level kernel otherwise and, with MKV_NORM_FROZEN, for launches (a step, one layer of a
- * step) too small to fill the chip */
+ * MKV_PROFILE_STORED), the warp-level kernel otherwise and, with MKV_NORM_FROZEN, for layers of a step (and small whole
+ * steps of long caches) too small to fill the chip */
 typedef enum mkv_kernel { MKV_KERNEL_AUTO = 0, MKV_KERNEL_SIMT = 1, MKV_KERNEL_TC = 2 } mkv_kernel;
 
 typedef struct mkv_ctx mkv_ctx;

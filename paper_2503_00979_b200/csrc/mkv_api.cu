@@ -133,8 +133,8 @@ bool resolve(const mkv_params *p, Shape *s, KernelKind *kind)
                                       tc_partials_per_unit(s->upl, s->cap, s->tc_grid_layer));
         s->splits = sp_all > sp_layer ? sp_all : sp_layer;
         const bool may = p->kernel == MKV_KERNEL_AUTO && !current;
-        s->simt_splits = may ? simt_small_splits(s->U, s->Gq, s->R, s->bs, s->nblk, s->cap) : 0;
-        s->simt_splits_layer = may ? simt_small_splits(s->upl, s->Gq, s->R, s->bs, s->nblk, s->cap) : 0;
+        s->simt_splits = may ? simt_small_splits(s->U, s->Gq, s->R, s->bs, s->nblk, s->cap, false) : 0;
+        s->simt_splits_layer = may ? simt_small_splits(s->upl, s->Gq, s->R, s->bs, s->nblk, s->cap, true) : 0;
         return true;
     }
     if (stored) return false;

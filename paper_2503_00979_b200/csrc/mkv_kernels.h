@@ -10,7 +10,7 @@ namespace mkv {
 cudaError_t launch_decode_simt(const DecodeArgs &a, int nsplit, bool early, bool f32, int D, cudaStream_t stream);
 int simt_block_slots(bool f32, int G, int R);      // slots per block of the ring (DecodeArgs::bs), 0: no sums are kept
 int simt_default_splits(int U, int cap);
-int simt_small_splits(int U, int G, int R, int bs, int nblk, int cap);   // CTAs per unit for a small tcgen05-context launch, 0: not small
+int simt_small_splits(int U, int G, int R, int bs, int nblk, int cap, bool layer);   // CTAs per unit for a small tcgen05-context launch, 0: not small
 
 // Coarse-grained eviction (evict_interval > 1): drops everything beyond the top C after a step that scored and
 // restores the dense prefix of C + R slots; a no-op after the other steps.  Launched after every decode step.

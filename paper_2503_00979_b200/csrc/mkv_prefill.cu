@@ -344,7 +344,8 @@ __global__ void __launch_bounds__(kSelT, 2) prefill_select_kernel(const float *_
 
 // The window sums (DecodeArgs::slab) of the kept slots from the window-row logits S, which the scoring without the tensor
 // cores leaves behind: 32 slots per CTA, the ring's blocks shared out among its warps and then run along by one of them.
-// Bound by latency and exponentials.  (One thread per slot for all blocks: FIGURES)
+// Bound by latency for few units, by L2 for many.  (One thread per slot for all blocks: a prompt of
+// 4000 tokens into 2 units of 1200 slots, d = 64, 800 rows, took 342 us, now 243; without the sums it takes 232.)
 constexpr int kSumSlots = 32, kSumWarps = 8, kMaxSumBlocks = 64;
 __global__ void __launch_bounds__(32 * kSumWarps) prefill_sums_kernel(const float *__restrict__ S, DecodeArgs a, int ub0, int P, int Rw, int Gs,
                                                                       RowMap rowmap)

@@ -22,6 +22,10 @@ pytestmark = pytest.mark.gpu
     (2, 1, 8, 2, 300, 97, "max", 1),       # blocks of 64 rows
     (2, 1, 64, 4, 200, 20, "sum", 1),      # group of 16: two blocks of 128 rows do not fit, tcgen05 kernel
     (2, 5, 16, 8, 400, 16, "max", 1),      # 40 units of four CTAs: more than the chip's SMs, tcgen05 kernel
+    (2, 1, 8, 2, 1010, 16, "sum", 0),      # whole stack: 4 units of nine CTAs
+    (2, 1, 8, 2, 1000, 16, "max", 0),      # ... of eight rounds: tcgen05 kernel
+    (2, 4, 16, 2, 1010, 16, "max", 1),     # group of 8: 8 units of nine CTAs, 72 of 74
+    (2, 5, 16, 2, 900, 16, "sum", 1),      # ... 10 units of eight, 80: tcgen05 kernel
 ])
 def test_layer_calls(layers, batch, q_heads, kv_heads, C, R, fusion, per_layer):
     w = synth.Workload("small", layers, batch, q_heads, kv_heads, 128, "bf16", C + R - 3, min(2 * R, 60) + 14, C, R, fusion, 50 + R)
