@@ -50,14 +50,16 @@ int chunk_rows(int G, int R)
 // of the ring that holds the new query's slot, whose other chunks are scored beside it.
 // Block size: bs * G' rows are scored per key on every step and once more when the block is finished, and a block's
 // slab costs 4 bytes per key beside the 512 of its K and V, so wide windows take larger blocks.  32 rows is what one
-// TMEM load brings; two blocks of 128 rows are the 256 one MMA takes.
+// TMEM load brings; two blocks of 128 rows are the 256 one MMA takes, but at G' = 16 leave room for two 32 KB stages only, so
+// narrow windows take half of that (148 units x 4096 slots, R = 16: 177 us per step with 8 slots, 174 with 4; a layer of 8 units
+// x 1056 38 and, on the warp-level kernel, which two blocks of 64 rows fit, 19).
 int tc_block_slots(int G, int R, bool current)
 {
     const int g = tc_padded_group(G);
     if (current) return tc_ring_chunks(G, R) > 1 ? chunk_rows(G, R) / g : R;
     int bs = R <= 96 ? 8 : R <= 384 ? 16 : 32;
     bs = std::max(bs, 32 / g);
-    bs = std::min(bs, 128 / g);
+    bs = std::min(bs, (R <= 96 ? 64 : 128) / g);
     return bs < R ? bs : R;
 }
 

@@ -20,7 +20,9 @@ pytestmark = pytest.mark.gpu
     (1, 1, 16, 1, 600, 12, "max", 0),      # group of 16, whole stack of one layer
     (2, 2, 4, 4, 500, 64, "sum", 2),       # MHA
     (2, 1, 8, 2, 300, 97, "max", 1),       # blocks of 64 rows
-    (2, 1, 64, 4, 200, 20, "sum", 1),      # group of 16: two blocks of 128 rows do not fit, tcgen05 kernel
+    (2, 1, 64, 4, 200, 20, "sum", 1),      # group of 16: blocks of four slots
+    (2, 1, 32, 2, 300, 100, "max", 1),     # group of 16: two blocks of 128 rows do not fit, tcgen05 kernel
+    (3, 1, 48, 4, 1000, 9, "sum", 1),      # group of 12 -> 16, four units of eight CTAs, a last block of one slot
     (2, 5, 16, 8, 400, 16, "max", 1),      # 40 units of four CTAs: more than the chip's SMs, tcgen05 kernel
     (2, 1, 8, 2, 1010, 16, "sum", 0),      # whole stack: 4 units of nine CTAs
     (2, 1, 8, 2, 1000, 16, "max", 0),      # ... of eight rounds: tcgen05 kernel
