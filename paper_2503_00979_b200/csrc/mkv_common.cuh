@@ -357,10 +357,10 @@ __device__ void renormalise_after_eviction(const DecodeArgs &a, int u, int e_slo
 // `sm` needs kFinalizeSmemFloats floats of shared memory, 8-byte aligned.  GT is the GQA
 // group size when known at compile time (0: use a.G); it lets the loads of a round be
 // issued together.  Loads are batched so that the whole epilogue costs a handful of L2
-// round trips.  `moved`: a slot of the unit holds another token than its window sums belong to.
+// round trips.  (Of the tensor-core kernel's modes only the chunked window ends here, which keeps no window sums.)
 template <typename T, int D, int GT>
 __device__ void finalize_unit(const DecodeArgs &a, int u, long long t, int n, int active, bool evict, float *sm,
-                              int tid, int nthr, int bar_id, int shift = 0, bool moved = false)
+                              int tid, int nthr, int bar_id, int shift = 0)
 {
     const int lane = tid & 31, warp = tid >> 5, nwarp = nthr >> 5;
     const int G = GT > 0 ? GT : a.G;
@@ -435,10 +435,6 @@ __device__ void finalize_unit(const DecodeArgs &a, int u, long long t, int n, in
     int *pos = a.pos + (size_t)u * a.cap;
     float *F = a.F + (size_t)u * a.cap;
     int e_slot = n, e_pos = -1;
-    if (moved) {
-        resum_moved<T, D>(a, u, 0, n, ring_slot(t, a.R), F, warp, nwarp, lane);
-        group_sync(bar_id, nthr);
-    }
     if (evict) {
         const float *sn = a.s_new + (size_t)u * G * a.cap;
         const long long thr = t - shift - a.R;        // positions are the row's own; ring slots follow t
@@ -530,7 +526,6 @@ __device__ void finalize_unit(const DecodeArgs &a, int u, long long t, int n, in
     if (tid < G) a.ring_c[((size_t)u * a.R + rs) * G + tid] = cnew[tid];
     if (tid == 0) {
         pos[e_slot] = (int)(t - shift);
-        if (a.nblk > 1) a.sum_pos[(size_t)u * a.cap + e_slot] = (int)(t - shift);
         a.evicted_pos[u] = e_pos;
         a.ticket[u] = 0;
     }

@@ -138,6 +138,9 @@ using Walk = WalkT<false>;
 // than kMergeTiles / 2 tiles longer: every unit is then cut into equal parts of its own and never shared by more CTAs than
 // it has parts (8 at most, what the fast epilogue merges), or is one CTA's alone, for which kMergeTiles are paid.
 // (64 units of 8 tiles in 128 parts 17.4 us per step against 21.1; 32 units of 16 tiles in 128 parts 18.8 against 22.9.)
+// Few units always get the 8 parts, although some SMs then stay idle: 8 units of 32 / 128 / 512 tiles take 19.2 / 46.5 / 157 us in
+// 8 parts and 24 / 45 / 139 in equal shares of 148 CTAs, whose 18 partials are merged first; 1 unit of 128 44 against 67; 16 of 512
+// 173 against 176.
 inline int sched_grid(int U, int cap, int splits_hint, int n_sm)
 {
     const long long ntiles = (cap + kSchedTile - 1) / kSchedTile, total = (long long)U * ntiles;

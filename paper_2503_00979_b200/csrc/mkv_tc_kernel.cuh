@@ -320,6 +320,56 @@ __device__ void finalize_fast(const DecodeArgs &a, int u, long long t, int n, in
     }
 }
 
+// Merges the partials of all CTAs of a unit into the first one, for units that more CTAs share than the epilogue merges by
+// itself.  `sm`: kMaxGroup floats.  (us per step with the general epilogue in its place -> now, 4 heads: 8 units x 16384 slots in 18
+// parts each 127 -> 44; 19 units x 16384, which share 148 CTAs evenly, 140 -> 57.)
+template <int G>
+__device__ __noinline__ void merge_partials(const DecodeArgs &a, int u, int nseg, float *sm, int tid, int bar_id)
+{
+    float *pml = a.part_ml + (size_t)u * a.splits * G * 2, *po = a.part_o + (size_t)u * a.splits * G * kD;
+    float m = -INFINITY, l = 0.f;
+    if (tid < G) {
+        for (int s0 = 0; s0 < nseg; s0 += 8) {               // eight loads in flight at a time
+            float pm[8], pl[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const bool ok = s0 + i < nseg;
+                pm[i] = ok ? __ldcg(pml + ((s0 + i) * G + tid) * 2) : -INFINITY;
+                pl[i] = ok ? __ldcg(pml + ((s0 + i) * G + tid) * 2 + 1) : 0.f;
+            }
+            float mn = m;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) mn = fmaxf(mn, pm[i]);
+            const float r = mn == -INFINITY ? 0.f : mn;
+            l *= exp2f(m - r);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) l += pl[i] * exp2f(pm[i] - r);
+            m = mn;
+        }
+        sm[tid] = m == -INFINITY ? 0.f : m;
+    }
+    group_sync(bar_id, kGroupThreads);
+    for (int g = 0; g < G; ++g) {
+        const float r = sm[g];
+        float x = 0.f;
+        for (int s0 = 0; s0 < nseg; s0 += 8) {
+            float pm[8], pv[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const bool ok = s0 + i < nseg;
+                pm[i] = ok ? __ldcg(pml + ((s0 + i) * G + g) * 2) : -INFINITY;
+                pv[i] = ok ? __ldcg(po + ((s0 + i) * G + g) * kD + tid) : 0.f;
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) x += pv[i] * exp2f(pm[i] - r);
+        }
+        po[g * kD + tid] = x;
+    }
+    group_sync(bar_id, kGroupThreads);                       // every maximum has been read
+    if (tid < G) { pml[2 * tid] = m; pml[2 * tid + 1] = l; }
+    group_sync(bar_id, kGroupThreads);
+}
+
 // MODE: which ring rows a step scores (TcMode).  RAGGED: the batch rows have their own fills and position offsets
 // (DecodeArgs::row_n); compiled separately so that the uniform kernel carries none of it.
 template <int G, int FUSION, int NG, int MODE, bool RAGGED>
@@ -1002,11 +1052,9 @@ decode_tc_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ C
                     group_sync(kEpiBar, kGroupThreads);
                     if (*flag) {
                         moved |= *flag > 1;
-                        if (ncta <= 8 && ncta * G * 2 <= 256)
-                            finalize_fast<G, false>(a, u, t, us.n, ncta, us.evict, fin_sm, etid, kEpiBar, o, nullptr, RAGGED ? us.shift : 0, rows, moved);
-                        else
-                            finalize_unit<__nv_bfloat16, kD, G>(a, u, t, us.n, ncta, us.evict, fin_sm, etid, kGroupThreads, kEpiBar,
-                                                                RAGGED ? us.shift : 0, moved);
+                        if (ncta > 8) merge_partials<G>(a, u, ncta, fin_sm, etid, kEpiBar);
+                        finalize_fast<G, false>(a, u, t, us.n, ncta > 8 ? 1 : ncta, us.evict, fin_sm, etid, kEpiBar, o, nullptr, RAGGED ? us.shift : 0,
+                                                rows, moved);
                     }
                 }
                 if (BLOCKS && etid == 0) *moved_flag = 0;

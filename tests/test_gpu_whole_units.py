@@ -23,3 +23,13 @@ def test_shares(layers, q_heads, kv_heads, P, C, R, fusion):
     w = synth.Workload("shares", layers, 1, q_heads, kv_heads, 128, "bf16", P, steps, C, R, fusion, 70 + layers)
     rep = run_parity(w, steps=steps, n_units=5, kernel="tc", check_F_every=7)
     assert rep.kernel == "tc" and rep.evictions > 0
+
+
+# units shared by more CTAs than the epilogue merges by itself: nine and more segments of one to three tiles, the last with a
+# few keys, while the cache fills and when it evicts
+@pytest.mark.parametrize("splits", [9, 13, 26])
+@pytest.mark.parametrize("q_heads,R,fusion", [(2, 33, "sum"), (8, 16, "max"), (14, 30, "sum"), (32, 9, "max")])
+def test_many_segments(splits, q_heads, R, fusion):
+    w = synth.Workload("segments", 2, 1, q_heads, 2, 128, "bf16", 3200, 30, 3220 - R, R, fusion, 90 + R)
+    rep = run_parity(w, steps=w.steps, n_units=4, kernel="tc", splits=splits, check_F_every=5)
+    assert rep.kernel == "tc" and rep.evictions > 0
