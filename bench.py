@@ -314,7 +314,7 @@ def secondary_record(w: synth.Workload, W: int, K: int, dev, per_layer: bool = F
     peak, _ = measured_peak_gbs()
     achieved = bytes_step / (ms / K * 1e-3) / 1e9
     rec = {"workload": w.name, "prompt_len": P, "cached_tokens_per_unit": n_steady, "steps": K, "warmup": W,
-           "ms_per_step": ms / K, "tokens_per_s": w.batch * K / (ms * 1e-3), "kernel": mk.kernel_name,
+           "ms_per_step": ms / K, "tokens_per_s": w.batch * K / (ms * 1e-3), "kernel": mk.step_kernel(per_layer),
            "gpu_launches": int(mk.launch_count - launches0),
            "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak, "nominal_peak": NOMINAL_HBM_GBS,
                         "frac_of_nominal": achieved / NOMINAL_HBM_GBS,
@@ -475,7 +475,7 @@ def run_ours(args, w):
     # ---- arm 2: host buffers through the C ABI, copies inside the timed region ----
     if args.no_e2e:
         if rank == 0:
-            print(json.dumps({"ms_per_step": ms / K, "kernel": mk.kernel_name, "note": "profiling run, no JSON contract"}))
+            print(json.dumps({"ms_per_step": ms / K, "kernel": mk.step_kernel(), "note": "profiling run, no JSON contract"}))
         mk.close()
         return
     hq = qs[W + K:].cpu().pin_memory(); hk = kn[W + K:].cpu().pin_memory(); hv = vn[W + K:].cpu().pin_memory()
@@ -509,7 +509,7 @@ def run_ours(args, w):
             "config": {"workload": w.name, "layers": w.layers, "batch": w.batch, "n_q_heads": w.n_q_heads,
                        "n_kv_heads": w.n_kv_heads, "head_dim": w.head_dim, "C": w.C, "R": w.R, "fusion": w.fusion,
                        "prompt_len": P, "evict_interval": T, "cached_tokens_per_unit": n_steady, "units_per_gpu": w.units,
-                       "kernel": mk.kernel_name, "profile_mode": args.profile, "parallelism": f"replicas x{world}",
+                       "kernel": mk.step_kernel(), "profile_mode": args.profile, "parallelism": f"replicas x{world}",
                        "l2": "inputs larger than L2: each step streams the whole K/V cache "
                              f"({bytes_step / 1e6:.0f} MB per step against 126 MB of L2)"},
             "clocks": clocks.summary(),
@@ -518,8 +518,8 @@ def run_ours(args, w):
             "gpu_launches": int(launches),
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak, "nominal_peak": NOMINAL_HBM_GBS,
                         "frac_of_nominal": achieved / NOMINAL_HBM_GBS,
-                         "traffic": measured_traffic(w.name) if mk.kernel_name == "tc" and args.prompt_len == 0 and T == 1 else None,
-                         "peak_source": peak_src, "kernel": f"decode_{mk.kernel_name}",
+                         "traffic": measured_traffic(w.name) if mk.step_kernel() == "tc" and args.prompt_len == 0 and T == 1 else None,
+                         "peak_source": peak_src, "kernel": f"decode_{mk.step_kernel()}",
                          "algorithmic_bytes_per_launch": bytes_step},
         }
         if world == 1 and args.also and w.name == "c1" and args.prompt_len == 0 and T == 1 and not (args.layers or args.batch):

@@ -246,9 +246,13 @@ mkv_status mkv_sync(mkv_ctx *ctx, void *stream);
 const char *mkv_last_error(const mkv_ctx *ctx);
 
 /* Counters for reporting: kernels launched by this context so far, and the name of the
- * decode kernel in use ("simt" or "tc"). */
+ * decode kernel the context is laid out for ("simt" or "tc"). */
 uint64_t mkv_launch_count(const mkv_ctx *ctx);
 const char *mkv_kernel_name(const mkv_ctx *ctx);
+
+/* The decode kernel that a call of this context launches: small launches of a "tc" context run the
+ * warp-level kernel (MKV_KERNEL_AUTO).  per_layer: 0 for mkv_decode_step, 1 for mkv_decode_step_layer. */
+const char *mkv_step_kernel_name(const mkv_ctx *ctx, int per_layer);
 
 #ifdef __cplusplus
 }

@@ -29,7 +29,7 @@ EXPORTS = [
     "mkv_default_params", "mkv_workspace_bytes", "mkv_create", "mkv_create_ex", "mkv_destroy", "mkv_reset", "mkv_prefill",
     "mkv_prefill_static", "mkv_prefill_ragged", "mkv_row_state",
     "mkv_decode_step", "mkv_decode_step_layer", "mkv_decode_steps", "mkv_decode_step_host", "mkv_cache_view", "mkv_sync", "mkv_last_error",
-    "mkv_launch_count", "mkv_kernel_name",
+    "mkv_launch_count", "mkv_kernel_name", "mkv_step_kernel_name",
 ]
 
 
@@ -95,6 +95,8 @@ def lib() -> C.CDLL:
         L.mkv_launch_count.restype = C.c_uint64
         L.mkv_kernel_name.argtypes = [vp]
         L.mkv_kernel_name.restype = C.c_char_p
+        L.mkv_step_kernel_name.argtypes = [vp, ip]
+        L.mkv_step_kernel_name.restype = C.c_char_p
         _lib = L
     return _lib
 
@@ -203,6 +205,10 @@ def mkv_launch_count(ctx) -> int:
 
 def mkv_kernel_name(ctx) -> str:
     return lib().mkv_kernel_name(ctx).decode()
+
+
+def mkv_step_kernel_name(ctx, per_layer: bool) -> str:
+    return lib().mkv_step_kernel_name(ctx, int(per_layer)).decode()
 
 
 # ---- convenience holder ---------------------------------------------------------------------
@@ -343,3 +349,7 @@ class MorphKV:
     @property
     def kernel_name(self) -> str:
         return mkv_kernel_name(self.ctx)
+
+    def step_kernel(self, per_layer: bool = False) -> str:
+        """The kernel that a decode call launches: small launches of a "tc" context run the warp-level one."""
+        return mkv_step_kernel_name(self.ctx, per_layer)

@@ -866,4 +866,9 @@ uint64_t mkv_launch_count(const mkv_ctx *ctx) { return ctx ? ctx->launches + (ct
 
 const char *mkv_kernel_name(const mkv_ctx *ctx) { return (ctx && ctx->kind == kKindTc) ? "tc" : "simt"; }
 
+const char *mkv_step_kernel_name(const mkv_ctx *ctx, int per_layer)
+{
+    return (ctx && (per_layer ? ctx->s.simt_splits_layer : ctx->s.simt_splits) == 0) ? "tc" : "simt";
+}
+
 }  // extern "C"

@@ -40,7 +40,8 @@ class ParityReport:
     min_rel_gap: float = float("inf")   # smallest relative gap between the oracle's C-th and (C+1)-th score
     max_F_rel_err: float = 0.0
     F_compared: int = 0
-    kernel: str = ""
+    kernel: str = ""                    # what the context is laid out for
+    step_kernel: str = ""               # what its launches run: of a whole step, or of a layer (per_layer != 0)
 
 
 def near_tie(a: float, b: float) -> bool:
@@ -134,7 +135,7 @@ def run_parity(w: synth.Workload, steps: int, units=None, n_units: int = 8, chun
     mk = binding.MorphKV(w.layers, w.batch, w.n_q_heads, w.n_kv_heads, d, C_, R, w.fusion, w.dtype, kernel=kernel,
                          splits=splits, device=device, full_layers=full_layers, max_tokens=max_tokens, norm=norm,
                          **ctx_kwargs)
-    rep.kernel = mk.kernel_name
+    rep.kernel, rep.step_kernel = mk.kernel_name, mk.step_kernel(per_layer != 0)
     C_of = {l: (max_tokens - R if l < full_layers else C_) for l in range(w.layers)}     # distant tokens kept per layer
     tol = TOL_OUT[w.dtype]
     Rw = min(R, P)
@@ -313,7 +314,7 @@ def run_parity_coarse(w: synth.Workload, T: int, steps: int, n_units: int = 4, k
     rep = ParityReport()
     mk = binding.MorphKV(w.layers, w.batch, w.n_q_heads, w.n_kv_heads, d, C_, R, w.fusion, w.dtype, evict_interval=T,
                          kernel=kernel, device=device)
-    rep.kernel = mk.kernel_name
+    rep.kernel, rep.step_kernel = mk.kernel_name, mk.step_kernel()
     tol = TOL_OUT[w.dtype]
     Rw = min(R, P)
     k32, v32 = st.kv(np.arange(P))
@@ -396,7 +397,7 @@ def run_parity_ragged(w: synth.Workload, prompt_lens, steps: int, kernel: str = 
     rep = ParityReport()
     mk = binding.MorphKV(L, B, w.n_q_heads, Hkv, d, C_, R, w.fusion, w.dtype, kernel=kernel, device=device, norm=norm,
                          full_layers=full_layers, max_tokens=max_tokens)
-    rep.kernel = mk.kernel_name
+    rep.kernel, rep.step_kernel = mk.kernel_name, mk.step_kernel(per_layer != 0)
     C_of = {l: (max_tokens - R if l < full_layers else C_) for l in range(L)}
     tol = TOL_OUT[w.dtype]
     k32, v32 = st.kv(np.arange(Pm))                       # [L,B,Hkv,Pm,d]

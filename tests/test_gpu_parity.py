@@ -894,3 +894,17 @@ def test_stored_profile_mode_with_per_layer_calls_and_reset():
     p.profile_mode = binding.PROFILE["stored"]
     st, h = binding.mkv_create_ex(p)
     assert st == binding.UNSUPPORTED and h is None
+
+
+# the tcgen05 kernel on shapes whose layer calls, or long caches, the automatic choice gives to the warp-level kernel
+@pytest.mark.parametrize("q_heads,R,C,P,per_layer,profile,T", [(8, 24, 200, 300, 2, "stored", 1), (8, 70, 400, 500, 1, "recompute", 1),
+                                                               (14, 12, 120, 140, 2, "recompute", 1), (8, 16, 1200, 1300, 0, "stored", 1),
+                                                               (14, 30, 1100, 1000, 0, "recompute", 1), (8, 32, 250, 330, 0, "recompute", 5)])
+def test_tc_kernel_where_small_launches_go_elsewhere(q_heads, R, C, P, per_layer, profile, T):
+    w = synth.Workload("tc_small", 2, 1, q_heads, 2, 128, "bf16", P, max(0, C + R - P) + 40, C, R, "sum", 88 + R)
+    if T > 1:
+        rep = run_parity_coarse(w, T, steps=w.steps, n_units=4, kernel="tc")
+    else:
+        rep = run_parity(w, steps=w.steps, n_units=4, kernel="tc", per_layer=per_layer, profile=profile, check_F_every=5)
+    _report(rep)
+    assert rep.step_kernel == "tc" and rep.evictions > 0

@@ -21,3 +21,11 @@ def test_rows_ending_at_edges(lens, C, R, q_heads, fusion, kernel):
     w = synth.Workload("ragged_edges", 1, len(lens), q_heads, kv, 128, "bf16", 0, 4, C, R, fusion, 31 + len(lens))
     rep = run_parity_ragged(w, lens, steps=4, kernel=kernel)
     assert rep.evictions > 0 and rep.kernel == ("tc" if kernel == "auto" else "simt")
+
+
+# the tcgen05 kernel's layer calls and its shares cut between units (more units than SMs), which small launches do not reach
+@pytest.mark.parametrize("layers,per_layer", [(2, 1), (20, 0)])
+def test_rows_on_the_tensor_core_kernel(layers, per_layer):
+    w = synth.Workload("ragged_tc", layers, 4, 8, 2, 128, "bf16", 0, 12, 200, 16, "max", 33)
+    rep = run_parity_ragged(w, [300, 40, 210, 129], steps=12, kernel="tc", per_layer=per_layer)
+    assert rep.evictions > 0 and rep.step_kernel == "tc"

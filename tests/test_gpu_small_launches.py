@@ -33,6 +33,9 @@ def test_layer_calls(layers, batch, q_heads, kv_heads, C, R, fusion, per_layer):
     w = synth.Workload("small", layers, batch, q_heads, kv_heads, 128, "bf16", C + R - 3, min(2 * R, 60) + 14, C, R, fusion, 50 + R)
     rep = run_parity(w, steps=w.steps, n_units=4, per_layer=per_layer, check_F_every=5)
     assert rep.kernel == "tc" and rep.evictions > 0
+    units, rounds, wide = (layers if per_layer == 0 else 1) * batch * kv_heads, -(-(C + R) // 128), q_heads // kv_heads > 4
+    small = units * min(rounds, 16) <= (74 if wide else 148) and (per_layer != 0 or rounds > 8)
+    assert rep.step_kernel == ("simt" if small and (q_heads // kv_heads, R) != (16, 100) else "tc")
 
 
 def test_coarse_grained_and_ragged():
