@@ -230,16 +230,11 @@ __device__ __forceinline__ void group_sync(int bar_id, int nthr)
     asm volatile("barrier.sync %0, %1;" ::"r"(bar_id), "r"(nthr) : "memory");
 }
 
-// The block of the ring that is open before the step at position t, and whether that step opens the next one (it then
-// scores block `open` for good: see DecodeArgs::slab).
+// The ring slot of position t, and the block of the ring that is open before the step at t (DecodeArgs::slab).
 // (Positions fit in 32 bits and start at 1, a prompt's length; 64-bit divisions would take most of a microsecond at the start
 // of every launch.)
 __host__ __device__ inline int ring_slot(long long t, int R) { return (int)((unsigned)t % (unsigned)R); }
 __host__ __device__ inline int open_block(long long t, int R, int bs) { return ring_slot(t - 1, R) / bs; }
-__host__ __device__ inline bool step_opens_block(long long t, int R, int bs, int nblk)
-{
-    return nblk > 1 && ring_slot(t, R) % bs == 0;
-}
 
 // The fused score S of ring block j joins the sums of one key; blocks come in descending order, acc and pre run along.
 __device__ __forceinline__ void take_block(float S, int j, int open, int fusion, float *slab, size_t cap, bool valid,

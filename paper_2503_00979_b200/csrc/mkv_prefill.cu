@@ -184,7 +184,8 @@ __global__ void __launch_bounds__(kPT) prefill_fuse_kernel(const float *__restri
 //
 // One CTA per unit; a warp owns a run of the keys, so that the compaction needs one scan over the warps and no barrier per
 // round.  The digits are 12 bits wide: the first takes sign, exponent and three bits of the mantissa, after which a bucket mostly holds a few hundredths of the keys; those move to a list in shared memory, on which the other digits
-// work.  The keys are read from memory once if a warp's run fits in its registers (up to 8192 keys), else three times.
+// work.  The keys are read from memory once if a warp's run fits in its registers (up to 8192 keys), else once per digit
+// until the bucket fits the list (the first digit as a rule; more where many scores tie), and twice more.
 // Bound by latency for short prompts, by L2 for long ones.  With 8-bit digits, every one of them over all keys, and a
 // compaction of 1024 keys per round between barriers: 31 us for 256 units of 6112 keys and 306 us for 131040, now 17 and 101.
 constexpr int kSelT = 1024;      // threads of the selection kernel

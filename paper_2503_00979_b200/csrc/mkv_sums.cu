@@ -6,7 +6,7 @@
 // a register on the way.  It has the decode kernel's orientation (keys in the TMEM lanes, ring rows as the N operand,
 // up to 256 at a time) and the CTA layout of the prompt phase's scoring passes: warps 0-3 and 6-9 are two consumer
 // groups on alternate key tiles and accumulator buffers, warp 4 feeds K tiles with TMA, warp 5 issues the MMAs.
-// Bound by the kept keys' bytes and R*G exponentials per key (256 units of 2048 slots, 128 rows: 38 us).
+// Bound by the kept keys' bytes and R*G exponentials per key (256 units of 2032 slots, 128 rows: 44 us).
 #include <string.h>
 
 #include "mkv_common.cuh"

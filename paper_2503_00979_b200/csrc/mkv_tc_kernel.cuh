@@ -34,7 +34,7 @@
 // ends in a warp-level sync.
 //
 // Why the kept sums: with all R*G rows scored on every step the compute warps' exponentials, not HBM, set the pace
-// of wide windows (R*G = 256: 1114 us per step of 2048 units x 4064 slots, 726 with the sums; R*G = 800: 465 us, 111)
+// of wide windows (R*G = 256: 1114 us per step of 2048 units x 4064 slots, 695 with the sums; R*G = 800: 465 us, 97)
 // and nearly did at R*G = 128.  Per key and step 32 rows and 8 bytes of sums take the place of R*G rows.
 #pragma once
 
@@ -464,7 +464,7 @@ decode_tc_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ C
     const int NCe = MC ? (evict ? geo.nc : 1) : 1;               // chunks walked per unit on this step
     const int c_main = MC || BLOCKS ? rs_new / a.bs : 0;
     const int rs_loc = MC || BLOCKS ? rs_new - c_main * a.bs : rs_new;   // the new query's slot inside its chunk or block
-    const bool fold = BLOCKS && a.nblk > 1 && rs_loc == 0;       // step_opens_block()
+    const bool fold = BLOCKS && a.nblk > 1 && rs_loc == 0;       // the step opens a block
     const int j_old = c_main > 0 ? c_main - 1 : a.nblk - 1;      // fold: the finished block, open_block()
     const int QB = BLOCKS ? geo.qbox : RGP;                      // ring rows per operand box
     const int NR = fold ? 2 * QB : QB;                           // ring rows of this step's operand (MMA N)
