@@ -47,7 +47,7 @@ NOMINAL_HBM_GBS = 7700.0
 
 # DRAM bytes per launch of the dominant kernel (dram__bytes_read.sum + dram__bytes_write.sum from one ncu
 # capture of a launch of that workload), valid only for the kernel sources it was taken with.
-_TRAFFIC = {"c1": {"bytes": 284.9e6, "sources_sha256": "5687faec5ff06122cd7ad7a0975de33c1dc8eefe2ac91bbdd3f1f3cf9f928e57"}}
+_TRAFFIC = {"c1": {"bytes": 280.1e6, "sources_sha256": "82b86ae45678e73d7c3be48b7d9c89225dd0edb42e24b444b9951149eb46b690"}}
 
 
 def measured_traffic(workload: str):
