@@ -284,7 +284,8 @@ mkv_status launch_step(mkv_ctx *ctx, int layer, const void *q, const void *k, co
     // A view of the cache has been handed out since the last step, and its holder may have rearranged the slots (their
     // order is free).  A step that is being recorded does not know when it will be replayed, and always looks.
     const bool capturing = is_capturing(stream);
-    bool viewed = false;
+    bool viewed = false, behind_holder = false;
+    for (int l = 0; layer == 0 && l < ctx->s.layers; ++l) behind_holder |= ctx->viewed[l] != 0;
     for (int l = layer < 0 ? 0 : layer; l < (layer < 0 ? ctx->s.layers : layer + 1); ++l) {
         viewed |= ctx->viewed[l] != 0;
         if (!capturing) ctx->viewed[l] = 0;
@@ -304,10 +305,10 @@ mkv_status launch_step(mkv_ctx *ctx, int layer, const void *q, const void *k, co
     }
     // A launch may run ahead of the end of the one before it in its stream if that belongs to another layer: what this layer
     // holds was then written before that one let this one start.  Not so behind a launch of the same layer (layers on streams of
-    // their own), behind the state copy above, or behind a view's holder's own work on the slots.  (cudaStreamPerThread names
-    // another stream in every thread.)
+    // their own), behind the state copy above, or (a step's first layer) behind a view's holder's own work on the slots.
+    // (cudaStreamPerThread names another stream in every thread.)
     const bool early = layer >= 0 && ctx->last_layer >= 0 && ctx->last_layer != layer && ctx->last_stream == stream &&
-                       stream != cudaStreamPerThread && ctx->last_capturing == capturing && ctx->launches == before && !viewed;
+                       stream != cudaStreamPerThread && ctx->last_capturing == capturing && ctx->launches == before && !behind_holder;
     ctx->last_layer = layer;
     ctx->last_stream = stream;
     ctx->last_capturing = capturing;
@@ -814,8 +815,9 @@ mkv_status mkv_decode_step_host(mkv_ctx *ctx, const void *q_host, const void *k_
     const size_t qb = (size_t)ctx->s.U * ctx->s.Gq * ctx->s.D * ctx->s.es, kb = (size_t)ctx->s.U * ctx->s.D * ctx->s.es;
     char *b = ctx->base;
     // Pinned host buffers are reachable from the device: the tensor-core kernel then reads q, k_new, v_new and
-    // writes `out` in place over the interconnect (a few hundred KB per step, read once or twice), which saves
-    // four copy launches per step.  (One launch that copies the inputs ahead of the kernel costs more than it saves: 48 instead
+    // writes `out` in place over the interconnect (a few hundred KB per step; read once or twice, in small launches by each of the
+    // up to 16 CTAs of a unit: 27 to 34 us per token for 1 to 37 units on either kernel), which saves four copy launches per
+    // step.  (One launch that copies the inputs ahead of the kernel costs more than it saves: 48 instead
     // of 42 us per token for 112 units of 7 heads, 98 instead of 82 for 448.)  Anything else goes through the staging buffers.
     if (ctx->kind == kKindTc) {
         const void *hp[4] = {q_host, k_new_host, v_new_host, out_host};

@@ -505,7 +505,7 @@ decode_simt_kernel(const __grid_constant__ DecodeArgs a, const int nsplit, const
                     st_w[g * kKT + lane] = s;
                     if (lane == 0) { fac[g] = f; mref[g] = mn == -INFINITY ? 0.f : mn; }
                 } else {
-                    const float p = valid ? exp2f(s - (mn == -INFINITY ? 0.f : mn)) : 0.f;      // (NaN stays NaN)
+                    const float p = mn == -INFINITY ? (s == -INFINITY ? 0.f : s) : exp2f(s - mn);        // (s -inf or NaN: NaN stays)
                     if (lane < kKT) st_w[g * kKT + lane] = p;
                     lsum[g] = lsum[g] * f + p;
                     if (f != 1.f && !first_tile)
@@ -644,10 +644,12 @@ decode_simt_kernel(const __grid_constant__ DecodeArgs a, const int nsplit, const
         float o = 0.f, l = 0.f;
 #pragma unroll
         for (int w = 0; w < kWarps; ++w) {
-            const float mw = wml[(w * GP + g) * 2];
-            const float f = mw > -INFINITY ? exp2f(mw - m) : 0.f;        // (a warp without keys, or with keys that are all NaN: 0 * NaN stays)
-            o += reinterpret_cast<const float *>(smem + L::stages + w * L::stage)[idx] * f;
-            l += wml[(w * GP + g) * 2 + 1] * f;
+            const float mw = wml[(w * GP + g) * 2], lw = wml[(w * GP + g) * 2 + 1];
+            if (lw != 0.f) {                                             // a warp with keys (NaN if they are not numbers)
+                const float f = exp2f(mw - m);
+                o += reinterpret_cast<const float *>(smem + L::stages + w * L::stage)[idx] * f;
+                l += lw * f;
+            }
         }
         const int r = idx / slice, at = sp * slice + idx - r * slice;
         if (nsplit == 1) co[at] = o; else st_cluster(mapa(smem_u32(co + at), r), o);
