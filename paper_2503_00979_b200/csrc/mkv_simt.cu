@@ -859,9 +859,11 @@ int simt_block_slots(bool f32, int G, int R)
 // Whether a launch over U units of a tcgen05 context is better off here, as clusters of as many CTAs as a unit has rounds of
 // tiles: CTAs per unit, or 0.  (us per call, tcgen05 kernel -> here; R * G' = 128)
 // - A layer's call starts ahead of the end of the one before it, so its chain of latencies is what counts: 8 units x 96 / 512 /
-//   2048 / 4096 slots at G' = 4: 8.1 -> 7.2 / 11.0 -> 7.8 / 14.9 -> 10.9 / 20.0 -> 16.8.  That needs the next layer's CTAs to find
-//   room beside this one's: one CTA per SM, or one per two SMs where a CTA takes a whole SM (G' > 4: 8 units x 1056, 72 CTAs:
-//   19.9 -> 13.3; 16 x 1056, 144 CTAs: 20.7 -> 26.6, as clusters of 9 do not all fit either).
+//   2048 / 4096 slots at G' = 4: 8.1 -> 7.2 / 11.0 -> 7.8 / 14.9 -> 10.9 / 20.0 -> 16.8.  The next layer's CTAs find room beside
+//   this one's up to one CTA per SM.  At G' > 4 a CTA takes a whole SM: half as many leave that room (8 units x 1056, 72 CTAs:
+//   19.9 -> 13.3), and more are worth it from 4 tiles per unit on while all clusters are resident at once: on the chip's seven
+//   larger groups of SMs and the smaller eighth (12 units of 8 CTAs 19.6 -> 15.3, 14: 19.7 -> 16.1, 22 of 6: 19.7 -> 18.1; not so 16 of
+//   8: 20.0 -> 26.5, 18 of 7: 19.9 -> 27.7, 16 of 9: 20.7 -> 26.6, 64 of 2: 14.4 -> 17.3).
 // - A launch of the whole stack starts from nothing here, while the tcgen05 kernel sets itself up ahead of its wait and gives
 //   units of up to eight tiles a CTA per tile: 8 units x 256 / 512 / 768: 9.2 -> 13.0 / 11.2 -> 12.9 / 12.2 -> 12.9.  Longer ones
 //   it merges from several tiles per CTA, or more partials: 1056 / 2048: 13.8 -> 13.0 / 14.7 -> 14.0 (G' = 8: 20.0 -> 17.3 at 1056).
@@ -871,7 +873,8 @@ int simt_small_splits(int U, int G, int R, int bs, int nblk, int cap, bool layer
     if ((nblk > 1 ? 2 : 1) * bs * g > SimtSmem<__nv_bfloat16, 128, 1>::rows) return 0;
     const int rounds = (cap + kRound - 1) / kRound, s = rounds < kMaxCluster ? rounds : kMaxCluster;
     if (!layer && rounds <= 8) return 0;
-    return (long long)U * s <= (g > 4 ? 74 : 148) && rounds <= 2 * kMaxCluster ? s : 0;
+    const bool fits = (long long)U * s <= (g > 4 ? 74 : 148) || (layer && g > 4 && s >= 4 && U <= 18 / s * 7 + 11 / s);
+    return fits && rounds <= 2 * kMaxCluster ? s : 0;
 }
 
 // CTAs per unit: enough to fill the chip (two CTAs per SM), at least one round of tiles each.

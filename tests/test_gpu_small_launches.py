@@ -27,14 +27,17 @@ pytestmark = pytest.mark.gpu
     (2, 1, 8, 2, 1010, 16, "sum", 0),      # whole stack: 4 units of nine CTAs
     (2, 1, 8, 2, 1000, 16, "max", 0),      # ... of eight rounds: tcgen05 kernel
     (2, 4, 16, 2, 1010, 16, "max", 1),     # group of 8: 8 units of nine CTAs, 72 of 74
-    (2, 5, 16, 2, 900, 16, "sum", 1),      # ... 10 units of eight, 80: tcgen05 kernel
+    (2, 7, 16, 2, 900, 16, "sum", 1),      # ... 14 units of eight, of 15 that are resident at once
+    (2, 8, 16, 2, 900, 16, "sum", 1),      # ... 16 units: tcgen05 kernel
 ])
 def test_layer_calls(layers, batch, q_heads, kv_heads, C, R, fusion, per_layer):
     w = synth.Workload("small", layers, batch, q_heads, kv_heads, 128, "bf16", C + R - 3, min(2 * R, 60) + 14, C, R, fusion, 50 + R)
     rep = run_parity(w, steps=w.steps, n_units=4, per_layer=per_layer, check_F_every=5)
     assert rep.kernel == "tc" and rep.evictions > 0
     units, rounds, wide = (layers if per_layer == 0 else 1) * batch * kv_heads, -(-(C + R) // 128), q_heads // kv_heads > 4
-    small = units * min(rounds, 16) <= (74 if wide else 148) and (per_layer != 0 or rounds > 8)
+    ctas = min(rounds, 16)
+    small = units * ctas <= (74 if wide else 148) and (per_layer != 0 or rounds > 8)
+    small |= bool(wide and per_layer and ctas >= 4 and units <= 18 // ctas * 7 + 11 // ctas)
     assert rep.step_kernel == ("simt" if small and (q_heads // kv_heads, R) != (16, 100) else "tc")
 
 
