@@ -51,13 +51,14 @@ cudaError_t run_prefill(const DecodeArgs &a, bool f32, int D, const void *k, con
                         int P, cudaStream_t stream, unsigned long long *launches, PrefillScratch *scratch, int n_states,
                         int padded_len);
 
-// Tensor-core scoring of the prompt phase (mkv_prefill_tc.cu): two passes over the prompt keys, window-row
-// normalisers into ring_c and fused scores of the older tokens into Fp [nb][P].
+// Tensor-core scoring of the prompt phase (mkv_prefill_tc.cu): window-row normalisers into ring_c and fused scores of the
+// older tokens into Fp [nb][P].
 bool prefill_tc_supported(bool f32, int D, int G, int R, const void *k, const void *qwin, int P);
-int prefill_tc_splits(int units_in_batch, int P, int window_rows);
-size_t prefill_tc_floats_per_unit(int P, int Rw, int G, int splits);
-cudaError_t run_prefill_scores_tc(const DecodeArgs &a, const void *k, const void *qwin, int P, int Ps, int ub0, int nb, int splits,
-                                  float *Fp, float *part, int *err, unsigned long long *launches, cudaStream_t stream);
+int prefill_tc_run(int units, int P);              // key tiles of an item
+size_t prefill_tc_words_per_unit(int P, int run);
+size_t prefill_tc_floats_per_unit(int P, int Rw, int G, int run);
+cudaError_t run_prefill_scores_tc(const DecodeArgs &a, const void *k, const void *qwin, int P, int Ps, int ub0, int nb, int units, int run, bool select,
+                                  float *Fp, float *part, int *words, int *err, unsigned long long *launches, cudaStream_t stream);
 
 // The same prompt phase with its scratch in a fixed device array of prefill_static_max_floats()
 // floats instead of a temporary allocation; cudaErrorInvalidConfiguration if one unit's

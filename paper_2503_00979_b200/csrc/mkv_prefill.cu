@@ -18,6 +18,7 @@ namespace {
 constexpr int kPT = 256;    // threads per CTA
 constexpr int kPK = 32;     // keys per tile
 constexpr int kPR = 64;     // window rows per sub-block
+constexpr size_t kScratchWords = 3;      // ticket, finished CTAs and error word of the scoring kernels
 
 __device__ __forceinline__ void ld4(const float *p, float (&o)[4])
 {
@@ -32,11 +33,11 @@ __device__ __forceinline__ void ld4(const __nv_bfloat16 *p, float (&o)[4])
 }
 
 // (launched in full stream order: what it waits for is complete for the kernels behind it too)
-__global__ void init_arena_kernel(DecodeArgs a, int *err)
+__global__ void init_arena_kernel(DecodeArgs a, int *words, int n_words)
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i == 0) *err = 0;
+    if (i < (size_t)n_words) words[i] = 0;
     const size_t ncap = (size_t)a.U * a.cap;
     if (i < ncap) { a.pos[i] = -1; a.F[i] = 0.f; }
     if (i < ncap && a.nblk > 1) a.sum_pos[i] = -1;
@@ -536,25 +537,28 @@ cudaError_t run_prefill_t(const DecodeArgs &a, const T *k, const T *v, const T *
     const bool select = P - Rw > C;
     const int n = select ? C + Rw : P;
     if (n > a.cap) return cudaErrorInvalidValue;
-    // bf16 / head_dim 128 shapes score on the tensor cores (two passes over the keys, no rows x P table); the
+    // bf16 / head_dim 128 shapes score on the tensor cores (no rows x P table); the
     // others materialise the window-row logits S [rows][P] per unit and reduce them with CUDA-core kernels
     // (the arena's group must be the padded one: a context that runs the CUDA-core decode kernel keeps G as it is)
     const bool tc = prefill_tc_supported(sizeof(T) == 4, D, a.Gq, R, k, qwin, P) && tc_padded_group(a.Gq) == G;
-    const int tc_splits = tc ? prefill_tc_splits(U, P, Rw * G) : 0;
-    const size_t per_unit = tc ? prefill_tc_floats_per_unit(P, Rw, G, tc_splits) : (size_t)rows * P + P;   // floats
-    if (per_unit + 1 > scratch_floats) return cudaErrorInvalidConfiguration;
-    size_t ub = (scratch_floats - 1) / per_unit;
+    const int tc_run = tc ? prefill_tc_run(U, P) : 0;
+    const size_t per_unit = tc ? prefill_tc_floats_per_unit(P, Rw, G, tc_run) : (size_t)rows * P + P;   // floats
+    const size_t fixed = tc ? kScratchWords : 1;
+    if (per_unit + fixed > scratch_floats) return cudaErrorInvalidConfiguration;
+    size_t ub = (scratch_floats - fixed) / per_unit;
     if (ub > (size_t)U) ub = U;
     if (ub > 65535) ub = 65535;
-    float *Fp = tc ? S : S + ub * (size_t)rows * P;
-    float *part = S + ub * (size_t)P;                          // tensor-core path: pass-1 partials behind the scores
-    int *err_word = reinterpret_cast<int *>(S + scratch_floats - 1);
+    // tensor-core path: the window rows' statistics, the scores, and the words of state, zero at the start, that end with the error word
+    const size_t unit_words = tc ? prefill_tc_words_per_unit(P, tc_run) : 0;
+    float *part = S, *Fp = S + ub * (tc ? per_unit - P - unit_words : (size_t)rows * P);
+    const int n_words = (int)(ub * unit_words + fixed);
+    int *words = reinterpret_cast<int *>(Fp + ub * (size_t)P), *err_word = words + n_words - 1;
 
     const size_t logits_smem = (size_t)(kPK * (D + 4) + kPR * (D + 4) + kPK * (kPR + 1)) * sizeof(float);
     cudaError_t e = cudaFuncSetAttribute(prefill_logits_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)logits_smem);
     if (e != cudaSuccess) return e;
-    const size_t init_n = max((size_t)U * a.cap, (size_t)U * R * G);
-    init_arena_kernel<<<(unsigned)((init_n + 255) / 256), 256, 0, stream>>>(a, err_word);
+    const size_t init_n = max(max((size_t)U * a.cap, (size_t)U * R * G), (size_t)n_words);
+    init_arena_kernel<<<(unsigned)((init_n + 255) / 256), 256, 0, stream>>>(a, words, n_words);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const bool waits = tc || a.nblk > 1;            // kernels with bounded waits are launched
@@ -574,7 +578,7 @@ cudaError_t run_prefill_t(const DecodeArgs &a, const T *k, const T *v, const T *
     for (int ub0 = 0; ub0 < U; ub0 += (int)ub) {
         const int nb = min((int)ub, U - ub0);
         if (tc) {
-            e = run_prefill_scores_tc(a, k, qwin, P, Ps, ub0, nb, tc_splits, Fp, part, err_word, launches, stream);
+            e = run_prefill_scores_tc(a, k, qwin, P, Ps, ub0, nb, (int)ub, tc_run, select, Fp, part, words, err_word, launches, stream);
             if (e != cudaSuccess) return e;
         } else {
             prefill_logits_kernel<T, D><<<dim3((P + kPK - 1) / kPK, nb), kPT, logits_smem, stream>>>(k, qwin, S, ub0, P, Rw,
@@ -678,13 +682,13 @@ cudaError_t run_prefill(const DecodeArgs &a, bool f32, int D, const void *k, con
 {
     const int Rw = P < a.R ? P : a.R;
     const bool tc = prefill_tc_supported(f32, D, a.Gq, a.R, k, q_window, P) && tc_padded_group(a.Gq) == a.G;
-    const size_t per_unit = (tc ? prefill_tc_floats_per_unit(P, Rw, a.G, prefill_tc_splits(a.U, P, Rw * a.G))
+    const size_t per_unit = (tc ? prefill_tc_floats_per_unit(P, Rw, a.G, prefill_tc_run(a.U, P))
                                 : (size_t)Rw * a.G * P + P) * sizeof(float);
     size_t ub = ((size_t)1 << 30) / per_unit;
     if (ub < 1) ub = 1;
     if (ub > (size_t)a.U) ub = a.U;
     if (ub > 65535) ub = 65535;
-    const size_t need = ub * per_unit + sizeof(float);          // + the error word of the scoring kernels
+    const size_t need = ub * per_unit + kScratchWords * sizeof(float);
     // The scratch belongs to the context and is kept until the context is destroyed: it only grows.
     // (Allocating and freeing it around every prompt put a cudaFree of up to 1 GiB right in front
     // of the first decode launches.)

@@ -135,7 +135,7 @@ window_sums_tc_kernel(const __grid_constant__ SumArgs a, const __grid_constant__
                 ok = __all_sync(0xffffffffu, k);
                 if (!ok) break;
                 tc_fence_after();
-                if (lane == 0) {
+                if (elect_one()) {
                     const uint32_t d_tmem = tmem_base + (uint32_t)(b * PR);
 #pragma unroll
                     for (int ks = 0; ks < kD / 16; ++ks) {
@@ -339,7 +339,7 @@ gather_sums_tc_kernel(const __grid_constant__ GatherArgs ga, const __grid_consta
             ok = __all_sync(0xffffffffu, k);
             if (!ok) break;
             tc_fence_after();
-            if (lane == 0) {
+            if (elect_one()) {
                 const uint32_t d_tmem = tmem_base + (uint32_t)(b * PR);
 #pragma unroll
                 for (int ks = 0; ks < kD / 16; ++ks) {
@@ -476,6 +476,23 @@ DecodeArgs unit_range(const DecodeArgs &d, int D, size_t es, int u0, int count)
 }
 constexpr int kMaxGridY = 65535;
 
+// CTAs per unit along the keys.  A CTA pays a set-up (TMEM, barriers, the ring's rows into shared memory) worth about
+// `kSetupTiles` key tiles, and the grid runs in waves of `slots` resident CTAs: the split with the fewest tile-times over all waves.
+int sums_splits(int units, int n, int rows)
+{
+    constexpr int kSetupTiles = 3;
+    const int nt = (n + kTile - 1) / kTile;
+    const int slots = 148 * (rows <= 128 ? 2 : 1);
+    int best = 1;
+    long long best_cost = -1;
+    for (int s = 1; s <= nt && s <= 64; ++s) {
+        const long long waves = ((long long)units * s + slots - 1) / slots;
+        const long long cost = waves * ((nt + s - 1) / s + kSetupTiles);
+        if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = s; }
+    }
+    return best;
+}
+
 }  // namespace
 
 bool gather_sums_supported(const DecodeArgs &d, const void *k, const void *v)
@@ -530,7 +547,7 @@ cudaError_t launch_finish_prompt(const DecodeArgs &d, bool sums, long long t, in
     const int chunk = kSumMaxRows / a.piece * a.piece;
     for (int u0 = 0; u0 < d.U; u0 += kMaxGridY) {
         a.d = unit_range(d, kD, 2, u0, min(kMaxGridY, d.U - u0));
-        a.splits = prefill_tc_splits(a.d.U, n, a.piece);
+        a.splits = sums_splits(a.d.U, n, a.piece);
         CUtensorMap tm;
         if (!encode_map(&tm, a.d.K, a.d.U, d.cap, kTile)) return cudaErrorInvalidValue;
         for (int row0 = (all - 1) / chunk * chunk; row0 >= 0; row0 -= chunk) {
