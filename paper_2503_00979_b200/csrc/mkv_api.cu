@@ -222,6 +222,7 @@ DecodeArgs make_args(const mkv_ctx *c, const void *q, const void *k, const void 
     a.B = c->s.B; a.Hkv = c->s.Hkv;
     a.n_hint = c->prefilled ? c->n : 0;
     a.check_moved = 0;
+    a.early = 0;
     return a;
 }
 
@@ -309,10 +310,11 @@ mkv_status launch_step(mkv_ctx *ctx, int layer, const void *q, const void *k, co
     // (cudaStreamPerThread names another stream in every thread.)
     const bool early = layer >= 0 && ctx->last_layer >= 0 && ctx->last_layer != layer && ctx->last_stream == stream &&
                        stream != cudaStreamPerThread && ctx->last_capturing == capturing && ctx->launches == before && !behind_holder;
+    a.early = early ? 1 : 0;
     ctx->last_layer = layer;
     ctx->last_stream = stream;
     ctx->last_capturing = capturing;
-    const cudaError_t e = nsplit > 0 ? launch_decode_simt(a, nsplit, early, ctx->p.dtype == MKV_DTYPE_F32, ctx->s.D, stream)
+    const cudaError_t e = nsplit > 0 ? launch_decode_simt(a, nsplit, ctx->p.dtype == MKV_DTYPE_F32, ctx->s.D, stream)
                                      : launch_decode_tc(layer < 0 ? ctx->plan : ctx->plan_layer, a, stream);
     if (e != cudaSuccess) return fail(ctx, MKV_CUDA, "decode launch failed: %s", cudaGetErrorString(e));
     ctx->launches += 1;

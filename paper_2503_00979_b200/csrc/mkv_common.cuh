@@ -80,6 +80,8 @@ struct DecodeArgs {
                                // sums again (resum_moved).  (On every launch it would cost 2 to 3 %: 57.6 to 58.9 us for 256
                                // units x 2032 slots, 844 to 870 for 8192 x 1056.)
     int bs, nblk;
+    int early;                 // 1: the launch before this one in the stream does not touch this launch's units: all that does not
+                               // need the inputs or write the output may run before that launch ends
     int n_hint;                // the host's view of st->n when the launch was enqueued (0: none).  Only used to
                                // prefetch: a stale value (steps replayed from a CUDA graph) costs time, not results
 };

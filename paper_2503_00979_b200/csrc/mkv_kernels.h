@@ -5,9 +5,8 @@
 
 namespace mkv {
 
-// Warp-level decode step (any supported shape).  `nsplit` CTAs per unit, at most 16.  `early`: the launch before this one
-// in the stream does not touch this launch's units, so all that does not need its inputs may run before that launch ends.
-cudaError_t launch_decode_simt(const DecodeArgs &a, int nsplit, bool early, bool f32, int D, cudaStream_t stream);
+// Warp-level decode step (any supported shape).  `nsplit` CTAs per unit, at most 16.
+cudaError_t launch_decode_simt(const DecodeArgs &a, int nsplit, bool f32, int D, cudaStream_t stream);
 int simt_block_slots(bool f32, int G, int R);      // slots per block of the ring (DecodeArgs::bs), 0: no sums are kept
 int simt_default_splits(int U, int cap);
 int simt_small_splits(int U, int G, int R, int bs, int nblk, int cap, bool layer);   // CTAs per unit for a small tcgen05-context launch, 0: not small

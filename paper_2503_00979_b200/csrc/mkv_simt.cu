@@ -21,7 +21,7 @@
 //
 // Bound by HBM for bf16 and, nearly, by FMA issue for f32; small launches by their chain of latencies.  Of those
 // everything that does not need the new query (state, tiles, ring rows, their scoring) may run before the launch before
-// this one has ended, when that launch works on another layer (`early`).
+// this one has ended, when that launch works on another layer (DecodeArgs::early).
 //
 // Measured: 512 units x 1056 slots, bf16, d = 64, R*G = 128: 65 us per step (all rows scored with scalar FMAs, CTA barriers
 // per tile: 838).  2 units x 80 slots, f32, d = 64: 10.6 us (30.6).  One layer of 8 units x 2032 slots, bf16, d = 128, as a
@@ -130,11 +130,10 @@ __device__ __forceinline__ void st_cluster64(uint32_t addr, unsigned long long v
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
-// GP: the group padded to a power of two (padding heads: zero query, weight 0).  `early`: the launch before this one
-// does not touch this launch's units.  CHECK: DecodeArgs::check_moved (compiled apart, as it costs a layer's call 0.4 us).
+// GP: the group padded to a power of two (padding heads: zero query, weight 0).  CHECK: DecodeArgs::check_moved (compiled apart, as it costs a layer's call 0.4 us).
 template <typename T, int D, int GP, bool CHECK>
 __global__ void __launch_bounds__(SimtSmem<T, D, GP>::threads, GP > 8 ? 1 : SimtSmem<T, D, GP>::ctas)
-decode_simt_kernel(const __grid_constant__ DecodeArgs a, const int nsplit, const int early)
+decode_simt_kernel(const __grid_constant__ DecodeArgs a, const int nsplit)
 {
     using L = SimtSmem<T, D, GP>;
     constexpr bool BF = sizeof(T) == 2;
@@ -155,8 +154,8 @@ decode_simt_kernel(const __grid_constant__ DecodeArgs a, const int nsplit, const
     if (nsplit > 1) cluster_arrive();      // waited for before the first access to another CTA's memory
     // see the tcgen05 kernel: the grid before this one is complete behind the wait, the next one may start and park there.
     // (Every grid releases the next one after its own wait, so the grid before the one before this one is complete here
-    // already: with `early` nothing in flight can still write this launch's units or their state.)
-    if (!early) {
+    // already: with DecodeArgs::early nothing in flight can still write this launch's units or their state.)
+    if (!a.early) {
         asm volatile("griddepcontrol.wait;" ::: "memory");
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     }
@@ -386,7 +385,7 @@ decode_simt_kernel(const __grid_constant__ DecodeArgs a, const int nsplit, const
             }
             if (!q_here) {
                 q_here = true;
-                if (early) {
+                if (a.early) {
                     asm volatile("griddepcontrol.wait;" ::: "memory");
                     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
                 }
@@ -794,7 +793,7 @@ decode_simt_kernel(const __grid_constant__ DecodeArgs a, const int nsplit, const
 }
 
 template <typename T, int D, int GP, bool CHECK>
-cudaError_t launch_simt_g(const DecodeArgs &a, int nsplit, bool early, cudaStream_t stream)
+cudaError_t launch_simt_g(const DecodeArgs &a, int nsplit, cudaStream_t stream)
 {
     auto kern = decode_simt_kernel<T, D, GP, CHECK>;
     const int smem = SimtSmem<T, D, GP>::total;
@@ -814,35 +813,35 @@ cudaError_t launch_simt_g(const DecodeArgs &a, int nsplit, bool early, cudaStrea
     attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = nsplit > 1 ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, kern, a, nsplit, early ? 1 : 0);
+    return cudaLaunchKernelEx(&cfg, kern, a, nsplit);
 }
 
 template <typename T, int D, bool CHECK>
-cudaError_t launch_simt_t(const DecodeArgs &a, int nsplit, bool early, cudaStream_t stream)
+cudaError_t launch_simt_t(const DecodeArgs &a, int nsplit, cudaStream_t stream)
 {
     switch (tc_padded_group(a.G)) {
-        case 1: return launch_simt_g<T, D, 1, CHECK>(a, nsplit, early, stream);
-        case 2: return launch_simt_g<T, D, 2, CHECK>(a, nsplit, early, stream);
-        case 4: return launch_simt_g<T, D, 4, CHECK>(a, nsplit, early, stream);
-        case 8: return launch_simt_g<T, D, 8, CHECK>(a, nsplit, early, stream);
-        case 16: return launch_simt_g<T, D, 16, CHECK>(a, nsplit, early, stream);
+        case 1: return launch_simt_g<T, D, 1, CHECK>(a, nsplit, stream);
+        case 2: return launch_simt_g<T, D, 2, CHECK>(a, nsplit, stream);
+        case 4: return launch_simt_g<T, D, 4, CHECK>(a, nsplit, stream);
+        case 8: return launch_simt_g<T, D, 8, CHECK>(a, nsplit, stream);
+        case 16: return launch_simt_g<T, D, 16, CHECK>(a, nsplit, stream);
     }
     return cudaErrorInvalidValue;
 }
 
 template <bool CHECK>
-cudaError_t launch_simt_c(const DecodeArgs &a, int nsplit, bool early, bool f32, int D, cudaStream_t stream)
+cudaError_t launch_simt_c(const DecodeArgs &a, int nsplit, bool f32, int D, cudaStream_t stream)
 {
-    if (f32) return D == 64 ? launch_simt_t<float, 64, CHECK>(a, nsplit, early, stream) : launch_simt_t<float, 128, CHECK>(a, nsplit, early, stream);
-    return D == 64 ? launch_simt_t<__nv_bfloat16, 64, CHECK>(a, nsplit, early, stream) : launch_simt_t<__nv_bfloat16, 128, CHECK>(a, nsplit, early, stream);
+    if (f32) return D == 64 ? launch_simt_t<float, 64, CHECK>(a, nsplit, stream) : launch_simt_t<float, 128, CHECK>(a, nsplit, stream);
+    return D == 64 ? launch_simt_t<__nv_bfloat16, 64, CHECK>(a, nsplit, stream) : launch_simt_t<__nv_bfloat16, 128, CHECK>(a, nsplit, stream);
 }
 
 }  // namespace
 
-cudaError_t launch_decode_simt(const DecodeArgs &a, int nsplit, bool early, bool f32, int D, cudaStream_t stream)
+cudaError_t launch_decode_simt(const DecodeArgs &a, int nsplit, bool f32, int D, cudaStream_t stream)
 {
     if (nsplit > kMaxCluster) return cudaErrorInvalidValue;
-    return a.check_moved ? launch_simt_c<true>(a, nsplit, early, f32, D, stream) : launch_simt_c<false>(a, nsplit, early, f32, D, stream);
+    return a.check_moved ? launch_simt_c<true>(a, nsplit, f32, D, stream) : launch_simt_c<false>(a, nsplit, f32, D, stream);
 }
 
 // Rows of a block are scored on every step and once more when it is finished: 16 where they cost scalar FMAs, 32 on the
