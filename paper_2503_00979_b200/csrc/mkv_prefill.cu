@@ -189,10 +189,12 @@ __global__ void __launch_bounds__(kPT) prefill_fuse_kernel(const float *__restri
 // until the bucket fits the list (the first digit as a rule; more where many scores tie), and twice more.
 // Bound by latency for short prompts, by L2 for long ones.  With 8-bit digits, every one of them over all keys, and a
 // compaction of 1024 keys per round between barriers: 31 us for 256 units of 6112 keys and 306 us for 131040, now 17 and 101.
-constexpr int kSelT = 1024;      // threads of the selection kernel
 constexpr int kSelRun = 8;       // keys a lane holds at a time
 constexpr int kSelList = 3072;   // keys of a bucket that fit the list
-__global__ void __launch_bounds__(kSelT, 2) prefill_select_kernel(const float *__restrict__ Fp, int *__restrict__ pos, int ub0,
+// T threads per CTA: 1024, or 512 for many units of short prompts, whose CTAs are bound by their barriers (2048 units x 1900 keys
+// on average: 60 -> 48 us).
+template <int kSelT>
+__global__ void __launch_bounds__(kSelT, 2048 / kSelT) prefill_select_kernel(const float *__restrict__ Fp, int *__restrict__ pos, int ub0,
                                                                   int P, int Rw, int C, int cap, RowMap rowmap)
 {
     constexpr int kW = kSelT / 32, kChunk = 32 * kSelRun, kBins = 4096, kPer = kBins / kSelT;
@@ -262,7 +264,7 @@ __global__ void __launch_bounds__(kSelT, 2) prefill_select_kernel(const float *_
         }
         if (lane == 0) wtot[warp] = incl;
         __syncthreads();
-        int wsum = lane > warp ? wtot[lane] : 0;                         // (as many warps as lanes)
+        int wsum = lane > warp && lane < kW ? wtot[lane] : 0;
         wsum = (int)__reduce_add_sync(0xffffffffu, (unsigned)wsum);
         int above = wsum + incl - own;
         if (above < remaining && remaining <= above + own) {
@@ -441,7 +443,7 @@ __global__ void prefill_ring_kernel(const T *__restrict__ qwin, DecodeArgs a, in
     }
 }
 
-// the same, 16 bytes per thread (q_window 16-byte aligned)
+// the same, 16 bytes at a time and four in flight per thread (q_window 16-byte aligned; 2048 units of 128 rows 34 -> 23 us)
 template <typename T, int D>
 __global__ void prefill_ring_vec_kernel(const T *__restrict__ qwin, DecodeArgs a, int P, int Rws, RowMap rowmap)
 {
@@ -450,12 +452,20 @@ __global__ void prefill_ring_vec_kernel(const T *__restrict__ qwin, DecodeArgs a
     const int u = blockIdx.x, G = a.G, Gq = a.Gq, shift = rowmap(u);
     P -= shift;
     const int Rw = min(P, a.R);
-    for (int idx = blockIdx.y * blockDim.x + threadIdx.x; idx < a.R * G * CH; idx += gridDim.y * blockDim.x) {
-        const int c = idx % CH, g = (idx / CH) % G, i = idx / (CH * G);
-        const int rslot = (P - Rw + i + shift) % a.R;
-        uint4 v = make_uint4(0, 0, 0, 0);
-        if (g < Gq && i < Rw) v = reinterpret_cast<const uint4 *>(qwin + (((size_t)u * Gq + g) * Rws + i) * D)[c];
-        reinterpret_cast<uint4 *>(static_cast<T *>(a.ring_q) + (((size_t)u * a.R + rslot) * G + g) * D)[c] = v;
+    const uint4 *src = reinterpret_cast<const uint4 *>(qwin) + (size_t)u * Gq * Rws * CH;
+    uint4 *dst = reinterpret_cast<uint4 *>(a.ring_q) + (size_t)u * a.R * G * CH;
+    for (int idx0 = (int)blockIdx.y * 4 * blockDim.x + threadIdx.x; idx0 < a.R * G * CH; idx0 += gridDim.y * 4 * blockDim.x) {
+        uint4 v[4];
+        int at[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int idx = idx0 + j * blockDim.x, c = idx % CH, g = (idx / CH) % G, i = idx / (CH * G);
+            at[j] = idx < a.R * G * CH ? ((P - Rw + i + shift) % a.R * G + g) * CH + c : -1;
+            v[j] = at[j] >= 0 && g < Gq && i < Rw ? src[(g * Rws + i) * CH + c] : make_uint4(0, 0, 0, 0);
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (at[j] >= 0) dst[at[j]] = v[j];
     }
 }
 
@@ -564,7 +574,7 @@ cudaError_t run_prefill_t(const DecodeArgs &a, const T *k, const T *v, const T *
     const bool waits = tc || a.nblk > 1;            // kernels with bounded waits are launched
     constexpr int CH = D * sizeof(T) / 16;
     e = ((uintptr_t)qwin & 15) == 0
-        ? launch_chained(prefill_ring_vec_kernel<T, D>, dim3(U, min(kMaxGridY, (R * G * CH + 255) / 256)), 256, 0, stream, qwin, a, P, Rws, rowmap)
+        ? launch_chained(prefill_ring_vec_kernel<T, D>, dim3(U, min(kMaxGridY, (R * G * CH + 1023) / 1024)), 256, 0, stream, qwin, a, P, Rws, rowmap)
         : launch_chained(prefill_ring_kernel<T, D>, dim3(U), 256, 0, stream, qwin, a, P, Rws, rowmap);
     if (e != cudaSuccess) return e;
     *launches += 2;
@@ -592,7 +602,8 @@ cudaError_t run_prefill_t(const DecodeArgs &a, const T *k, const T *v, const T *
                     S, a.ring_c, Fp, ub0, P, Rw, a.Gq, G, R, a.fusion, rowmap);
                 ++*launches;
             }
-            e = launch_chained(prefill_select_kernel, dim3(nb), kSelT, 0, stream, Fp, a.pos, ub0, P, Rw, C, a.cap, rowmap);
+            e = nb > 2 * 148 && P - Rw <= 512 * kSelRun ? launch_chained(prefill_select_kernel<512>, dim3(nb), 512, 0, stream, Fp, a.pos, ub0, P, Rw, C, a.cap, rowmap)
+                                                       : launch_chained(prefill_select_kernel<1024>, dim3(nb), 1024, 0, stream, Fp, a.pos, ub0, P, Rw, C, a.cap, rowmap);
             if (e != cudaSuccess) return e;
             ++*launches;
         }
