@@ -117,11 +117,12 @@ __device__ __forceinline__ float warp_sum(float v)
     return v;
 }
 
+// (one instruction instead of five shuffles and maxima; like fmaxf it passes over NaN)
 __device__ __forceinline__ float warp_max(float v)
 {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
+    float r;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
 }
 
 // Ordering key of a candidate: larger key = better.  Fused scores are non-negative floats,
