@@ -147,7 +147,7 @@ template <int G, bool LOCAL>
 __device__ void finalize_fast(const DecodeArgs &a, int u, long long t, int n, int nseg, bool evict, float *sm, int tid,
                               int bar_id, const float (&l_o)[G], const float *l_ml, int shift, const NewRows<G> &x, bool moved)
 {
-    constexpr int NT_ = kGroupThreads;
+    constexpr int NT_ = kGroupThreads, NS = LOCAL ? 1 : 8;
     const int lane = tid & 31, warp = tid >> 5;
     float *s_self = sm, *mfin = sm + kMaxGroup, *lfin = sm + 2 * kMaxGroup, *cnew = sm + 3 * kMaxGroup;
     float *vsm = sm + 4 * kMaxGroup;                       // [128] new value row as floats
@@ -162,11 +162,11 @@ __device__ void finalize_fast(const DecodeArgs &a, int u, long long t, int n, in
     // ---- phase A: every load that does not depend on another one
     constexpr int QCH = NewRows<G>::chunks;
     for (int i = tid; i < nseg * G * 2; i += NT_) pml_s[i] = LOCAL ? l_ml[i] : __ldcg(pml + i);
-    float pov[G][8];
+    float pov[G][NS];
 #pragma unroll
     for (int g = 0; g < G; ++g)
 #pragma unroll
-        for (int sp = 0; sp < 8; ++sp)
+        for (int sp = 0; sp < NS; ++sp)
             pov[g][sp] = sp < nseg ? (LOCAL ? l_o[g] : __ldcg(po + (sp * G + g) * kD + tid)) : 0.f;
 
     // self logit: 8-element partial dots, reduced over the 16 threads that share a head
@@ -213,7 +213,7 @@ __device__ void finalize_fast(const DecodeArgs &a, int u, long long t, int n, in
         const float m = mfin[g];
         float o = exp2f(s_self[g] - m) * vsm[tid];
 #pragma unroll
-        for (int sp = 0; sp < 8; ++sp)
+        for (int sp = 0; sp < NS; ++sp)
             if (sp < nseg) o += pov[g][sp] * exp2f(pml_s[(sp * G + g) * 2] - m);
         if (g < Gq) out[g * kD + tid] = __float2bfloat16_rn(o / lfin[g]);
     }
@@ -584,7 +584,7 @@ decode_tc_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ C
         RingPos rk(0, SK), rb(0, NB);
         while (ok && w.next(x)) {
             {
-                if (w.nitems > 0 && lane == 0) umma_commit(bar_qempty);   // MMAs of the previous unit done with the ring
+                if (w.nitems > 0 && elect_one()) umma_commit(bar_qempty);   // MMAs of the previous unit done with the ring
                 // the new query replaces ring row t % R (the row of the token leaving the window)
                 const int u = MC ? x.unit / NCe : x.unit;
                 const bool main_item = MC ? (NCe == 1 || x.unit - u * NCe == c_main) : true;   // the chunk with the new query's slot
@@ -614,7 +614,7 @@ decode_tc_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ C
                 ok = __all_sync(0xffffffffu, k);
                 if (!ok) break;
                 tc_fence_after();
-                if (lane == 0) {
+                if (elect_one()) {
                     const uint32_t d_tmem = tmem_base + (uint32_t)(b * RGP);
 #pragma unroll
                     for (int ks = 0; ks < kD / 16; ++ks) {
@@ -977,18 +977,21 @@ decode_tc_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ C
                 if (group_any(kEpiBar, !mbar_wait(bar_udone, (uint32_t)(k & 1), abort_flag, kWaitUDone, WL))) { ok = false; break; }
                 bool moved = BLOCKS && *moved_flag != 0;
                 // merge the compute warps' partials: common reference = max of theirs
-                if (etid < G && main_item) {
-                    float m = -INFINITY;
-                    for (int cwi = 0; cwi < NCW; ++cwi) m = fmaxf(m, wml[cwi * 2 * kMaxGroup + etid * 2]);
-                    float l = 0.f;
-                    for (int cwi = 0; cwi < NCW; ++cwi) {
-                        const float mw = wml[cwi * 2 * kMaxGroup + etid * 2];
-                        const float f = mw == -INFINITY ? 0.f : ex2f(mw - m);
-                        sc[cwi * kMaxGroup + etid] = f;
-                        l += wml[cwi * 2 * kMaxGroup + etid * 2 + 1] * f;
+                {   // (eight lanes per head, one per warp; by one thread per head this and the outputs took 0.8 us of every unit's epilogue)
+                    static_assert(NCW == 8 && NCW * kMaxGroup == kGroupThreads, "a lane per compute warp and head");
+                    const int g = etid / NCW, cwi = etid % NCW;
+                    const float mw = wml[cwi * 2 * kMaxGroup + g * 2];
+                    float m = mw;
+#pragma unroll
+                    for (int o = NCW / 2; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+                    const float f = mw == -INFINITY ? 0.f : ex2f(mw - m);
+                    float l = wml[cwi * 2 * kMaxGroup + g * 2 + 1] * f;
+#pragma unroll
+                    for (int o = NCW / 2; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+                    if (g < G && main_item) {
+                        sc[cwi * kMaxGroup + g] = f;
+                        if (cwi == 0) { cml[g * 2] = m; cml[g * 2 + 1] = l; }
                     }
-                    cml[etid * 2] = m;
-                    cml[etid * 2 + 1] = l;
                 }
                 group_sync(kEpiBar, kGroupThreads);
                 float o[G];
