@@ -384,7 +384,7 @@ def run_prefill_arm(args, w):
         "clocks": clocks.summary(), "e2e": None, "gpu_launches": int(mk.launch_count - launches0),
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak, "nominal_peak": NOMINAL_HBM_GBS,
                         "frac_of_nominal": achieved / NOMINAL_HBM_GBS,
-                     "traffic": None, "peak_source": peak_src, "kernel": "prefill (two scoring passes + select + gather)",
+                     "traffic": None, "peak_source": peak_src, "kernel": "prefill (scoring + select + gather)",
                      "algorithmic_bytes_per_launch": bytes_step},
     }
     print(json.dumps(line), flush=True)
