@@ -50,7 +50,6 @@ constexpr int kPfDesc = 4;                   // item descriptors in flight
 constexpr int kPfMaxStages = 4;
 constexpr int kPfSm = 148;
 constexpr int kPfL2Tiles = 2048;             // 64 MB of keys
-constexpr float kPfFarBelow = 1099511627776.f;        // 2^40
 constexpr int kPfMerge = 16;                 // statistics merged at a time
 enum PfWait { kPfKEmpty = 21, kPfKFull, kPfTEmpty, kPfTFull, kPfDrain, kPfDEmpty, kPfDFull, kPfQEmpty, kPfQFull, kPfNEmpty, kPfNFull,
               kPfSEmpty, kPfSFull, kPfFlag, kPfPair };
@@ -546,20 +545,19 @@ prefill_tc_kernel(const __grid_constant__ PfArgs a, const __grid_constant__ CUte
                                 for (int i = 0; i < 32; ++i)
                                     if (kc + i > lim) v[i] = 0xff800000u;        // -inf: weight 0
                             }
-                            // the reference is the maximum of the row's first chunk, and moves only when a sum shows that
-                            // it is far below another one (2^40 against 2^127): sums relative to it are as exact as those
-                            // relative to the maximum, which would have to be taken in every chunk
-                            float t = m > -INFINITY ? sum_chunk(v, a.scale2, m) : INFINITY;
-                            if (!(t < kPfFarBelow)) {
-                                // the scale is positive, so the maximum is taken on the raw logits and scaled once
-                                float cm = -INFINITY;
+                            // The reference is the maximum so far, rounded up: the weights that count have exponents near 0, and factors
+                            // between references, here and where sums are merged, are whole powers of two.  The scale is positive, so
+                            // the maximum is taken on the raw logits and scaled once.
+                            float cm = -INFINITY;
 #pragma unroll
-                                for (int i = 0; i < 32; ++i) cm = fmaxf(cm, __uint_as_float(v[i]));
-                                cm *= a.scale2;
-                                if (cm > m) { l *= ex2f(m - cm); m = cm; }
-                                t = sum_chunk(v, a.scale2, m);
+                            for (int i = 0; i < 32; ++i) cm = fmaxf(cm, __uint_as_float(v[i]));
+                            cm *= a.scale2;
+                            if (cm > m) {
+                                const float up = ceilf(cm);
+                                l *= ex2f(m - up);
+                                m = up;
                             }
-                            l += t;
+                            l += sum_chunk(v, a.scale2, m);
                         }
                         __syncwarp();                        // the lanes meet again in front of the aligned TMEM load
                     }
