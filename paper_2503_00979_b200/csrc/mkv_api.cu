@@ -444,7 +444,7 @@ mkv_status core_prefill(mkv_ctx *ctx, const void *k, const void *v, const void *
     const int n_states = 1 + ctx->s.layers;
     const cudaError_t e = use_static
         ? run_prefill_static(a, f32, ctx->s.D, k, v, q_window, prompt_len, stream, &ctx->launches, ctx->device, n_states)
-        : run_prefill(a, f32, ctx->s.D, k, v, q_window, prompt_len, stream, &ctx->launches, &ctx->prefill_scratch, n_states, prompt_len);
+        : run_prefill(a, f32, ctx->s.D, k, v, q_window, prompt_len, stream, &ctx->launches, &ctx->prefill_scratch, n_states, prompt_len, nullptr);
     if (e == cudaErrorMemoryAllocation) { cudaGetLastError(); return fail(ctx, MKV_OOM, "%s: no memory for scratch", where); }
     if (e == cudaErrorLaunchTimeout) { cudaGetLastError(); return fail(ctx, MKV_DEVICE_TIMEOUT, "%s: a device-side wait of the prompt phase ran out", where); }
     if (e != cudaSuccess) return fail(ctx, MKV_CUDA, "prompt phase: %s", cudaGetErrorString(e));
@@ -487,7 +487,7 @@ mkv_status core_prefill_ragged(mkv_ctx *ctx, const void *k, const void *v, const
     const DecodeArgs a = make_args(ctx, nullptr, nullptr, nullptr, nullptr);
     if (e == cudaSuccess)
         e = run_prefill(a, ctx->p.dtype == MKV_DTYPE_F32, s.D, k, v, q_window, longest, stream, &ctx->launches, &ctx->prefill_scratch, ns,
-                        padded_len);
+                        padded_len, ctx->row_shift);
     delete[] rows_h;
     if (e == cudaErrorMemoryAllocation) { cudaGetLastError(); return fail(ctx, MKV_OOM, "mkv_prefill_ragged: no memory for scratch%s"); }
     if (e == cudaErrorLaunchTimeout) { cudaGetLastError(); return fail(ctx, MKV_DEVICE_TIMEOUT, "mkv_prefill_ragged: a device-side wait of the prompt phase ran out%s"); }

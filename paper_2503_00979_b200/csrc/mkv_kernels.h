@@ -44,19 +44,19 @@ struct PrefillScratch {
     size_t bytes;
     int *host_err;       // pinned word (nullptr: none could be had)
 };
-// With prompts of different lengths in the batch (a.row_shift) P is the longest prompt's length; the tensors are padded
-// to padded_len tokens (P otherwise).
+// With prompts of different lengths in the batch (a.row_shift; `row_shift`: the same [B] numbers on the host, else nullptr) P is
+// the longest prompt's length; the tensors are padded to padded_len tokens (P otherwise).
 cudaError_t run_prefill(const DecodeArgs &a, bool f32, int D, const void *k, const void *v, const void *q_window,
                         int P, cudaStream_t stream, unsigned long long *launches, PrefillScratch *scratch, int n_states,
-                        int padded_len);
+                        int padded_len, const int *row_shift);
 
 // Tensor-core scoring of the prompt phase (mkv_prefill_tc.cu): window-row normalisers into ring_c and fused scores of the
 // older tokens into Fp [nb][P].
 bool prefill_tc_supported(bool f32, int D, int G, int R, const void *k, const void *qwin, int P);
-int prefill_tc_run(int units, int P);              // key tiles of an item
+int prefill_tc_run(const DecodeArgs &a, int P, const int *row_shift);       // key tiles of an item
 size_t prefill_tc_words_per_unit(int P, int run);
 size_t prefill_tc_floats_per_unit(int P, int Rw, int G, int run);
-cudaError_t run_prefill_scores_tc(const DecodeArgs &a, const void *k, const void *qwin, int P, int Ps, int ub0, int nb, int units, int run, bool select,
+cudaError_t run_prefill_scores_tc(const DecodeArgs &a, const void *k, const void *qwin, int P, int Ps, const int *row_shift, int ub0, int nb, int units, int run, bool select,
                                   float *Fp, float *part, int *words, int *err, unsigned long long *launches, cudaStream_t stream);
 
 // The same prompt phase with its scratch in a fixed device array of prefill_static_max_floats()

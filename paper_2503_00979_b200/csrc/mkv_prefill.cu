@@ -534,7 +534,8 @@ __global__ void __launch_bounds__(kPT) prefill_renorm_kernel(DecodeArgs a, int P
 
 template <typename T, int D>
 cudaError_t run_prefill_t(const DecodeArgs &a, const T *k, const T *v, const T *qwin, int P, cudaStream_t stream,
-                          unsigned long long *launches, float *S, size_t scratch_floats, int *host_err, int n_states, int padded_len)
+                          unsigned long long *launches, float *S, size_t scratch_floats, int *host_err, int n_states, int padded_len,
+                          const int *row_shift)
 {
     // With prompts of different lengths (a.row_shift) P is the longest one and the tensors are padded to padded_len
     // tokens; the ring slots follow the common time axis, on which every row ends at P.
@@ -551,7 +552,7 @@ cudaError_t run_prefill_t(const DecodeArgs &a, const T *k, const T *v, const T *
     // others materialise the window-row logits S [rows][P] per unit and reduce them with CUDA-core kernels
     // (the arena's group must be the padded one: a context that runs the CUDA-core decode kernel keeps G as it is)
     const bool tc = prefill_tc_supported(sizeof(T) == 4, D, a.Gq, R, k, qwin, P) && tc_padded_group(a.Gq) == G;
-    const int tc_run = tc ? prefill_tc_run(U, P) : 0;
+    const int tc_run = tc ? prefill_tc_run(a, P, row_shift) : 0;
     const size_t per_unit = tc ? prefill_tc_floats_per_unit(P, Rw, G, tc_run) : (size_t)rows * P + P;   // floats
     const size_t fixed = tc ? kScratchWords : 1;
     if (per_unit + fixed > scratch_floats) return cudaErrorInvalidConfiguration;
@@ -588,7 +589,7 @@ cudaError_t run_prefill_t(const DecodeArgs &a, const T *k, const T *v, const T *
     for (int ub0 = 0; ub0 < U; ub0 += (int)ub) {
         const int nb = min((int)ub, U - ub0);
         if (tc) {
-            e = run_prefill_scores_tc(a, k, qwin, P, Ps, ub0, nb, (int)ub, tc_run, select, Fp, part, words, err_word, launches, stream);
+            e = run_prefill_scores_tc(a, k, qwin, P, Ps, row_shift, ub0, nb, (int)ub, tc_run, select, Fp, part, words, err_word, launches, stream);
             if (e != cudaSuccess) return e;
         } else {
             prefill_logits_kernel<T, D><<<dim3((P + kPK - 1) / kPK, nb), kPT, logits_smem, stream>>>(k, qwin, S, ub0, P, Rw,
@@ -642,17 +643,17 @@ cudaError_t run_prefill_t(const DecodeArgs &a, const T *k, const T *v, const T *
 
 cudaError_t dispatch_prefill(const DecodeArgs &a, bool f32, int D, const void *k, const void *v, const void *q_window, int P,
                              cudaStream_t stream, unsigned long long *launches, float *S, size_t scratch_floats, int *host_err, int n_states,
-                             int padded_len)
+                             int padded_len, const int *row_shift)
 {
     if (f32) {
         auto kk = static_cast<const float *>(k), vv = static_cast<const float *>(v), qq = static_cast<const float *>(q_window);
-        return D == 64 ? run_prefill_t<float, 64>(a, kk, vv, qq, P, stream, launches, S, scratch_floats, host_err, n_states, padded_len)
-                       : run_prefill_t<float, 128>(a, kk, vv, qq, P, stream, launches, S, scratch_floats, host_err, n_states, padded_len);
+        return D == 64 ? run_prefill_t<float, 64>(a, kk, vv, qq, P, stream, launches, S, scratch_floats, host_err, n_states, padded_len, row_shift)
+                       : run_prefill_t<float, 128>(a, kk, vv, qq, P, stream, launches, S, scratch_floats, host_err, n_states, padded_len, row_shift);
     }
     auto kk = static_cast<const __nv_bfloat16 *>(k), vv = static_cast<const __nv_bfloat16 *>(v),
          qq = static_cast<const __nv_bfloat16 *>(q_window);
-    return D == 64 ? run_prefill_t<__nv_bfloat16, 64>(a, kk, vv, qq, P, stream, launches, S, scratch_floats, host_err, n_states, padded_len)
-                   : run_prefill_t<__nv_bfloat16, 128>(a, kk, vv, qq, P, stream, launches, S, scratch_floats, host_err, n_states, padded_len);
+    return D == 64 ? run_prefill_t<__nv_bfloat16, 64>(a, kk, vv, qq, P, stream, launches, S, scratch_floats, host_err, n_states, padded_len, row_shift)
+                   : run_prefill_t<__nv_bfloat16, 128>(a, kk, vv, qq, P, stream, launches, S, scratch_floats, host_err, n_states, padded_len, row_shift);
 }
 
 // ---- scratch of mkv_prefill_static -------------------------------------------------------------------------
@@ -689,11 +690,11 @@ cudaError_t static_scratch_address(int device, float **out)
 
 cudaError_t run_prefill(const DecodeArgs &a, bool f32, int D, const void *k, const void *v, const void *q_window, int P,
                         cudaStream_t stream, unsigned long long *launches, PrefillScratch *scratch, int n_states,
-                        int padded_len)
+                        int padded_len, const int *row_shift)
 {
     const int Rw = P < a.R ? P : a.R;
     const bool tc = prefill_tc_supported(f32, D, a.Gq, a.R, k, q_window, P) && tc_padded_group(a.Gq) == a.G;
-    const size_t per_unit = (tc ? prefill_tc_floats_per_unit(P, Rw, a.G, prefill_tc_run(a.U, P))
+    const size_t per_unit = (tc ? prefill_tc_floats_per_unit(P, Rw, a.G, prefill_tc_run(a, P, row_shift))
                                 : (size_t)Rw * a.G * P + P) * sizeof(float);
     size_t ub = ((size_t)1 << 30) / per_unit;
     if (ub < 1) ub = 1;
@@ -716,7 +717,7 @@ cudaError_t run_prefill(const DecodeArgs &a, bool f32, int D, const void *k, con
         scratch->host_err = nullptr;
     }
     return dispatch_prefill(a, f32, D, k, v, q_window, P, stream, launches, static_cast<float *>(scratch->ptr),
-                            scratch->bytes / sizeof(float), scratch->host_err, n_states, padded_len);
+                            scratch->bytes / sizeof(float), scratch->host_err, n_states, padded_len, row_shift);
 }
 
 namespace {
@@ -747,7 +748,7 @@ cudaError_t run_prefill_static(const DecodeArgs &a, bool f32, int D, const void 
     float *S = nullptr;
     const cudaError_t e = static_scratch_address(device, &S);
     if (e != cudaSuccess) return e;
-    return dispatch_prefill(a, f32, D, k, v, q_window, P, stream, launches, S, kStaticScratchFloats, nullptr, n_states, P);
+    return dispatch_prefill(a, f32, D, k, v, q_window, P, stream, launches, S, kStaticScratchFloats, nullptr, n_states, P, nullptr);
 }
 
 }  // namespace mkv

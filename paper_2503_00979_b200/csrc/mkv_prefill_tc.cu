@@ -37,6 +37,7 @@
 
 #include "mkv_common.cuh"
 #include "mkv_kernels.h"
+#include "mkv_schedule.h"
 #include "mkv_sm100.cuh"
 
 namespace mkv {
@@ -54,7 +55,7 @@ constexpr int kPfMerge = 16;                 // statistics merged at a time
 enum PfWait { kPfKEmpty = 21, kPfKFull, kPfTEmpty, kPfTFull, kPfDrain, kPfDEmpty, kPfDFull, kPfQEmpty, kPfQFull, kPfNEmpty, kPfNFull,
               kPfSEmpty, kPfSFull, kPfFlag, kPfPair };
 
-// Rows of different lengths go through the same launches (rowmap): runs beyond the end of a unit's prompt are passed over.
+// Rows of different lengths go through the same launches (rowmap); a unit has the runs of its own prompt.
 struct PfArgs {
     float *part_ml;              // [nb][runs][qrows][2] (max, sum) of a run per window row, log2 domain
     float *ring_c;               // [U][R][G] arena: normaliser of the row of position p in ring slot p % R
@@ -73,7 +74,9 @@ struct PfArgs {
     int accumulate;              // fuse the scores into Fp (a later piece) instead of writing them
     int qrows;                   // rows padded to a multiple of 128 (statistics: MMA M blocks)
     int rpad;                    // rows padded to a multiple of 32 (scores: MMA N)
-    int run, runs, lag;          // tiles of a run, runs of the longest prompt, distance of its two visits
+    int run, runs;               // tiles of a run, runs of the longest prompt
+    RunOrder order;              // of the batch's units' runs (order.shift: in this device's memory)
+    int items, lag;              // runs of the batch's units, distance of a run's two visits in runs
     int select;                  // 0: nothing has to be selected, the normalisers are all there is to do
     int visit;                   // 0: both visits in this launch; 1, 2: one of them
     int stages, bufs;            // K stages, TMEM accumulator buffers (as many as fit 512 columns)
@@ -83,7 +86,7 @@ struct PfArgs {
 
 struct PfItem { int kind, ul, tile0, ntile; };        // kind: 0 none left, 1 statistics, 2 scores
 
-struct PfSmem { int q, kst, negc, stat, pair, desc, bars, total; };
+struct PfSmem { int q, kst, negc, stat, pair, desc, bars, table, total; };
 __host__ __device__ inline PfSmem pf_smem(int qrows, int stages)
 {
     PfSmem L;
@@ -95,20 +98,16 @@ __host__ __device__ inline PfSmem pf_smem(int qrows, int stages)
     L.pair = o; o += 2 * 128 * 4;                              // scores over the rows from 128 on, of two buffers' keys
     L.desc = o; o += kPfDesc * 16;
     L.bars = o; o += 512;
+    L.table = o; o += (kRunTable + 1) * 4;
     L.total = o;
     return L;
 }
 
-// The t-th item of the launch: false beyond the last one.  Statistics of run i come before its scores, by `lag` runs.
+// The t-th item of the launch: false beyond the last one.
 __device__ __forceinline__ bool pf_item(const PfArgs &a, int t, int *kind, int *i)
 {
-    const int n1 = a.nb * a.runs, lag = min(a.lag, n1), both = 2 * (n1 - lag);
-    if (a.visit != 0 || !a.select) { *kind = a.visit == 2 ? 2 : 1; *i = t; return t < n1; }
-    if (t < lag) { *kind = 1; *i = t; return true; }
-    const int s = t - lag;
-    if (s < both) { *kind = 1 + (s & 1); *i = (s >> 1) + ((s & 1) ? 0 : lag); return true; }
-    *kind = 2; *i = s - both + (both >> 1);
-    return *i < n1;
+    if (a.visit != 0 || !a.select) { *kind = a.visit == 2 ? 2 : 1; *i = t; return t < a.items; }
+    return prompt_item(t, a.items, a.lag, kind, i);
 }
 
 // Waits for the flag that another CTA raises; bounded like mbar_wait.
@@ -217,6 +216,7 @@ prefill_tc_kernel(const __grid_constant__ PfArgs a, const __grid_constant__ CUte
     volatile int *abort_flag = reinterpret_cast<volatile int *>(bars + 37);
     int *last_s = reinterpret_cast<int *>(bars + 38);
     const uint32_t bar_pair = smem_u32(bars + 39);
+    int *table = reinterpret_cast<int *>(smem + L.table);                  // RunOrder::place
     const long long WL = a.wait_cycles;
 
     if (tid == 0) {
@@ -236,6 +236,9 @@ prefill_tc_kernel(const __grid_constant__ PfArgs a, const __grid_constant__ CUte
         fence_barrier_init();
     }
     if (warp == 1) tmem_alloc(smem_u32(tmem_slot), 512);
+    // (the rows' lengths were there before the first launch of the chain)
+    const int entries = a.order.entries;
+    for (int e = tid; e < entries; e += kPfThreads) table[e + 1] = a.order.entry(e);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -256,6 +259,18 @@ prefill_tc_kernel(const __grid_constant__ PfArgs a, const __grid_constant__ CUte
 
     if (warp == 0) {
         // ------------------------------------------------ tickets, queries, K tiles (one lane)
+        for (int e0 = 0, sum = 0; e0 < entries; e0 += 32) {
+            int v = e0 + lane < entries ? table[e0 + lane + 1] : 0;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int up = __shfl_up_sync(0xffffffffu, v, o);
+                if (lane >= o) v += up;
+            }
+            if (e0 + lane < entries) table[e0 + lane + 1] = sum + v;
+            if (e0 + lane == 0) table[0] = 0;
+            sum += __shfl_sync(0xffffffffu, v, 31);
+        }
+        __syncwarp();
         if (lane == 0) {
             // the keys stay in L2 between their two visits, and are not needed there afterwards
             const uint64_t pol_first = l2_policy_evict_normal(), pol_last = l2_policy_evict_first();
@@ -266,17 +281,17 @@ prefill_tc_kernel(const __grid_constant__ PfArgs a, const __grid_constant__ CUte
                 const int t = ticket;
                 ticket = atomicAdd(a.ticket, 1);               // (on its way while this one is worked on)
                 PfItem x;
-                int i;
-                bool more = pf_item(a, t, &x.kind, &i);
+                int i, u, r;
+                const bool more = pf_item(a, t, &x.kind, &i);
                 if (more) {
-                    x.ul = i / a.runs;
-                    x.tile0 = (i - x.ul * a.runs) * a.run;
-                    const int P = a.P - a.rowmap(a.ub0 + x.ul), Rw = min(P, a.R);
+                    const int P = a.order.place(i, table, &u, &r), Rw = min(P, a.R);
+                    x.ul = u - a.ub0;
+                    x.tile0 = r * a.run;
                     const int nkeys = x.kind == 1 ? P : P - Rw;
                     x.ntile = min(a.run, (nkeys + kTile - 1) / kTile - x.tile0);
                     if (x.kind == 2 && (!a.select || P - Rw <= a.C)) x.ntile = 0;        // a prompt that is kept whole
                     if (x.ntile <= 0) {
-                        if (a.visit != 2 || x.tile0 != 0) continue;        // nothing to do, or beyond this unit's prompt
+                        if (a.visit != 2 || x.tile0 != 0) continue;        // no candidates in the run
                         x.ntile = 0;                                       // (the unit's normalisers are merged)
                     }
                     if (Rw <= a.i0) continue;                              // a piece of the window that the unit does not have
@@ -291,7 +306,7 @@ prefill_tc_kernel(const __grid_constant__ PfArgs a, const __grid_constant__ CUte
                 ++items;
                 if (!more) break;
                 if (x.ntile == 0) continue;
-                const int qs = queries & 1, u = a.ub0 + x.ul;
+                const int qs = queries & 1;
                 ok = mbar_wait(bar_qempty + 8 * qs, (uint32_t)(((queries >> 1) & 1) ^ 1), abort_flag, kPfQEmpty, WL);
                 if (!ok) break;
                 // K-major with the 128-byte swizzle the MMA descriptors expect: two 64-column panels of QR rows; heads and window
@@ -650,7 +665,7 @@ cudaError_t launch_scores(const PfArgs &a, const CUtensorMap &tmK, const CUtenso
     const int smem = pf_smem(a.qrows, a.stages).total + 1024;
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    return launch_chained(kern, dim3((unsigned)std::min(kPfSm, a.nb * a.runs)), kPfThreads, smem, stream, a, tmK, tmQ);
+    return launch_chained(kern, dim3((unsigned)std::min(kPfSm, a.items)), kPfThreads, smem, stream, a, tmK, tmQ);
 }
 
 // The window queries [units][heads][slots][128] as boxes of `slots` window slots x `group` heads x 64 columns: window slot by window
@@ -681,10 +696,11 @@ bool prefill_tc_supported(bool f32, int D, int G, int R, const void *k, const vo
 // Tiles of an item.  Eight: an item then brings 256 KB of keys beside the 32 KB of its queries, while the items between the two
 // visits of a run stay in L2 (256 units x 6144 tokens: 355 us with four, 334 with eight, 330 with sixteen at the time); fewer where
 // that leaves CTAs without items.
-int prefill_tc_run(int units, int P)
+int prefill_tc_run(const DecodeArgs &a, int P, const int *row_shift)
 {
-    const long long tiles = (long long)units * ((P + kTile - 1) / kTile);
-    return (int)std::min<long long>(8, std::max<long long>(1, (tiles + 2 * kPfSm - 1) / (2 * kPfSm)));
+    int tiles;
+    run_order(row_shift, P, a.Hkv, a.B, 1, 0, a.U, &tiles);
+    return std::min(8, std::max(1, (tiles + 2 * kPfSm - 1) / (2 * kPfSm)));
 }
 
 static int pf_runs(int P, int run) { return ((P + kTile - 1) / kTile + run - 1) / run; }
@@ -700,7 +716,7 @@ size_t prefill_tc_floats_per_unit(int P, int Rw, int G, int run)
 // Window-row normalisers into ring_c and, if `select`, fused scores of the prompt's older tokens into Fp [nb][P] for units
 // ub0 .. ub0+nb-1.  `part` holds the statistics of `units` >= nb units; `words`: prefill_tc_words_per_unit words a unit and two more that are
 // zero, and are again afterwards; `err` is a zeroed error word.
-cudaError_t run_prefill_scores_tc(const DecodeArgs &a, const void *k, const void *qwin, int P, int Ps, int ub0, int nb, int units, int run, bool select,
+cudaError_t run_prefill_scores_tc(const DecodeArgs &a, const void *k, const void *qwin, int P, int Ps, const int *row_shift, int ub0, int nb, int units, int run, bool select,
                                   float *Fp, float *part, int *words, int *err, unsigned long long *launches, cudaStream_t stream)
 {
     CUtensorMap tmK, tmQ;
@@ -712,20 +728,20 @@ cudaError_t run_prefill_scores_tc(const DecodeArgs &a, const void *k, const void
     pa.flag = words; pa.ticket = words + units; pa.left = pa.ticket + 1; pa.done = pa.left + 1; pa.err = err;
     pa.ub0 = ub0; pa.nb = nb; pa.P = P; pa.C = a.C; pa.rowmap = {a.row_shift, a.Hkv, a.B}; pa.G = a.G; pa.R = a.R; pa.Gq = a.Gq;
     pa.run = run; pa.runs = pf_runs(P, run);
+    pa.order = run_order(row_shift, P, a.Hkv, a.B, run, ub0, nb, &pa.items);
+    pa.order.shift = a.row_shift;
     pa.select = select ? 1 : 0;
     pa.scale2 = a.scale2;
     pa.wait_cycles = kWaitCycles;
-    // A unit's last statistics are published some two items after they have been handed out, while every CTA takes two items of
-    // either kind: with fewer than some 200 runs in between the scores wait for them (256 units x 6144: 317 us with 170, 297 with 220,
-    // 295 with 340; x 131072, where the lag holds 32 MB of the unit itself, 150 and 240 are alike).  Of prompts of different
-    // lengths a third of the runs or so are empty.
-    pa.lag = pa.runs + (a.row_shift ? 400 : 240);
+    pa.lag = prompt_lag(pa.items, pa.runs);
     // One launch per visit where the batch's keys stay in L2 by themselves (64 MB), the second of which merges the statistics: the
     // normalisers then take the end of a launch instead of a chain of tickets and a flag (prompt phase in us, one launch -> two;
     // units x tokens, 128 rows: 2 x 900 69 -> 63, 64 x 2000 97 -> 90, 128 x 2000 122 -> 115, 256 x 2000 160 -> 163, 256 x 6144 285 -> 299;
     // 32 x 3000 with 800 rows 270 -> 242).  Not where nothing is selected, as the second visit then has nothing else to do (32 x 600
     // 59 -> 62), unless there are fewer tiles than SMs, nor where a unit's runs are too many for every item to merge.
-    const bool apart = (long long)nb * ((P + kTile - 1) / kTile) <= (select ? kPfL2Tiles : kPfSm) && pa.runs <= kPfMerge;
+    int tiles;
+    run_order(row_shift, P, a.Hkv, a.B, 1, ub0, nb, &tiles);
+    const bool apart = tiles <= (select ? kPfL2Tiles : kPfSm) && pa.runs <= kPfMerge;
     // up to 256 window rows per launch; the rows of a wider window are taken in pieces of whole window
     // slots, whose normalisers are independent and whose scores fuse associatively (Eq. 5 / 6)
     for (int i0 = 0; i0 < Rw; i0 += slots_per_piece) {

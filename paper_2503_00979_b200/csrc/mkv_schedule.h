@@ -1,6 +1,6 @@
-// Work schedule of the tensor-core decode kernel: plain integer arithmetic, compiled for the device by nvcc
-// and for the host by any C++ compiler (the CPU tests replay it for every cache length and check that every
-// tile has exactly one owner and that the partial slots suffice).
+// Work schedules of the tensor-core decode kernel and of the prompt phase's scoring: plain integer arithmetic, compiled for
+// the device by nvcc and for the host by any C++ compiler (the CPU tests replay them: for every cache length that every
+// tile has exactly one owner and that the partial slots suffice, for prompts that every run is visited once).
 #pragma once
 
 #if defined(__CUDACC__)
@@ -177,5 +177,98 @@ inline int sched_partials_per_unit(int U, int cap, int grid)
     }
     return worst;
 }
+
+// ---- prompt phase: the key tiles of a unit's prompt in runs of `run` tiles (the last one shorter), unit after unit
+constexpr int kRunTable = 512;       // most entries of the table of the rows' runs
+
+struct RunOrder {
+    const int *shift;              // [B] how much shorter a batch row's prompt is than the longest one, or nullptr
+    int P, Hkv, B, run, most;      // most: runs of the longest prompt
+    int u0;                        // first unit of the batch; with prompts of different lengths also
+    int first, layer;              // the runs of the units before it, and of the units of a layer
+    int step, entries;             // batch rows of a table entry, entries
+    MKV_HD int runs(int b) const
+    {
+        const int tiles = (P - (shift != nullptr ? shift[b] : 0) + kSchedTile - 1) / kSchedTile;
+        return (tiles + run - 1) / run;
+    }
+    // runs of one unit of each of the rows e * step .. (e + 1) * step - 1
+    MKV_HD int entry(int e) const
+    {
+        int n = 0;
+        for (int b = e * step; b < (e + 1) * step && b < B; ++b) n += runs(b);
+        return n;
+    }
+    // The i-th run from the first one of unit u0 on: its unit and which of the unit's runs it is; returns the length of the unit's
+    // prompt.  `before`: the sum of the entries in front of each entry and, behind the last one, of them all (not used where the
+    // lengths are equal).  It is on the way of a CTA's next loads, so two divisions are all it takes.
+    MKV_HD int place(int i, const int *before, int *unit, int *r) const
+    {
+        if (shift == nullptr) {
+            const int u = (int)((unsigned)i / (unsigned)most);
+            *unit = u0 + u;
+            *r = i - u * most;
+            return P;
+        }
+        i += first;
+        const int l = (int)((unsigned)i / (unsigned)layer);
+        i -= l * layer;
+        int lo = 0, hi = entries;
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (before[mid] * Hkv <= i) lo = mid;
+            else hi = mid;
+        }
+        i -= before[lo] * Hkv;
+        int b = lo * step, n = before[lo + 1] - before[lo];
+        if (step > 1) {
+            n = runs(b);
+            while (i >= n * Hkv) { i -= n * Hkv; n = runs(++b); }
+        }
+        const int len = P - shift[b], h = (int)((unsigned)i / (unsigned)n);
+        *unit = (l * B + b) * Hkv + h;
+        *r = i - h * n;
+        return len;
+    }
+};
+
+// The order of the runs of units u0 .. u0 + count - 1, and their number.
+inline RunOrder run_order(const int *shift, int P, int Hkv, int B, int run, int u0, int count, int *items)
+{
+    RunOrder o = {shift, P, Hkv, B, run, ((P + kSchedTile - 1) / kSchedTile + run - 1) / run, u0, 0, 0, 0, 0};
+    if (shift == nullptr) { *items = count * o.most; return o; }
+    o.step = (B + kRunTable - 1) / kRunTable;
+    o.entries = (B + o.step - 1) / o.step;
+    for (int b = 0; b < B; ++b) o.layer += o.runs(b) * Hkv;
+    auto before = [&](int u) {
+        const int row = u / Hkv;
+        int n = row / B * o.layer + (u - row * Hkv) * o.runs(row % B);
+        for (int b = 0; b < row % B; ++b) n += o.runs(b) * Hkv;
+        return n;
+    };
+    o.first = before(u0);
+    *items = before(u0 + count) - o.first;
+    return o;
+}
+
+// The t-th item of a launch that visits each of `items` runs twice: false beyond the last one.  *kind 1: the first visit of run *i,
+// 2: its second one, which comes behind the first visits of the `lag` runs after it.
+MKV_HD inline bool prompt_item(int t, int items, int lag, int *kind, int *i)
+{
+    if (lag > items) lag = items;
+    const int s = t - lag, both = 2 * (items - lag);
+    if (s < 0) { *kind = 1; *i = t; return true; }
+    if (s < both) { *kind = 1 + (s & 1); *i = (s >> 1) + ((s & 1) ? 0 : lag); return true; }
+    *kind = 2;
+    *i = s - both + (both >> 1);
+    return *i < items;
+}
+
+// Distance of the two visits, in runs (none of which is empty, whatever the prompts' lengths).  A unit's last statistics are
+// published some two items after they have been handed out, while every CTA takes two items of either kind: with fewer than some
+// 200 runs in between the scores wait for them.  With more the keys in between leave L2, which costs little where the launch
+// ends soon after (us, prompt phase, 200 / 240 / 300 / 400 runs in between; units x tokens: 64 x 9000 222 / 215 / 211 / 210, 256 x 4000 372 / 365 / 359 / 360,
+// 256 x 6144 298 / 295 / 293 / 290; 2048 x 3000 1030 / 1032 / 1054 / 1068, 256 x 131072 3341 / 3319 / 3546 / 3585).
+MKV_HD inline int prompt_lag(int items, int longest_runs) { return longest_runs + (items <= 2048 ? 400 : 240); }
 
 }  // namespace mkv

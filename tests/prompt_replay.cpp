@@ -1,0 +1,70 @@
+// Replays the order in which the prompt phase's scoring visits the key tiles, for prompts of the given lengths, and checks what
+// the kernel relies on:
+//   - every run of every unit's own prompt is visited once by each kind of item, in the units' order, and no other run is;
+//   - between a unit's last first visit and its first second visit lie the first visits of 240 other runs at least (all that are left at the
+//     end), so that its statistics are there in time, and a run's visits are no further apart than the longest prompt and those;
+//   - the host's counts of runs agree with the order, also for batches that start and end inside a row, and the table of a layer's
+//     runs has room for any number of rows.
+// usage: prompt_replay Hkv layers run P shift_0 .. shift_{B-1} (no shifts: B = 1, equal lengths)   -> "ok <items>" or a diagnostic
+#include <cstdio>
+#include <cstdlib>
+#include <vector>
+
+#include "mkv_schedule.h"
+
+using namespace mkv;
+
+#define CHECK(c) do { if (!(c)) { printf("line %d: %s\n", __LINE__, #c); return 1; } } while (0)
+
+int main(int argc, char **argv)
+{
+    if (argc < 5) { fprintf(stderr, "usage: %s Hkv layers run P shift...\n", argv[0]); return 2; }
+    const int Hkv = atoi(argv[1]), layers = atoi(argv[2]), run = atoi(argv[3]), P = atoi(argv[4]);
+    std::vector<int> shift;
+    for (int i = 5; i < argc; ++i) shift.push_back(atoi(argv[i]));
+    const int B = shift.empty() ? 1 : (int)shift.size(), U = layers * B * Hkv;
+    const int *sh = shift.empty() ? nullptr : shift.data();
+    const int longest = ((P + 127) / 128 + run - 1) / run;
+    long long seen_total = 0;
+    for (int u0 : {0, 1, Hkv, U / 3, U - 1}) {
+        const int count = u0 == 0 ? U : (U - u0 + 1) / 2;
+        if (u0 < 0 || u0 >= U || count < 1) continue;
+        std::vector<int> unit, r;                                  // the runs, one after the other
+        for (int u = u0; u < u0 + count; ++u) {
+            const int len = P - (sh ? sh[(u / Hkv) % B] : 0), n = ((len + 127) / 128 + run - 1) / run;
+            for (int k = 0; k < n; ++k) { unit.push_back(u); r.push_back(k); }
+        }
+        const int items = (int)unit.size();
+        int counted = -1;
+        const RunOrder order = run_order(sh, P, Hkv, B, run, u0, count, &counted);
+        CHECK(counted == items);
+        std::vector<int> before(1, 0);
+        for (int e = 0; e < order.entries; ++e) before.push_back(before.back() + order.entry(e));
+        CHECK((int)before.size() <= kRunTable + 1 && (!sh || before.back() * Hkv == order.layer));
+        const int lag = prompt_lag(items, longest);
+        CHECK(lag - longest >= 240 && lag - longest <= 400);
+        std::vector<int> at1(items, -1), at2(items, -1);
+        for (int t = 0;; ++t) {
+            int kind, i, u, k;
+            if (!prompt_item(t, items, lag, &kind, &i)) { CHECK(t == 2 * items); break; }
+            CHECK(i >= 0 && i < items);
+            CHECK(order.place(i, before.data(), &u, &k) == P - (sh ? sh[(unit[i] / Hkv) % B] : 0));
+            CHECK(u == unit[i] && k == r[i]);
+            std::vector<int> &at = kind == 1 ? at1 : at2;
+            CHECK(at[i] < 0 && (i == 0 || at[i - 1] >= 0));
+            at[i] = t;
+        }
+        for (int i = 0; i < items; ++i) {
+            CHECK(at1[i] >= 0 && at2[i] > at1[i]);
+            if (r[i] != 0) continue;
+            int last = i;                                          // the unit's last run
+            while (last + 1 < items && unit[last + 1] == unit[i]) ++last;
+            const int need = items - 1 - last < 240 ? items - 1 - last : 240;
+            for (int k = 1; k <= need; ++k) CHECK(at1[last + k] < at2[i]);
+            if (i + lag + 1 < items) CHECK(at1[i + lag + 1] > at2[i]);
+        }
+        seen_total += items;
+    }
+    printf("ok %lld\n", seen_total);
+    return 0;
+}
