@@ -49,8 +49,6 @@ constexpr int kPfFirstConsumer = 8, kPfFirstPublisher = 4;
 constexpr int kPfThreads = 32 * (kPfFirstConsumer + 4 * kPfGroups);
 constexpr int kPfDesc = 4;                   // item descriptors in flight
 constexpr int kPfMaxStages = 4;
-constexpr int kPfSm = 148;
-constexpr int kPfL2Tiles = 2048;             // 64 MB of keys
 constexpr int kPfMerge = 16;                 // statistics merged at a time
 enum PfWait { kPfKEmpty = 21, kPfKFull, kPfTEmpty, kPfTFull, kPfDrain, kPfDEmpty, kPfDFull, kPfQEmpty, kPfQFull, kPfNEmpty, kPfNFull,
               kPfSEmpty, kPfSFull, kPfFlag, kPfPair };
@@ -219,21 +217,21 @@ prefill_tc_kernel(const __grid_constant__ PfArgs a, const __grid_constant__ CUte
     int *table = reinterpret_cast<int *>(smem + L.table);                  // RunOrder::place
     const long long WL = a.wait_cycles;
 
-    if (tid == 0) {
+    // one barrier each: the launch's start is in the way of the first copies
+    if (tid < 38) {
+        int n = 1;                                              // the pairs and fours "full": one arrival, and the copies' bytes
+        if (tid >= 12 && tid < 16) n = 4 * kPfGroups / NB;      // tempty
+        else if (tid >= 20 && tid < 24) n = 3 + 4 + 4 * kPfGroups;     // dempty: the MMA warps, the normalisers' warp, four publishing and all consumer warps
+        else if (tid == 26 || tid == 27) n = 2;                 // qempty
+        else if (tid >= 30 && tid < 34) n = 4 * kPfGroups;      // nempty, sfull
+        else if (tid >= 34) n = 4;                              // sempty, pair
+        mbar_init(smem_u32(bars + (tid < 36 ? tid : tid + 3)), (uint32_t)n);
+        fence_barrier_init();
+    }
+    if (tid == 64) {
         prefetch_tensormap(&tmK);
         prefetch_tensormap(&tmQ);
-        for (int s = 0; s < ST; ++s) { mbar_init(bar_kfull + 8 * s, 1); mbar_init(bar_kempty + 8 * s, 1); }
-        for (int b = 0; b < NB; ++b) { mbar_init(bar_tfull + 8 * b, 1); mbar_init(bar_tempty + 8 * b, 4 * kPfGroups / NB); }
-        // a descriptor is read by the MMA warps, the normalisers' warp, four publishing and all consumer warps
-        for (int i = 0; i < kPfDesc; ++i) { mbar_init(bar_dfull + 8 * i, 1); mbar_init(bar_dempty + 8 * i, 3 + 4 + 4 * kPfGroups); }
-        for (int i = 0; i < 2; ++i) {
-            mbar_init(bar_qfull + 8 * i, 1); mbar_init(bar_qempty + 8 * i, 2);
-            mbar_init(bar_nfull + 8 * i, 1); mbar_init(bar_nempty + 8 * i, 4 * kPfGroups);
-            mbar_init(bar_sfull + 8 * i, 4 * kPfGroups); mbar_init(bar_sempty + 8 * i, 4);
-            mbar_init(bar_pair + 8 * i, 4);
-        }
         *abort_flag = 0;
-        fence_barrier_init();
     }
     if (warp == 1) tmem_alloc(smem_u32(tmem_slot), 512);
     // (the rows' lengths were there before the first launch of the chain)
@@ -276,10 +274,15 @@ prefill_tc_kernel(const __grid_constant__ PfArgs a, const __grid_constant__ CUte
             const uint64_t pol_first = l2_policy_evict_normal(), pol_last = l2_policy_evict_first();
             bool ok = true;
             int issued = 0, items = 0, queries = 0;
-            int ticket = atomicAdd(a.ticket, 1);
+            // Items are taken by ticket, the next one's on its way while this one is worked on.  In the launches of one visit of two,
+            // whose items are few and about as long, a CTA has its own: one that starts early would take two while others get none.  They
+            // are one place further on in every round, or the units' shorter last runs could all be the same CTAs'.
+            const bool tickets = a.visit == 0;
+            int ticket = tickets ? atomicAdd(a.ticket, 1) : (int)blockIdx.x, round = 0;
             while (ok) {
                 const int t = ticket;
-                ticket = atomicAdd(a.ticket, 1);               // (on its way while this one is worked on)
+                ++round;
+                ticket = tickets ? atomicAdd(a.ticket, 1) : round * (int)gridDim.x + ((int)blockIdx.x + round) % (int)gridDim.x;
                 PfItem x;
                 int i, u, r;
                 const bool more = pf_item(a, t, &x.kind, &i);
@@ -526,7 +529,7 @@ prefill_tc_kernel(const __grid_constant__ PfArgs a, const __grid_constant__ CUte
             }
             for (int row = pt; row < rows; row += kGroupThreads) to_ring(row, ncl > 1 ? merged(row, 0, kPfMerge, nrun) : merged(row, 0, 1, nrun));
             group_sync(kBar, kGroupThreads);
-            if (pt == 0) asm volatile("st.release.gpu.global.s32 [%0], 1;" ::"l"(a.flag + x.ul) : "memory");
+            if (pt == 0 && a.select) asm volatile("st.release.gpu.global.s32 [%0], 1;" ::"l"(a.flag + x.ul) : "memory");
         }
     } else if (warp >= kPfFirstConsumer) {
         // ------------------------------------------------ consumers: tile T is in buffer T % NB, the business of the groups grp
@@ -563,10 +566,10 @@ prefill_tc_kernel(const __grid_constant__ PfArgs a, const __grid_constant__ CUte
                             // The reference is the maximum so far, rounded up: the weights that count have exponents near 0, and factors
                             // between references, here and where sums are merged, are whole powers of two.  The scale is positive, so
                             // the maximum is taken on the raw logits and scaled once.
-                            float cm = -INFINITY;
+                            float c4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-                            for (int i = 0; i < 32; ++i) cm = fmaxf(cm, __uint_as_float(v[i]));
-                            cm *= a.scale2;
+                            for (int i = 0; i < 32; ++i) c4[i & 3] = fmaxf(c4[i & 3], __uint_as_float(v[i]));
+                            const float cm = fmaxf(fmaxf(c4[0], c4[1]), fmaxf(c4[2], c4[3])) * a.scale2;
                             if (cm > m) {
                                 const float up = ceilf(cm);
                                 l *= ex2f(m - up);
@@ -646,8 +649,9 @@ prefill_tc_kernel(const __grid_constant__ PfArgs a, const __grid_constant__ CUte
         tc_fence_after();
         tmem_dealloc(tmem_base, 512);
     }
+    if (tid == 0 && *abort_flag) atomicCAS(a.err, 0, *abort_flag);
+    if (a.visit != 0) return;                                  // (no ticket was taken, no flag is looked at)
     if (tid == 0) {
-        if (*abort_flag) atomicCAS(a.err, 0, *abort_flag);
         __threadfence();
         *last_s = atomicAdd(a.left, 1) == (int)gridDim.x - 1;
     }
@@ -665,7 +669,7 @@ cudaError_t launch_scores(const PfArgs &a, const CUtensorMap &tmK, const CUtenso
     const int smem = pf_smem(a.qrows, a.stages).total + 1024;
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    return launch_chained(kern, dim3((unsigned)std::min(kPfSm, a.items)), kPfThreads, smem, stream, a, tmK, tmQ);
+    return launch_chained(kern, dim3((unsigned)std::min(kPromptCtas, a.items)), kPfThreads, smem, stream, a, tmK, tmQ);
 }
 
 // The window queries [units][heads][slots][128] as boxes of `slots` window slots x `group` heads x 64 columns: window slot by window
@@ -693,15 +697,7 @@ bool prefill_tc_supported(bool f32, int D, int G, int R, const void *k, const vo
     return !f32 && D == kD && G >= 1 && G <= kMaxGroup && R >= 1 && (((uintptr_t)k | (uintptr_t)qwin) & 15) == 0 && P >= 1;
 }
 
-// Tiles of an item.  Eight: an item then brings 256 KB of keys beside the 32 KB of its queries, while the items between the two
-// visits of a run stay in L2 (256 units x 6144 tokens: 355 us with four, 334 with eight, 330 with sixteen at the time); fewer where
-// that leaves CTAs without items.
-int prefill_tc_run(const DecodeArgs &a, int P, const int *row_shift)
-{
-    int tiles;
-    run_order(row_shift, P, a.Hkv, a.B, 1, 0, a.U, &tiles);
-    return std::min(8, std::max(1, (tiles + 2 * kPfSm - 1) / (2 * kPfSm)));
-}
+int prefill_tc_run(const DecodeArgs &a, int P, const int *row_shift) { return prompt_run(row_shift, P, a.Hkv, a.B, a.U, std::min(P, a.R) * a.G, P - std::min(P, a.R) > a.C); }
 
 static int pf_runs(int P, int run) { return ((P + kTile - 1) / kTile + run - 1) / run; }
 
@@ -734,14 +730,12 @@ cudaError_t run_prefill_scores_tc(const DecodeArgs &a, const void *k, const void
     pa.scale2 = a.scale2;
     pa.wait_cycles = kWaitCycles;
     pa.lag = prompt_lag(pa.items, pa.runs);
-    // One launch per visit where the batch's keys stay in L2 by themselves (64 MB), the second of which merges the statistics: the
-    // normalisers then take the end of a launch instead of a chain of tickets and a flag (prompt phase in us, one launch -> two;
-    // units x tokens, 128 rows: 2 x 900 69 -> 63, 64 x 2000 97 -> 90, 128 x 2000 122 -> 115, 256 x 2000 160 -> 163, 256 x 6144 285 -> 299;
-    // 32 x 3000 with 800 rows 270 -> 242).  Not where nothing is selected, as the second visit then has nothing else to do (32 x 600
-    // 59 -> 62), unless there are fewer tiles than SMs, nor where a unit's runs are too many for every item to merge.
+    // One launch per visit where the batch's keys stay in L2 by themselves, the second of which merges the statistics: the normalisers
+    // then take the end of a launch instead of a chain of tickets and a flag.  Not where nothing is selected, as the second visit then has
+    // nothing else to do (32 units x 600 tokens 59 -> 62), unless there are fewer tiles than SMs.
     int tiles;
     run_order(row_shift, P, a.Hkv, a.B, 1, ub0, nb, &tiles);
-    const bool apart = tiles <= (select ? kPfL2Tiles : kPfSm) && pa.runs <= kPfMerge;
+    const bool apart = tiles <= (select ? prompt_apart_tiles(Rw * a.G) : kPromptCtas);
     // up to 256 window rows per launch; the rows of a wider window are taken in pieces of whole window
     // slots, whose normalisers are independent and whose scores fuse associatively (Eq. 5 / 6)
     for (int i0 = 0; i0 < Rw; i0 += slots_per_piece) {

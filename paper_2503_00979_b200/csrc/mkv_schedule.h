@@ -251,6 +251,40 @@ inline RunOrder run_order(const int *shift, int P, int Hkv, int B, int run, int 
     return o;
 }
 
+constexpr int kPromptCtas = 148;         // CTAs of the scoring's launches
+// Up to how many tiles one launch makes each visit, as their keys stay in L2 (96 MB) by themselves.  With two blocks of rows fewer:
+// what a launch of both visits gains by mixing them grows with the work per tile.  (Prompt phase in us, both visits in one launch -> a
+// launch each; units x tokens, 128 rows: 64 x 2000 97 -> 77, 256 x 1499 139 -> 131, 64 x 6107 137 -> 132, 256 x 2000 156 -> 155; 240 rows:
+// 32 x 9000 161 -> 146, 128 x 3035 178 -> 190.)
+MKV_HD inline int prompt_apart_tiles(int rows) { return rows <= 128 ? 3072 : 2304; }
+
+// Tiles of a run.  Eight for many tiles: an item then brings 256 KB of keys beside the 32 KB of its queries, while the items between
+// the two visits of a run stay in L2 (256 units x 6144 tokens: 355 us with four, 334 with eight, 330 with sixteen at the time).
+// Where nothing is selected, and items are taken by ticket once, two items per CTA.  With a launch for each visit, the length that fills the rounds of items best, in items as short as that allows: an item's own time
+// is some third of a tile's, and more where there are many statistics of its unit to merge.  Rounds of a few items less than there are
+// SMs, as now and then one of them is not free when the launch starts (2 units x 259 tiles, runs of seven: 148 items 127 us or 157).
+// (Before, tiles / 296 and both visits in one launch from 17 runs per unit on -> now: 8 x 25600 104 -> 91, 2 x 60000 120 -> 94, 4 x 40000 with
+// 256 rows 136 -> 115, 112 x 1200 with 240 rows 115 -> 104, 32 x 1500 64 -> 54.)
+inline int prompt_run(const int *shift, int P, int Hkv, int B, int units, int rows, bool select)
+{
+    int tiles, best = 8, least = 0;
+    run_order(shift, P, Hkv, B, 1, 0, units, &tiles);
+    if (tiles > prompt_apart_tiles(rows)) return best;
+    const int longest = (P + kSchedTile - 1) / kSchedTile;
+    if (!select) {
+        const long long run = ((long long)units * longest + 2 * kPromptCtas - 1) / (2 * kPromptCtas);
+        return run < best ? (int)run : best;
+    }
+    for (int run = longest > 1 ? 2 : 1; run <= 24 && run <= longest; ++run) {
+        int items;
+        const RunOrder o = run_order(shift, P, Hkv, B, run, 0, units, &items);
+        const int rounds = (items + kPromptCtas - 5) / (kPromptCtas - 4);
+        const int cost = rounds * (10 * run + 3 + o.most / 4) + run;      // tenths of a tile
+        if (least == 0 || cost < least) { least = cost; best = run; }
+    }
+    return best;
+}
+
 // The t-th item of a launch that visits each of `items` runs twice: false beyond the last one.  *kind 1: the first visit of run *i,
 // 2: its second one, which comes behind the first visits of the `lag` runs after it.
 MKV_HD inline bool prompt_item(int t, int items, int lag, int *kind, int *i)

@@ -5,7 +5,9 @@
 //     end), so that its statistics are there in time, and a run's visits are no further apart than the longest prompt and those;
 //   - the host's counts of runs agree with the order, also for batches that start and end inside a row, and the table of a layer's
 //     runs has room for any number of rows.
+//   - with run 0: the run that the host chooses leaves no CTA much more than its share of the tiles.
 // usage: prompt_replay Hkv layers run P shift_0 .. shift_{B-1} (no shifts: B = 1, equal lengths)   -> "ok <items>" or a diagnostic
+#include <algorithm>
 #include <cstdio>
 #include <cstdlib>
 #include <vector>
@@ -19,11 +21,36 @@ using namespace mkv;
 int main(int argc, char **argv)
 {
     if (argc < 5) { fprintf(stderr, "usage: %s Hkv layers run P shift...\n", argv[0]); return 2; }
-    const int Hkv = atoi(argv[1]), layers = atoi(argv[2]), run = atoi(argv[3]), P = atoi(argv[4]);
+    const int Hkv = atoi(argv[1]), layers = atoi(argv[2]), P = atoi(argv[4]);
+    int run = atoi(argv[3]);
     std::vector<int> shift;
     for (int i = 5; i < argc; ++i) shift.push_back(atoi(argv[i]));
     const int B = shift.empty() ? 1 : (int)shift.size(), U = layers * B * Hkv;
     const int *sh = shift.empty() ? nullptr : shift.data();
+    if (run == 0) {
+        run = prompt_run(sh, P, Hkv, B, U, 128, true);
+        int items;
+        const RunOrder order = run_order(sh, P, Hkv, B, run, 0, U, &items);
+        std::vector<int> before(1, 0);
+        for (int e = 0; e < order.entries; ++e) before.push_back(before.back() + order.entry(e));
+        std::vector<long long> cta(kPromptCtas, 0);
+        long long all = 0, most = 0;
+        std::vector<int> taken(items, 0);
+        for (int round = 0; round * kPromptCtas < items; ++round)
+        for (int c = 0; c < kPromptCtas; ++c) {                    // (as in a launch of one visit)
+            int u, k;
+            const int t = round * kPromptCtas + (c + round) % kPromptCtas;
+            if (t >= items) continue;
+            CHECK(taken[t]++ == 0);
+            const int len = order.place(t, before.data(), &u, &k), left = (len + 127) / 128 - k * run;
+            const int n = left < run ? left : run;
+            CHECK(n >= 1);
+            all += n;
+            most = std::max(most, cta[c] += n);
+        }
+        printf("run %d, the busiest of %d CTAs has %lld of %lld tiles\n", run, kPromptCtas, most, all);
+        if (all <= prompt_apart_tiles(128)) CHECK(4 * kPromptCtas * (most - 2) <= 5 * all);            // a quarter and two tiles more than its share
+    }
     const int longest = ((P + 127) / 128 + run - 1) / run;
     long long seen_total = 0;
     for (int u0 : {0, 1, Hkv, U / 3, U - 1}) {
