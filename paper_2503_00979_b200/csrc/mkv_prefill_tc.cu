@@ -101,11 +101,20 @@ __host__ __device__ inline PfSmem pf_smem(int qrows, int stages)
     return L;
 }
 
-// The t-th item of the launch: false beyond the last one.
-__device__ __forceinline__ bool pf_item(const PfArgs &a, int t, int *kind, int *i)
+// The t-th item of the launch.
+__device__ __forceinline__ RunVisit pf_item(const PfArgs &a, int t)
 {
-    if (a.visit != 0 || !a.select) { *kind = a.visit == 2 ? 2 : 1; *i = t; return t < a.items; }
-    return prompt_item(t, a.items, a.lag, kind, i);
+    if (a.visit != 0 || !a.select) return RunVisit{a.visit == 2 ? 2 : 1, t, t < a.items};
+    return prompt_item(t, a.items, a.lag);
+}
+
+// The next ticket, or `own`.  (One predicated instruction: with a branch around atomicAdd its result was waited for at once, 2 to 7 % of
+// the prompt phase: 448 units x 66 tokens 91 -> 98 us, 256 x 9000 306 -> 312.)
+__device__ __forceinline__ int take_ticket(int *count, bool tickets, int own)
+{
+    int t = own;
+    asm volatile("{\n.reg .pred p;\nsetp.ne.s32 p, %2, 0;\n@p atom.global.add.s32 %0, [%1], 1;\n}" : "+r"(t) : "l"(count), "r"((int)tickets) : "memory");
+    return t;
 }
 
 // Waits for the flag that another CTA raises; bounded like mbar_wait.
@@ -278,18 +287,22 @@ prefill_tc_kernel(const __grid_constant__ PfArgs a, const __grid_constant__ CUte
             // whose items are few and about as long, a CTA has its own: one that starts early would take two while others get none.  They
             // are one place further on in every round, or the units' shorter last runs could all be the same CTAs'.
             const bool tickets = a.visit == 0;
-            int ticket = tickets ? atomicAdd(a.ticket, 1) : (int)blockIdx.x, round = 0;
+            int place = (int)blockIdx.x, round0 = 0, ticket = take_ticket(a.ticket, tickets, place);
             while (ok) {
                 const int t = ticket;
-                ++round;
-                ticket = tickets ? atomicAdd(a.ticket, 1) : round * (int)gridDim.x + ((int)blockIdx.x + round) % (int)gridDim.x;
+                place = place + 1 == (int)gridDim.x ? 0 : place + 1;
+                round0 += (int)gridDim.x;
+                ticket = take_ticket(a.ticket, tickets, round0 + place);
                 PfItem x;
-                int i, u, r;
-                const bool more = pf_item(a, t, &x.kind, &i);
-                if (more) {
-                    const int P = a.order.place(i, table, &u, &r), Rw = min(P, a.R);
+                int u = 0;
+                const RunVisit v = pf_item(a, t);
+                x.kind = v.kind;
+                if (v.more) {
+                    const RunAt at = a.order.place(v.i, table);
+                    const int P = at.P, Rw = min(P, a.R);
+                    u = at.unit;
                     x.ul = u - a.ub0;
-                    x.tile0 = r * a.run;
+                    x.tile0 = at.r * a.run;
                     const int nkeys = x.kind == 1 ? P : P - Rw;
                     x.ntile = min(a.run, (nkeys + kTile - 1) / kTile - x.tile0);
                     if (x.kind == 2 && (!a.select || P - Rw <= a.C)) x.ntile = 0;        // a prompt that is kept whole
@@ -307,7 +320,7 @@ prefill_tc_kernel(const __grid_constant__ PfArgs a, const __grid_constant__ CUte
                 desc[d] = x;
                 mbar_arrive(bar_dfull + 8 * d);
                 ++items;
-                if (!more) break;
+                if (!v.more) break;
                 if (x.ntile == 0) continue;
                 const int qs = queries & 1;
                 ok = mbar_wait(bar_qempty + 8 * qs, (uint32_t)(((queries >> 1) & 1) ^ 1), abort_flag, kPfQEmpty, WL);
@@ -566,10 +579,10 @@ prefill_tc_kernel(const __grid_constant__ PfArgs a, const __grid_constant__ CUte
                             // The reference is the maximum so far, rounded up: the weights that count have exponents near 0, and factors
                             // between references, here and where sums are merged, are whole powers of two.  The scale is positive, so
                             // the maximum is taken on the raw logits and scaled once.
-                            float c4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+                            float cm = -INFINITY;
 #pragma unroll
-                            for (int i = 0; i < 32; ++i) c4[i & 3] = fmaxf(c4[i & 3], __uint_as_float(v[i]));
-                            const float cm = fmaxf(fmaxf(c4[0], c4[1]), fmaxf(c4[2], c4[3])) * a.scale2;
+                            for (int i = 0; i < 32; ++i) cm = fmaxf(cm, __uint_as_float(v[i]));
+                            cm *= a.scale2;
                             if (cm > m) {
                                 const float up = ceilf(cm);
                                 l *= ex2f(m - up);

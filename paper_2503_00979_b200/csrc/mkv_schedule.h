@@ -181,6 +181,10 @@ inline int sched_partials_per_unit(int U, int cap, int grid)
 // ---- prompt phase: the key tiles of a unit's prompt in runs of `run` tiles (the last one shorter), unit after unit
 constexpr int kRunTable = 512;       // most entries of the table of the rows' runs
 
+struct RunAt {
+    int unit, r, P;                // the unit, which of its runs it is, the length of its prompt
+};
+
 struct RunOrder {
     const int *shift;              // [B] how much shorter a batch row's prompt is than the longest one, or nullptr
     int P, Hkv, B, run, most;      // most: runs of the longest prompt
@@ -199,16 +203,13 @@ struct RunOrder {
         for (int b = e * step; b < (e + 1) * step && b < B; ++b) n += runs(b);
         return n;
     }
-    // The i-th run from the first one of unit u0 on: its unit and which of the unit's runs it is; returns the length of the unit's
-    // prompt.  `before`: the sum of the entries in front of each entry and, behind the last one, of them all (not used where the
+    // The i-th run from the first one of unit u0 on.  `before`: the sum of the entries in front of each entry and, behind the last one, of them all (not used where the
     // lengths are equal).  It is on the way of a CTA's next loads, so two divisions are all it takes.
-    MKV_HD int place(int i, const int *before, int *unit, int *r) const
+    MKV_HD RunAt place(int i, const int *before) const
     {
         if (shift == nullptr) {
             const int u = (int)((unsigned)i / (unsigned)most);
-            *unit = u0 + u;
-            *r = i - u * most;
-            return P;
+            return RunAt{u0 + u, i - u * most, P};
         }
         i += first;
         const int l = (int)((unsigned)i / (unsigned)layer);
@@ -226,9 +227,7 @@ struct RunOrder {
             while (i >= n * Hkv) { i -= n * Hkv; n = runs(++b); }
         }
         const int len = P - shift[b], h = (int)((unsigned)i / (unsigned)n);
-        *unit = (l * B + b) * Hkv + h;
-        *r = i - h * n;
-        return len;
+        return RunAt{(l * B + b) * Hkv + h, i - h * n, len};
     }
 };
 
@@ -285,24 +284,28 @@ inline int prompt_run(const int *shift, int P, int Hkv, int B, int units, int ro
     return best;
 }
 
-// The t-th item of a launch that visits each of `items` runs twice: false beyond the last one.  *kind 1: the first visit of run *i,
+// The t-th item of a launch that visits each of `items` runs twice (`more`: not beyond the last one).  Kind 1: the first visit of run i,
 // 2: its second one, which comes behind the first visits of the `lag` runs after it.
-MKV_HD inline bool prompt_item(int t, int items, int lag, int *kind, int *i)
+struct RunVisit {
+    int kind, i;
+    bool more;
+};
+MKV_HD inline RunVisit prompt_item(int t, int items, int lag)
 {
     if (lag > items) lag = items;
     const int s = t - lag, both = 2 * (items - lag);
-    if (s < 0) { *kind = 1; *i = t; return true; }
-    if (s < both) { *kind = 1 + (s & 1); *i = (s >> 1) + ((s & 1) ? 0 : lag); return true; }
-    *kind = 2;
-    *i = s - both + (both >> 1);
-    return *i < items;
+    if (s < 0) return RunVisit{1, t, true};
+    if (s < both) return RunVisit{1 + (s & 1), (s >> 1) + ((s & 1) ? 0 : lag), true};
+    const int i = s - both + (both >> 1);
+    return RunVisit{2, i, i < items};
 }
 
 // Distance of the two visits, in runs (none of which is empty, whatever the prompts' lengths).  A unit's last statistics are
 // published some two items after they have been handed out, while every CTA takes two items of either kind: with fewer than some
-// 200 runs in between the scores wait for them.  With more the keys in between leave L2, which costs little where the launch
-// ends soon after (us, prompt phase, 200 / 240 / 300 / 400 runs in between; units x tokens: 64 x 9000 222 / 215 / 211 / 210, 256 x 4000 372 / 365 / 359 / 360,
-// 256 x 6144 298 / 295 / 293 / 290; 2048 x 3000 1030 / 1032 / 1054 / 1068, 256 x 131072 3341 / 3319 / 3546 / 3585).
-MKV_HD inline int prompt_lag(int items, int longest_runs) { return longest_runs + (items <= 2048 ? 400 : 240); }
+// 200 runs in between the scores wait for them.  With more the keys in between leave L2 (400 runs of eight tiles are 105 MB), which costs
+// little where the launch ends soon after.  (Prompt phase in us, 200 / 240 / 300 / 400 runs in between; units x tokens: 24 x 17600 133 / 132 / 131 /
+// 120, 64 x 9000 219 / 213 / 207 / 207, 256 x 3500 195 / 190 / 182 / 181; 256 x 6144 292 / 286 / 284 / 282, but 367 at 240 and 371 at 400 with
+// its first step and prompt after prompt; 2048 x 3000 1030 / 1032 / 1054 / 1068, 256 x 131072 3341 / 3319 / 3546 / 3585.)
+MKV_HD inline int prompt_lag(int items, int longest_runs) { return longest_runs + (items <= 1024 ? 400 : 240); }
 
 }  // namespace mkv

@@ -38,11 +38,11 @@ int main(int argc, char **argv)
         std::vector<int> taken(items, 0);
         for (int round = 0; round * kPromptCtas < items; ++round)
         for (int c = 0; c < kPromptCtas; ++c) {                    // (as in a launch of one visit)
-            int u, k;
             const int t = round * kPromptCtas + (c + round) % kPromptCtas;
             if (t >= items) continue;
             CHECK(taken[t]++ == 0);
-            const int len = order.place(t, before.data(), &u, &k), left = (len + 127) / 128 - k * run;
+            const RunAt at = order.place(t, before.data());
+            const int left = (at.P + 127) / 128 - at.r * run;
             const int n = left < run ? left : run;
             CHECK(n >= 1);
             all += n;
@@ -72,11 +72,12 @@ int main(int argc, char **argv)
         CHECK(lag - longest >= 240 && lag - longest <= 400);
         std::vector<int> at1(items, -1), at2(items, -1);
         for (int t = 0;; ++t) {
-            int kind, i, u, k;
-            if (!prompt_item(t, items, lag, &kind, &i)) { CHECK(t == 2 * items); break; }
+            const RunVisit v = prompt_item(t, items, lag);
+            if (!v.more) { CHECK(t == 2 * items); break; }
+            const int i = v.i, kind = v.kind;
             CHECK(i >= 0 && i < items);
-            CHECK(order.place(i, before.data(), &u, &k) == P - (sh ? sh[(unit[i] / Hkv) % B] : 0));
-            CHECK(u == unit[i] && k == r[i]);
+            const RunAt placed = order.place(i, before.data());
+            CHECK(placed.unit == unit[i] && placed.r == r[i] && placed.P == P - (sh ? sh[(unit[i] / Hkv) % B] : 0));
             std::vector<int> &at = kind == 1 ? at1 : at2;
             CHECK(at[i] < 0 && (i == 0 || at[i - 1] >= 0));
             at[i] = t;
