@@ -450,6 +450,8 @@ decode_tc_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ C
     // A layer's launch behind another layer's (`early`) waits where it first needs something of another kernel's: the MMA warp
     // before it reads the new query, the epilogue group before it reads the new rows and writes the output.  State, ring and tiles are
     // this layer's own, complete since the launch before the one before this one (which let this one start after its own wait).
+    // The producers and the compute warps wait for it too before the first of their bounded waits that the MMA warp has to end: the
+    // limit of those does not count what is left of another launch.
     // (us per call in a sequence of layers, wait at the start -> here, 4 heads: 32 units x 1056 slots 17.3 -> 15.7, 64: 20.0 -> 18.1,
     // 256: 36.9 -> 33.8; 32 x 4064 28.0 -> 26.0; 64 x 2048 of 8 heads 35.1 -> 32.5.)
     if (!a.early) {
@@ -507,6 +509,7 @@ decode_tc_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ C
             RingPos rk(0, SK);
             const uint64_t pol_stream = l2_policy_evict_first(), pol_keep = l2_policy_evict_last();
             while (ok && w.next(x)) {
+                if (a.early && rings == 1) asm volatile("griddepcontrol.wait;" ::: "memory");
                 ok = mbar_wait(bar_qempty, (uint32_t)((w.nitems & 1) ^ 1), abort_flag, kWaitQEmpty, WL);
                 if (!ok) break;
                 const int u = MC ? x.unit / NCe : x.unit;
@@ -521,6 +524,7 @@ decode_tc_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ C
                 ++rings;
                 for (int j = 0; j < x.nk && ok; ++j, rk.step(1, SK)) {
                     const int T = w.T0 + j, s = rk.idx;
+                    if (a.early && T == SK) asm volatile("griddepcontrol.wait;" ::: "memory");
                     ok = mbar_wait(bar_kempty + 8 * s, (uint32_t)(rk.lap ^ 1), abort_flag, kWaitKEmpty, WL);
                     if (!ok) break;
                     const int row = (x.tile0 + j) * kTile;
@@ -555,6 +559,7 @@ decode_tc_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ C
                 const bool main_item = MC ? (NCe == 1 || x.unit - u * NCe == c_main) : true;
                 for (int j = 0; main_item && j < x.nk && ok; ++j, rv.step(1, SV)) {
                     const int s = rv.idx;
+                    if (a.early && issued == SV) asm volatile("griddepcontrol.wait;" ::: "memory");
                     ok = mbar_wait(bar_vempty + 8 * s, (uint32_t)(rv.lap ^ 1), abort_flag, kWaitVEmpty, WL);
                     if (!ok) break;
                     const int row = (x.tile0 + j) * kTile;
@@ -676,6 +681,7 @@ decode_tc_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ C
         int Tn = grp;                                  // next tile of this group
         int skipped = 0;                               // MC: tiles of the items that read no V
         RingPos rb(grp, NB), rv(grp, SV);
+        if (a.early) asm volatile("griddepcontrol.wait;" ::: "memory");
         while (w.next(x)) {
             const int u = MC ? x.unit / NCe : x.unit;
             const int cc = MC ? (NCe == 1 ? c_main : x.unit - u * NCe) : 0;      // ring chunk of this item
