@@ -48,7 +48,6 @@ constexpr int kPfGroups = 4;                 // consumer groups of four warps
 constexpr int kPfFirstConsumer = 8, kPfFirstPublisher = 4;
 constexpr int kPfThreads = 32 * (kPfFirstConsumer + 4 * kPfGroups);
 constexpr int kPfDesc = 4;                   // item descriptors in flight
-constexpr int kPfMaxStages = 4;
 constexpr int kPfMerge = 16;                 // statistics merged at a time
 enum PfWait { kPfKEmpty = 21, kPfKFull, kPfTEmpty, kPfTFull, kPfDrain, kPfDEmpty, kPfDFull, kPfQEmpty, kPfQFull, kPfNEmpty, kPfNFull,
               kPfSEmpty, kPfSFull, kPfFlag, kPfPair };
@@ -152,7 +151,6 @@ __device__ __forceinline__ F32x2 pack2(float a, float b) { F32x2 r; asm("mov.b64
 __device__ __forceinline__ float2 unpack2(F32x2 v) { float2 r; asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v)); return r; }
 __device__ __forceinline__ F32x2 fma2(F32x2 a, F32x2 b, F32x2 c) { F32x2 r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
 __device__ __forceinline__ F32x2 add2(F32x2 a, F32x2 b) { F32x2 r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
-__device__ __forceinline__ F32x2 mul2(F32x2 a, F32x2 b) { F32x2 r; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
 __device__ __forceinline__ F32x2 both(float a) { return pack2(a, a); }
 __device__ __forceinline__ F32x2 ex2_pair(F32x2 x)
 {

@@ -1,5 +1,5 @@
-"""Prompt-phase scoring where both visits of the keys share a launch: runs and clusters of runs that do not divide the prompt,
-one and two operands of window rows, rows of different lengths, the order in which CTAs take the items."""
+"""Prompt-phase scoring of some 2300 to 2600 tiles, a launch for each visit of the keys: runs that do not divide the prompt,
+one and two operands of window rows, rows of different lengths, the same result again."""
 import numpy as np
 import pytest
 import torch
@@ -11,8 +11,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("layers,q_heads,kv_heads,P,C,R,fusion", [
-    (32, 32, 8, 1090, 700, 32, "sum"),      # 2304 tiles, runs of seven tiles of nine
-    (1, 8, 2, 17500, 1000, 30, "max"),      # 137 runs of one tile: nine clusters, the last of nine
+    (32, 32, 8, 1090, 700, 32, "sum"),      # 2304 tiles, a run for every prompt
+    (1, 8, 2, 17500, 1000, 30, "max"),      # 137 tiles, 69 runs of two, the last of one
     (24, 8, 2, 6000, 900, 64, "max"),       # 256 rows: two groups per tile
     (24, 28, 4, 2900, 600, 30, "sum"),      # padded group, 240 rows
     (40, 8, 2, 3500, 800, 100, "sum"),      # two pieces, of 256 and 144 rows

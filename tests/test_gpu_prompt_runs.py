@@ -1,8 +1,9 @@
 """Prompt-phase scoring at the edges of its forms: a launch for each visit with few and with many runs per unit, runs of two to
 fourteen tiles, both visits in one launch with a last cluster of runs that is not full, nothing to select, three blocks of rows."""
 import pytest
+import torch
 
-from paper_2503_00979_b200 import synth
+from paper_2503_00979_b200 import binding, synth
 from tests.parity import run_parity, run_parity_ragged
 
 pytestmark = pytest.mark.gpu
@@ -31,3 +32,36 @@ def test_rows_that_end_in_different_clusters():
     w = synth.Workload("clusters", 4, 3, 8, 2, 128, "bf16", 0, 2, 900, 30, "max", 91)
     rep = run_parity_ragged(w, [40000, 16385, 20000], steps=2, kernel="tc")
     assert rep.units == 4 * 3 * 2
+
+
+def test_result_does_not_depend_on_the_order_of_items():
+    # 3328 tiles: both visits in one launch, items by ticket
+    g = torch.Generator(device="cuda:0")
+    g.manual_seed(5)
+    L, P, C, R = 26, 2000, 700, 32
+    k, v = (torch.randn((L, 1, 8, P, 128), generator=g, device="cuda:0").bfloat16() for _ in range(2))
+    q = torch.randn((L, 1, 32, R, 128), generator=g, device="cuda:0").bfloat16()
+    got = []
+    mk = binding.MorphKV(L, 1, 32, 8, 128, C, R, "sum", "bf16")
+    for _ in range(6):
+        mk.reset()
+        mk.prefill(k, v, q)
+        got.append([torch.cat([mk.view(l)[name].flatten() for l in range(L)]).clone() for name in ("pos", "ring_c")])
+    assert all(torch.equal(a, b) for r in got[1:] for a, b in zip(r, got[0]))
+    mk.close()
+
+
+@pytest.mark.parametrize("P,C", [(1030, 1), (1040, 1003), (4112, 700), (4113, 4000)])
+def test_tied_scores_of_many_units(P, C):
+    # more units than twice the SMs: the selection in smaller CTAs, up to 4096 candidates; every older token has the same score
+    L, R, dev = 38, 16, torch.device("cuda:0")
+    gen = torch.Generator(device=dev)
+    gen.manual_seed(P)
+    q = torch.randn((L, 1, 8, R, 128), generator=gen, device=dev).bfloat16()
+    k = torch.zeros((L, 1, 8, P, 128), dtype=torch.bfloat16, device=dev)
+    mk = binding.MorphKV(L, 1, 8, 8, 128, C, R, "sum", "bf16")
+    mk.prefill(k, k, q)
+    want = torch.cat([torch.arange(C, device=dev), torch.arange(P - R, P, device=dev)])
+    for l in (0, L // 2, L - 1):
+        assert torch.equal(mk.view(l)["pos"][0, :, :C + R].long(), want.expand(8, -1))
+    mk.close()
