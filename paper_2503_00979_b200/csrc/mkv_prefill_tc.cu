@@ -11,12 +11,13 @@
 //               every thread owns one key, turns its row of logits into weights exp2(s - c_row), sums them over the
 //               group and fuses them over the window; F[k] is written for the candidates (P floats per unit).
 //
-// One launch does both, so that the second visit of a key finds it in L2: its persistent CTAs take items, each a visit of one
-// kind to a run of a unit's key tiles, from one sequence in which the scores of a run follow its statistics `lag` runs later -
-// late enough for all of its unit's statistics to be there, early enough for the runs in between (some 60 MB, and a unit's own
-// keys) to stay in the 126 MB L2.  Items are handed out by a ticket, in order: an item waits only for items that running CTAs
-// hold, so no number of resident CTAs is needed.  The CTA that completes a unit's statistics merges them into the
-// normalisers and raises the unit's flag.
+// One launch does both where the keys are too many to stay in L2 by themselves (prompt_apart_tiles), so that the second visit of a key
+// finds it there: its persistent CTAs take items, each a visit of one kind to a run of a unit's key tiles, from one sequence in which the
+// scores of a run follow its statistics `lag` runs later - late enough for all of its unit's statistics to be there, early enough for the
+// runs in between (some 60 MB, and a unit's own keys) to stay in the 126 MB L2.  Items are handed out by a ticket, in order: an item waits
+// only for items that running CTAs hold, so no number of resident CTAs is needed.  The CTA that completes a unit's statistics merges them
+// into the normalisers and raises the unit's flag.  Otherwise each visit has a launch, whose items wait for nothing and are every
+// CTA's own, and the items of the second merge their unit's statistics.
 //
 // CTA layout: warp 0 takes the tickets and feeds queries and K tiles with TMA; warps 1 and 3 issue the MMAs into the TMEM
 // accumulator buffers; warp 2 waits for the units' flags and fetches their normalisers, ahead of the items that need them;
@@ -25,12 +26,15 @@
 // (two buffers), K tiles, normalisers and statistics pass through rings of their own, so that nothing drains between items.
 // Every wait is bounded; a wait that runs out raises an error word that the host reads after the call.
 //
-// What bounds it: the 1000 W of the card for long prompts (two MMAs, 2 x 4 bytes of TMEM and two exponentials per key and row, the
-// SM clock falls to 1.4 GHz), the MUFU's exponentials for the others (2048 cycles of a tile's two visits, 2600 taken).
-// Prompt phase in us, one pass of launches over the keys per visit -> now (both warm): 256 units x 6144 tokens, 128 rows, 317 -> 291;
-// 64 x 32768, 256 rows, 526 -> 491; 128 x 2600 (8 rows a layer) 555 -> 534; 256 x 131072 3854 -> 3820; 112 x 560 102 -> 84.  Taken
-// back: every fourth exponential as a polynomial on the FMA pipe (6144: 285 us cold, but 131072 3850 -> 3910: more power); keys
-// kept with evict_last, or without a policy at the second visit (no change, 131072 up to 15 % slower).
+// What bounds it: the MUFU's exponentials, two per key and row: 2048 cycles of a tile's two visits with 128 rows, of 3290 taken for 256
+// units x 6144 tokens (159 us at 1.70 GHz: MUFU 73 % busy, tensor pipe 31 %, 441 MB from HBM of which the keys are 403); prompt after
+// prompt also the 1000 W of the card (256 x 131072: 3236 us at 1965 MHz, 3717 at 1500 after a second of it).  A launch for each visit is bound by the
+// same and by the start of a launch that needs whole SMs: up to two tiles per unit take 3 to 8 us longer than with smaller CTAs, two to an SM.
+// Prompt phase in us, one pass of launches over the keys per visit -> now (L2 flushed): 256 units x 6144 tokens, 128 rows, 304 -> 288;
+// 64 x 32768, 256 rows, 528 -> 485; 128 x 12291, 800 rows in pieces, 1341 -> 1226; 256 x 131072 3259 -> 3254;
+// 112 x 560 91 -> 75.  Taken back: every fourth exponential as a polynomial on the FMA pipe (6144: 285 us cold, but 131072 3850 -> 3910:
+// more power); keys kept with evict_last, or without a policy at the second visit (no change, 131072 up to 15 % slower); a row's maximum
+// only where a chunk's sum shows that the reference is far below it (no faster, and the exponents of the weights that count rounded coarsely).
 #include <stdio.h>
 
 #include <algorithm>
