@@ -228,26 +228,48 @@ prefill_tc_kernel(const __grid_constant__ PfArgs a, const __grid_constant__ CUte
     int *table = reinterpret_cast<int *>(smem + L.table);                  // RunOrder::place
     const long long WL = a.wait_cycles;
 
-    // one barrier each: the launch's start is in the way of the first copies
-    if (tid < 38) {
-        int n = 1;                                              // the pairs and fours "full": one arrival, and the copies' bytes
-        if (tid >= 12 && tid < 16) n = 4 * kPfGroups / NB;      // tempty
-        else if (tid >= 20 && tid < 24) n = 3 + 4 + 4 * kPfGroups;     // dempty: the MMA warps, the normalisers' warp, four publishing and all consumer warps
-        else if (tid == 26 || tid == 27) n = 2;                 // qempty
-        else if (tid >= 30 && tid < 34) n = 4 * kPfGroups;      // nempty, sfull
-        else if (tid >= 34) n = 4;                              // sempty, pair
-        mbar_init(smem_u32(bars + (tid < 36 ? tid : tid + 3)), (uint32_t)n);
+    // a barrier per lane: the launch's start is in the way of the first copies (by thread index, in all warps' code, it cost the consumers
+    // three registers and spills)
+    if (warp == 0) {
+        for (int i = lane; i < 38; i += 32) {
+            const int n = i >= 34 ? 4                                   // sempty, pair
+                          : i >= 30 ? 4 * kPfGroups                     // nempty, sfull
+                          : i >= 28 ? 1                                 // nfull
+                          : i >= 26 ? 2                                 // qempty
+                          : i >= 24 ? 1                                 // qfull
+                          : i >= 20 ? 3 + 4 + 4 * kPfGroups             // dempty: the MMA warps, the normalisers' warp, four publishing and all consumer warps
+                          : i >= 16 ? 1                                 // dfull
+                          : i >= 12 ? 4 * kPfGroups / NB                // tempty
+                                    : 1;                                // tfull, kempty, kfull
+            mbar_init(smem_u32(bars) + 8 * (i < 36 ? i : i + 3), (uint32_t)n);
+        }
+        if (lane == 0) {
+            prefetch_tensormap(&tmK);
+            prefetch_tensormap(&tmQ);
+            *abort_flag = 0;
+        }
         fence_barrier_init();
-    }
-    if (tid == 64) {
-        prefetch_tensormap(&tmK);
-        prefetch_tensormap(&tmQ);
-        *abort_flag = 0;
     }
     if (warp == 1) tmem_alloc(smem_u32(tmem_slot), 512);
     // (the rows' lengths were there before the first launch of the chain)
     const int entries = a.order.entries;
-    for (int e = tid; e < entries; e += kPfThreads) table[e + 1] = a.order.entry(e);
+    if (entries > 0) {         // (by a warp that has time: ahead of the copying lane's code it slowed that down, 1 to 5 % of a prompt)
+        for (int e = tid; e < entries; e += kPfThreads) table[e + 1] = a.order.entry(e);
+        __syncthreads();
+        if (warp == 2) {
+            for (int e0 = 0, sum = 0; e0 < entries; e0 += 32) {
+                int v = e0 + lane < entries ? table[e0 + lane + 1] : 0;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int up = __shfl_up_sync(0xffffffffu, v, o);
+                    if (lane >= o) v += up;
+                }
+                if (e0 + lane < entries) table[e0 + lane + 1] = sum + v;
+                if (e0 + lane == 0) table[0] = 0;
+                sum += __shfl_sync(0xffffffffu, v, 31);
+            }
+        }
+    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -268,18 +290,6 @@ prefill_tc_kernel(const __grid_constant__ PfArgs a, const __grid_constant__ CUte
 
     if (warp == 0) {
         // ------------------------------------------------ tickets, queries, K tiles (one lane)
-        for (int e0 = 0, sum = 0; e0 < entries; e0 += 32) {
-            int v = e0 + lane < entries ? table[e0 + lane + 1] : 0;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int up = __shfl_up_sync(0xffffffffu, v, o);
-                if (lane >= o) v += up;
-            }
-            if (e0 + lane < entries) table[e0 + lane + 1] = sum + v;
-            if (e0 + lane == 0) table[0] = 0;
-            sum += __shfl_sync(0xffffffffu, v, 31);
-        }
-        __syncwarp();
         if (lane == 0) {
             // the keys stay in L2 between their two visits, and are not needed there afterwards
             const uint64_t pol_first = l2_policy_evict_normal(), pol_last = l2_policy_evict_first();
